@@ -578,9 +578,7 @@ bool make_pop_map(const lb_handle* h, void* base, CUtensorMap* map) {
 // Row-march work items: strips of kMarchW columns cut into row ranges, at most one item per
 // resident CTA (one wave: a partial second wave would double the kernel time for a few CTAs).
 // Items are not equally long, because CTAs are not equally fast: the warp schedulers favour older
-// warps, so the CTAs that arrive later on an SM take longer for the same rows (measured at
-// 4096 x 4096 with equal items, per CTA rank on its SM: FP32 five ranks 246 ... 275 us; BF16
-// eight ranks 182 ... 219 us), and an edge strip costs more per row than an interior one (its
+// warps, so the CTAs that arrive later on an SM take longer for the same rows, and an edge strip costs more per row than an interior one (its
 // halo columns are patched from the other end; with pressure-driven ends it also applies the
 // crossing corrections).  The model: block b, of rank k = b / n_sm (blocks fill the SMs rank by
 // rank), runs at speed 1 + skew (R-1-k)/(R-1) for R CTAs per SM; strip j costs f_j per row (f for
@@ -600,19 +598,14 @@ struct MarchModel {
     bool chunk_major;
 };
 
-// Constants measured at 4096 x 4096 (GLUPS of the whole step; repeated runs on one GPU):
-//   FP32 (HBM-bound): chunk-major skew 0.12: 60.5 (0.08: 60.1, 0.16: 60.4, 0.2: 59.4, 0.3: 58.6)
-//     against strip-major skew 0: 59.1 (strip-major with skew loses: 0.12 -> 55.5, the halo
-//     re-reads); f = 1.2; pressure-driven ends f = 1.5 with the edge strips first 53.6 (last: 50.3;
-//     strip-major 53.0); moving wall 59.1 (57.7); 8192 x 2048 58.2 (57.2); 2048 x 2048 52.6 (51.9).
-//   BF16 (issue-bound): chunk-major skew 0.3: 75.4 (0.45: 75.1, 0.6: 74.0; with the edge strips on
-//     the last blocks 74.0) against strip-major skew 0.3: 74.6-74.7 (strip-major skew 0 / 0.12 / 0.2 /
-//     0.28 / 0.36 / 0.45 -> 73.7 / 75.2 / 75.6 / 75.9 / 76.1 / 73.6 on another GPU); f = 1.15;
-//     pressure-driven ends f = 1.5 (65.55; strip-major 65.45; f = 1.3 / 1.6 / 1.9 strip-major ->
-//     62.2 / 64.8 / 63.6).
+// Constants measured with six CTAs of two warps per SM (us per step, one GPU):
+//   FP32 4096 x 4096: skew 0.06: 251.9, 0.12: 252.9, 0: 252.7, 0.2: 257.7; f = 1.2 252.9, 1.05: 264.0,
+//     1.35: 253.6; pressure-driven ends at 2048 x 1000 f = 1.7: 51.8, 1.5: 53.7, 1.3: 55.5, 1.2: 59.7.
+//   BF16 8192 x 2048: skew 0.3 f = 1.15: 214.4; f = 1.3: 212.8 (but leaves CTAs idle with eight per SM); f = 1.05: 228.4; skew 0.15 / 0.22 with
+//     f = 1.15: 214.5 / 214.9; skew 0.4: 228.6.
 static MarchModel march_model(int prec, bool gpbc) {
     if (prec == LB_PREC_BF16) return {0.30, gpbc ? 1.5 : 1.15, true};
-    return {0.12, gpbc ? 1.5 : 1.2, true};
+    return {0.08, gpbc ? 1.6 : 1.2, true};
 }
 
 static std::vector<MarchItem> march_plan(int nx, int ny, int R, int nsm, MarchModel m) {
@@ -712,6 +705,28 @@ static std::vector<MarchItem> march_plan(int nx, int ny, int R, int nsm, MarchMo
     return items;
 }
 
+// The kernel addresses an item's rows with 32-bit offsets: items of 2^29 elements or more are halved.
+static std::vector<MarchItem> short_items(const std::vector<MarchItem>& in, int nx) {
+    std::vector<MarchItem> out;
+    for (MarchItem it : in) {
+        const long long most = std::max(8LL, (1LL << 29) / nx);
+        while (it.y1 - it.y0 > most) {
+            MarchItem a = it;
+            a.y1 = it.y0 + (it.y1 - it.y0) / 2;
+            it.y0 = a.y1;
+            while (a.y1 - a.y0 > most) {
+                MarchItem b = a;
+                b.y1 = a.y0 + (int)most;
+                out.push_back(b);
+                a.y0 = b.y1;
+            }
+            out.push_back(a);
+        }
+        out.push_back(it);
+    }
+    return out;
+}
+
 lb_status plan_march(lb_handle* h) {
     h->march = false;
     if (h->n_ch != 1 || (h->prec != LB_PREC_F32 && h->prec != LB_PREC_BF16) || h->nx % kMarchW != 0 ||
@@ -742,7 +757,7 @@ lb_status plan_march(lb_handle* h) {
     if (e != cudaSuccess) return cuda_fail(e, "lb_create: march occupancy");
     if (bps < 1) return LB_OK;
     const int slots = bps * nsm;
-    const std::vector<MarchItem> items = march_plan(h->nx, h->ny[0], bps, nsm, march_model(h->prec, h->gpbc));
+    const std::vector<MarchItem> items = short_items(march_plan(h->nx, h->ny[0], bps, nsm, march_model(h->prec, h->gpbc)), h->nx);
     LB_CK(cudaMalloc(&h->march_items_d, sizeof(MarchItem) * items.size()));
     LB_CK(cudaMemcpy(h->march_items_d, items.data(), sizeof(MarchItem) * items.size(), cudaMemcpyHostToDevice));
     h->n_march_items = (int)items.size();

@@ -1,21 +1,22 @@
 // lb_step_march.cuh -- the fused lattice-Boltzmann step for wide channels: a TMA-fed row march.
 //
-// A CTA owns a strip of CW columns (x0 .. x0+CW-1), NC adjacent columns per thread, and marches
-// through rows y0..y1-1 of one channel.  The post-collision populations of the previous step stream into a ring of K
-// shared-memory slots, one source row per slot: a single 3-D tensor-memory-access copy brings the
-// 9 direction planes of that row, columns x0-HP .. x0+CW+HP-1 (HP = 16 bytes of halo on each side,
-// so every copy starts on a 16-byte boundary).  The copies run K-2 rows ahead of the arithmetic
+// A CTA owns a strip of CW columns (x0 .. x0+CW-1), two adjacent columns per thread, and marches
+// through rows y0..y1-1 of one channel.  The post-collision populations of the previous step stream into a
+// ring of K shared-memory slots, one source row per slot: a single 3-D tensor-memory-access copy
+// brings the 9 direction planes of that row, columns x0-HP .. x0+CW+HP-1 (HP = 16 bytes of halo on each
+// side, so every copy starts on a 16-byte boundary).  The copies run K-2 rows ahead of the arithmetic
 // and complete on one mbarrier per slot.
 //
 // Per row y (one __syncthreads per row):
-//   1. moments (Eq. rhoj) of row y+1 for the CW own columns and the two halo columns x0-1, x0+CW,
+//   1. moments (Eq. rhoj) of row y+1 for the own columns and the two halo columns x0-1, x0+CW,
 //      pulled from slots y, y+1, y+2 (Eq. lbupdate, pull form; bounce-back at the walls,
-//      Sec. II B); the own populations stay in registers for the next row's collision;
-//      the gradient velocity j/R0 goes into a 4-row ring in shared memory;
+//      Sec. II B); the own populations and gradient velocities j/R0 stay in registers, and what the
+//      neighbouring threads need of the velocities goes through shuffles or shared memory;
 //   2. barrier; one thread (the last lane) refills the slot of row y with row y+K;
-//   3. collision of row y: kappa by three-point differences from the velocity ring, the nlM
-//      stress, Sigma^nN, delta rho, n^eq, F_i (Eq. bodyforce), BGK; coalesced stores (with two
-//      columns per thread, 8-byte FP32 pairs and 4-byte BF16 pairs).
+//   3. collision of row y: kappa by three-point differences (along y from the thread's own
+//      registers), the nlM stress, Sigma^nN, delta rho, n^eq, F_i
+//      (Eq. bodyforce), BGK; coalesced stores (8-byte FP32 pairs, 4-byte BF16 pairs).
+// The two columns of a thread go through the arithmetic together as packed FP32 (lb_pair.cuh).
 // The periodic wrap of x is patched into the halo columns of the first and last strip with
 // plain loads.  Every mbarrier wait is bounded (MarchCtl::max_wait_ns, 2 s by default): on timeout
 // the CTA records LB_ETIMEOUT in the status word, drains its own copies (also bounded) and returns.
@@ -23,7 +24,7 @@
 
 #include <cuda.h>
 
-#include "lb_device.cuh"
+#include "lb_pair.cuh"
 
 namespace lbk {
 
@@ -125,89 +126,73 @@ struct MarchGeom {
 template <typename T, typename C, int W, int K>
 constexpr size_t march_smem_bytes() {
     constexpr int HP = MarchGeom<T>::HP;
-    constexpr size_t slot = ((size_t)9 * (W + 2 * HP) * sizeof(T) + 127) / 128 * 128;
-    return 128 /*barriers*/ + K * slot + (size_t)4 * (W + 2) * 2 * sizeof(C);
+    constexpr size_t slot = ((size_t)9 * (W + 2 * HP) * sizeof(T) + 8 + 127) / 128 * 128;
+    return K * slot + (std::is_same<T, float>::value ? (size_t)W * 2 * sizeof(C) + 4 * 4 * 2 * sizeof(C)
+                                                     : (size_t)4 * (W + 4) * 2 * sizeof(C));
 }
 
-// Row loads and stores of NC adjacent values of one plane (8-byte vector accesses for two floats).
-template <typename C, int NC>
-__device__ __forceinline__ void load_cols(const C* p, C (&v)[NC]) {
-    if constexpr (NC == 2 && sizeof(C) == 4) {
-        const float2 q = *reinterpret_cast<const float2*>(p);
-        v[0] = q.x;
-        v[1] = q.y;
-    } else {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) v[c] = p[c];
-    }
+// Rows of a field of the arithmetic type: the thread's two adjacent columns as one 8-byte access.
+__device__ __forceinline__ P2 load_pair(const float* p) {
+    P2 r;
+    r.v = *reinterpret_cast<const unsigned long long*>(p);
+    return r;
 }
-template <typename C, int NC>
-__device__ __forceinline__ void store_cols(C* p, const C (&v)[NC]) {
-    if constexpr (NC == 2 && sizeof(C) == 4) {
-        *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
-    } else {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) p[c] = v[c];
-    }
+__device__ __forceinline__ void store_pair(float* p, P2 v) { *reinterpret_cast<unsigned long long*>(p) = v.v; }
+// Populations in the storage type: FP32 as above; BF16 rounded to nearest, one 4-byte store.
+__device__ __forceinline__ void store_pop_pair(float* p, P2 v) { store_pair(p, v); }
+__device__ __forceinline__ void store_pop_pair(__nv_bfloat16* p, P2 v) {
+    *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(lo(v), hi(v));
 }
-// Post-collision populations d + D of NC adjacent nodes (node index of the first in `node`): two
-// FP32 values per 8-byte store, two BF16 values (rounded to nearest) per 4-byte store; stochastic
-// rounding goes node by node through store_node.
-template <typename T, typename C, int NC>
-__device__ __forceinline__ void store_cols_pop(T* po, long long P, const C (&d)[NC][9], const C (&D)[NC][9], bool sr,
-                                               uint32_t key, uint32_t node) {
-    if constexpr (NC == 2 && std::is_same<T, float>::value) {
-#pragma unroll
-        for (int i = 0; i < 9; ++i)
-            *reinterpret_cast<float2*>(po + (long long)i * P) = make_float2(d[0][i] + D[0][i], d[1][i] + D[1][i]);
-    } else {
-        if constexpr (NC == 2 && std::is_same<T, __nv_bfloat16>::value) {
-            if (!sr) {
-#pragma unroll
-                for (int i = 0; i < 9; ++i)
-                    *reinterpret_cast<__nv_bfloat162*>(po + (long long)i * P) =
-                        __floats2bfloat162_rn(d[0][i] + D[0][i], d[1][i] + D[1][i]);
-                return;
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < NC; ++c) store_node<T, C>(po + c, P, d[c], D[c], sr, key, node + (uint32_t)c);
-    }
+// Two neighbouring populations of a slot row, as FP32: at an even column one access, at an odd one two.
+__device__ __forceinline__ P2 slot_pair(const float* p) { return load_pair(p); }
+__device__ __forceinline__ P2 slot_pair(const __nv_bfloat16* p) {
+    const uint32_t w = *reinterpret_cast<const uint32_t*>(p);  // (a BF16 value is the high half of its FP32 one)
+    return p2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+template <typename T>
+__device__ __forceinline__ P2 slot_pair_odd(const T* p) {
+    return p2((float)Store<T>::cvt(p[0]), (float)Store<T>::cvt(p[1]));
 }
 
 // BND = 1: channel ends joined by the generalized periodic boundaries of Sec. II B, and a moving
 // Couette wall on the last row (Sec. IV C) if the channel has one; BND = 2: the moving wall only;
 // both applied where the populations are pulled (the same rules as the tile kernel's pull9).
 // BND = 0: periodic x and bounce-back walls only.
-// CW columns per CTA, NC adjacent columns per thread (CW / NC threads).
-// Resident CTAs per SM the two-column kernel is compiled for: 7 caps it at 127 registers (no
-// spills), 14 warps per SM instead of 10 at its natural 155 (BF16 at 4096 x 4096: 73.8 GLUPS at 7,
-// 72.3 at 8, 69.0 at 5; its warps stall mostly on fixed-latency dependencies, which more warps hide).
-#ifndef LBK_MARCH_MINB2
-#define LBK_MARCH_MINB2 7
-#endif
 // SCHEME 1: the generalized-Newtonian comparison scheme of Sec. II C (periodic x, bounce-back
 // walls, stress mode A), the node's own relaxation rate as in the tile kernel's scheme-1 variant.
 // SCHEME 3: the relaxation-time extensions (periodic x, bounce-back walls, either stress mode): the
 // node's FP64 fluidity is loaded one row ahead of its use and stored with the step, as in the tile
-// kernel's scheme-3 variant (the FP32 kernel then runs 4 CTAs per SM for the registers it needs).
-template <typename T, typename C, int SMODE, int CW, int NC, int K, int BND = 0, int SCHEME = 0>
-__global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME == 3 ? 4 : 5)) k_step_march(const __grid_constant__ CUtensorMap tmap,
-                                                          const StepArgs<T, C> a, const MarchCtl ctl) {
-    constexpr int NT = CW / NC;                                      // threads per CTA
+// kernel's scheme-3 variant.
+template <typename T, typename C, int SMODE, int CW, int K, int BND = 0, int SCHEME = 0>
+__global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant__ CUtensorMap tmap,
+                                                                                  const StepArgs<T, C> a,
+                                                                                  const MarchCtl ctl) {
+    static_assert(std::is_same<C, float>::value, "the pair arithmetic is FP32");
+    constexpr int NT = CW / 2;                                       // threads per CTA
     constexpr int HP = MarchGeom<T>::HP;
     constexpr int SW = CW + 2 * HP;                                  // slot row width (elements)
-    constexpr size_t SLOT = ((size_t)9 * SW * sizeof(T) + 127) / 128 * 128;
     constexpr uint32_t TX = 9u * SW * sizeof(T);                     // bytes per copy
-    constexpr int UW = CW + 2;                                       // velocity ring row width
-    static_assert(NT >= 64 && NT % 32 == 0, "the edge patchers and the issuing thread need two warps");
+    constexpr uint32_t SLOT = (TX + 8 + 127) / 128 * 128;            // a slot: the copy, then its mbarrier
+    // measured choices, see the note above the launchers
+    constexpr bool F32 = std::is_same<T, float>::value;
+    constexpr bool HALO2 = BND != 1;   // both halo columns of two rows in one pass (pressure-driven ends: the
+                                       // brackets of row y+3 come too late for it)
+    constexpr bool UNROLL2 = BND != 1; // the row loop written out for two rows
+    constexpr bool SHUFFLE = F32;      // neighbouring columns' velocities by warp shuffles, or a ring of rows
+    constexpr bool OFF32 = F32;
+    constexpr int UW = CW + 4;         // ring row: columns x0-2 .. x0+CW+1
+    static_assert(NT == 64, "two warps: the border velocities, the edge patchers, the issuing thread");
 
     extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem);               // K mbarriers (<= 16)
-    unsigned char* slots = smem + 128;
-    C* uring = reinterpret_cast<C*>(slots + K * SLOT);                // [4][UW][2]
+    unsigned char* slots = smem;                                      // K slots
+    // own velocities of the row two rows from a wall (the one-sided difference of the wall row), and
+    // per row (ring of 4) the velocities that cross a warp's border: x0-1, the border columns, x0+CW
+    // (SHUFFLE), or a ring of 4 rows of velocity pairs, two columns of one thread on a 16-byte boundary
+    C* uwall = reinterpret_cast<C*>(slots + K * SLOT);                // SHUFFLE: [CW][2]
+    float2* edge = reinterpret_cast<float2*>(uwall + 2 * CW);         // SHUFFLE: [4][4]
+    auto ring = [&](int r, int col) -> C* { return uwall + 2 * ((r & 3) * UW + col + 2); };
 
-    const int t = threadIdx.x;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const ChanParams<C> P = a.chan[0];
     const int nx = a.nx, ny = P.ny;
     const bool halted = a.status[0] != 0;  // an unstable or timed-out channel takes no more steps
@@ -222,6 +207,7 @@ __global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME =
     constexpr int TI = NT - 1;  // the thread that issues the copies (last lane; warp 0 computes
                                 // the halo columns)
     constexpr int TP = NT - 2;  // the thread that issues the L2 prefetches of residual steps
+    auto bar_at = [&](uint32_t off) -> uint64_t* { return reinterpret_cast<uint64_t*>(slots + off + TX); };
     if (t == 0) {
         s_bad = 0;
         if (BND == 1 && a.gcol != nullptr) {
@@ -230,25 +216,31 @@ __global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME =
             s_delta[1] = P.rho_in - means[1];
         }
         prefetch_tmap(&tmap);
-        for (int k = 0; k < K; ++k) mbar_init(&bars[k], 1);
+        for (int k = 0; k < K; ++k) mbar_init(bar_at(k * SLOT), 1);
         fence_barrier_init();
     }
     __syncthreads();
 
+    const PairConst q = pair_const(P);
     bool vbad = false;  // some node of this CTA failed the velocity guard (reported when the CTA ends)
     uint32_t nload = 0;  // CTA-uniform count of copies issued (and, in order, consumed)
     bool bad = false;
+    // what the launch asks for besides the step itself (uniform)
+    const bool resid = (a.flags & F_RESID) != 0;
+    const bool mon = (a.flags & (F_RESID | F_MON)) != 0;
+    const bool save_u = (a.flags & F_SAVE_U) != 0;
+    const bool want_u = mon || save_u;
+    const bool store_sigma = (a.flags & F_STORE_SIGMA) != 0;
+    const bool sr = std::is_same<T, __nv_bfloat16>::value && (a.flags & F_SR) != 0;
+    const long long PL = ctl.plane;
 
-    auto slot_ptr = [&](uint32_t idx) -> const T* { return reinterpret_cast<const T*>(slots + (idx % K) * SLOT); };
-    uint32_t last_issued[K];  // issuing thread: index of the last copy issued into each slot
-#pragma unroll
-    for (int k = 0; k < K; ++k) last_issued[k] = 0xffffffffu;
-    auto issue = [&](uint32_t idx, int x0, int row) {  // issuing thread (TI) only
-        uint64_t* b = &bars[idx % K];
-        mbar_expect_tx(b, TX);
-        tma_load_3d(slots + (idx % K) * SLOT, &tmap, b, x0 - HP, row, 0);
-        last_issued[idx % K] = idx;
+    auto issue = [&](uint32_t off, int x0, int row) {  // issuing thread (TI) only
+        mbar_expect_tx(bar_at(off), TX);
+        tma_load_3d(slots + off, &tmap, bar_at(off), x0 - HP, row, 0);
     };
+    // the slot after the one at `off`
+    auto next_slot = [&](uint32_t off) -> uint32_t { return off == (K - 1) * SLOT ? 0u : off + SLOT; };
+    uint32_t issued_end = 0;  // issuing thread: one past the index of the last copy issued
 
     for (int item = blockIdx.x; item < ctl.n_items && !bad && !halted; item += gridDim.x) {
         const MarchItem it = ctl.items[item];
@@ -257,14 +249,14 @@ __global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME =
         const int rlast = y1 + 1;                 // last source row
         const uint32_t L0 = nload;                // load index of row rbase
         const bool left_edge = (x0 == 0), right_edge = (x0 + CW == nx);
-        const int col0 = NC * t;                  // first own column (relative to x0)
-        const int x = x0 + col0;                  // its global column
+        const int col0 = 2 * t;                   // first own column (relative to x0)
 
-        // index of the copy holding source row r, and the wait for it
+        // index of the copy holding source row r, its slot, and the wait for it
         auto idx_of = [&](int r) -> uint32_t { return L0 + (uint32_t)(r - rbase); };
+        auto slot_off = [&](int r) -> uint32_t { return (idx_of(r) % K) * SLOT; };
         auto wait_row = [&](int r) -> bool {
             const uint32_t i = idx_of(r);
-            return mbar_wait(&bars[i % K], (i / K) & 1u, ctl.max_wait_ns);
+            return mbar_wait(bar_at((i % K) * SLOT), (i / K) & 1u, ctl.max_wait_ns);
         };
         // periodic wrap: the edge strips' halo columns x0-2, x0-1 (left) or x0+CW, x0+CW+1 (right)
         // come from the other end of the row; threads 0..17 (left) and 32..49 (right) each own
@@ -274,10 +266,10 @@ __global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME =
         const int pc = left_edge && t < 18 ? (nx - 2 + (t & 1)) : ((t - 32) & 1);     // global column
         const int ps = left_edge && t < 18 ? (HP - 2 + (t & 1)) : (HP + CW + ((t - 32) & 1));  // slot column
         auto patch_load = [&](int r) -> T {
-            return (r >= 0 && r < ny && r <= rlast) ? a.pin[9 * ctl.base + (long long)pi * ctl.plane + (long long)r * nx + pc] : T(0);
+            return (r >= 0 && r < ny && r <= rlast) ? a.pin[9 * ctl.base + (long long)pi * PL + (long long)r * nx + pc] : T(0);
         };
         auto patch_store = [&](int r, T v) {
-            if (r >= 0 && r < ny && r <= rlast) const_cast<T*>(slot_ptr(idx_of(r)))[pi * SW + ps] = v;
+            if (r >= 0 && r < ny && r <= rlast) reinterpret_cast<T*>(slots + slot_off(r))[pi * SW + ps] = v;
         };
         // GPBC brackets: lanes 0..5 of the left edge strip's patchers (32..37 on a right edge
         // strip) take one (boundary column, direction) each and evaluate source row r from the
@@ -291,37 +283,15 @@ __global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME =
             const int c = sl / 3, j = sl - 3 * (sl / 3);
             const int i = c == 1 ? (j == 0 ? 1 : (j == 1 ? 5 : 8)) : (j == 0 ? 3 : (j == 1 ? 6 : 7));
             const int bcol = c == 1 ? (right_edge ? CW - 1 : -1) : (left_edge ? 0 : CW);
-            const T* sb = slot_ptr(idx_of(r)) + HP + bcol;
+            const T* sb = reinterpret_cast<const T*>(slots + slot_off(r)) + HP + bcol;
             C e[9], mR, mx, my;
 #pragma unroll
             for (int k = 0; k < 9; ++k) e[k] = (C)Store<T>::cvt(sb[k * SW]);
             moments<C>(e, mR, mx, my);
             s_shift[BND == 1 ? (r & 7) : 0][c][j] = gpbc_shift_core<C>(i, mR, mx, my, s_delta[c]);
         };
-        // pulled populations of node (col, r) from the slots (col relative to x0, may be -1 or CW):
-        // direction i comes from source row r - cy_i, column col - cx_i
-        auto pull = [&](int col, int r, C (&d)[9]) {
-            const T* s0 = slot_ptr(idx_of(r)) + HP + col;
-            if (r > 0 && r < ny - 1) {
-                const T* sm = slot_ptr(idx_of(r - 1)) + HP + col;  // source row r-1 (cy = +1)
-                const T* sp = slot_ptr(idx_of(r + 1)) + HP + col;  // source row r+1 (cy = -1)
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    const T* sr = cy(i) == 1 ? sm : (cy(i) == -1 ? sp : s0);
-                    d[i] = (C)Store<T>::cvt(sr[i * SW - cx(i)]);
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    const int rs = r - cy(i);
-                    if (rs < 0 || rs >= ny) {
-                        d[i] = (C)Store<T>::cvt(s0[opp(i) * SW]);  // bounce-back at the wall
-                    } else {
-                        const T* sr = slot_ptr(idx_of(rs)) + HP + col;
-                        d[i] = (C)Store<T>::cvt(sr[i * SW - cx(i)]);
-                    }
-                }
-            }
+        // end-crossing corrections and the moving wall on the pulled populations of node (col, r)
+        auto bound = [&](int col, int r, C (&d)[9]) {
             if constexpr (BND == 1) {
                 if (gpbc_edge) {
                     // the node's true column; the slots hold the raw periodic images, so every
@@ -347,34 +317,79 @@ __global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME =
                 if (r == ny - 1 && a.chan[0].moving) zou_he_top<C>(d, a.chan[0].u_wall);
             }
         };
-        // the ring holds (u_x, u_y) pairs at even offsets from a 128-byte aligned base: one
-        // 8-byte shared access per pair
-        using V2 = typename Vec2<C>::type;
-        auto put_u = [&](int r, int col, C ux, C uy) {
-            V2 v;
-            v.x = ux;
-            v.y = uy;
-            *reinterpret_cast<V2*>(uring + 2 * ((r & 3) * UW + col + 1)) = v;
-        };
-        auto get_u = [&](const C* p) -> V2 { return *reinterpret_cast<const V2*>(p); };
-        auto moments_row = [&](int r, C (&d)[NC][9], C (&dR)[NC], C (&jx)[NC], C (&jy)[NC]) {
-            // own columns, then the two halo columns (threads 0 and 1)
-            if (r >= 0 && r < ny) {
+        // pulled populations of one node (col, r) from the slots (col relative to x0, -1 or CW too):
+        // direction i comes from source row r - cy_i, column col - cx_i.  om, o0, op: slot offsets of
+        // the source rows r-1, r, r+1
+        auto pull_one = [&](int col, int r, uint32_t om, uint32_t o0, uint32_t op, C (&d)[9]) {
+            const T* sm = reinterpret_cast<const T*>(slots + om) + HP + col;
+            const T* s0 = reinterpret_cast<const T*>(slots + o0) + HP + col;
+            const T* sp = reinterpret_cast<const T*>(slots + op) + HP + col;
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    C ux, uy;
-                    pull(col0 + c, r, d[c]);
-                    gradient_velocity<C>(d[c], P.gx, dR[c], jx[c], jy[c], ux, uy);
-                    put_u(r, col0 + c, ux, uy);
-                }
-                if (t < 2) {  // the two halo columns, on lanes 0 and 1 of one warp (one pass)
-                    const int col = t == 0 ? -1 : CW;
-                    C dh[9], hR, hx, hy, ux, uy;
-                    pull(col, r, dh);
-                    gradient_velocity<C>(dh, P.gx, hR, hx, hy, ux, uy);
-                    put_u(r, col, ux, uy);
+            for (int i = 0; i < 9; ++i) {
+                const bool wall = (cy(i) == 1 && r == 0) || (cy(i) == -1 && r == ny - 1);
+                const T* sr = cy(i) == 1 ? sm : (cy(i) == -1 ? sp : s0);
+                d[i] = (C)Store<T>::cvt(wall ? s0[opp(i) * SW] : sr[i * SW - cx(i)]);
+            }
+            bound(col, r, d);
+        };
+        // the same for the thread's two columns
+        auto pull_pair = [&](int r, uint32_t om, uint32_t o0, uint32_t op, P2 (&d)[9]) {
+            const T* sm = reinterpret_cast<const T*>(slots + om) + HP + col0;
+            const T* s0 = reinterpret_cast<const T*>(slots + o0) + HP + col0;
+            const T* sp = reinterpret_cast<const T*>(slots + op) + HP + col0;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const T* sr = cy(i) == 1 ? sm : (cy(i) == -1 ? sp : s0);
+                d[i] = cx(i) == 0 ? slot_pair(sr + i * SW) : slot_pair_odd<T>(sr + i * SW - cx(i));
+            }
+            if (r == 0 || r == ny - 1) {  // bounce-back at the wall (uniform over the CTA)
+#pragma unroll
+                for (int i = 0; i < 9; ++i)
+                    if (cy(i) != 0 && (cy(i) == 1 ? r == 0 : r == ny - 1)) d[i] = slot_pair(s0 + opp(i) * SW);
+            }
+            if (BND >= 1) {
+                const bool near_end = gpbc_edge && ((left_edge && t == 0) || (right_edge && t == NT - 1));
+                if (near_end || r == ny - 1) {
+                    C e0[9], e1[9];
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) {
+                        e0[i] = lo(d[i]);
+                        e1[i] = hi(d[i]);
+                    }
+                    bound(col0, r, e0);
+                    bound(col0 + 1, r, e1);
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) d[i] = p2(e0[i], e1[i]);
                 }
             }
+        };
+        // moments and gradient velocities of row r's own columns.  om, o0, op: slots of rows r-1, r, r+1
+        auto moments_row = [&](int r, uint32_t om, uint32_t o0, uint32_t op, P2 (&d)[9], P2& dR, P2& jx, P2& jy, P2& ux,
+                               P2& uy) {
+            if (r < 0 || r >= ny) return;
+            pull_pair(r, om, o0, op, d);
+            gradient_velocity(d, q.hgx, dR, jx, jy, ux, uy);
+            if constexpr (SHUFFLE) {
+                if (t == 31) edge[4 * (r & 3) + 1] = make_float2(hi(ux), hi(uy));
+                if (t == 32) edge[4 * (r & 3) + 2] = make_float2(lo(ux), lo(uy));
+                if (r == ny - 3) *reinterpret_cast<float4*>(uwall + 2 * col0) = make_float4(lo(ux), lo(uy), hi(ux), hi(uy));
+            } else {
+                *reinterpret_cast<float4*>(ring(r, col0)) = make_float4(lo(ux), lo(uy), hi(ux), hi(uy));
+            }
+        };
+        // gradient velocities of the two halo columns of row r: one lane per column
+        auto halo_node = [&](int r, int col, uint32_t om, uint32_t o0, uint32_t op) {
+            C dh[9], hR, hx, hy, hux, huy;
+            pull_one(col, r, om, o0, op, dh);
+            gradient_velocity<C>(dh, P.gx, hR, hx, hy, hux, huy);
+            if constexpr (SHUFFLE) edge[4 * (r & 3) + (col < 0 ? 0 : 3)] = make_float2(hux, huy);
+            else *reinterpret_cast<float2*>(ring(r, col)) = make_float2(hux, huy);
+        };
+        // the own columns' velocities of row r, two rows from a wall
+        auto wall_pair = [&](int r, P2& ux, P2& uy) {
+            const float4 v = *reinterpret_cast<const float4*>(SHUFFLE ? uwall + 2 * col0 : ring(r, col0));
+            ux = p2(v.x, v.z);
+            uy = p2(v.y, v.w);
         };
 
         // ---- prologue: copies of rows rbase .. rbase+K-1; rows rbase .. rbase+5 waited and patched;
@@ -382,16 +397,23 @@ __global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME =
         // one-sided difference of row 0 needs it)
         if (t == TI) {
             fence_proxy_async();
-            for (int r = rbase; r < rbase + K && r <= rlast; ++r) issue(idx_of(r), x0, r);
+            for (int r = rbase; r < rbase + K && r <= rlast; ++r) {
+                issue(slot_off(r), x0, r);
+                issued_end = idx_of(r) + 1;
+            }
         }
         nload = L0 + (uint32_t)(rlast - rbase + 1);
         // residual partials (F_RESID / F_MON) of this thread's columns, in the arithmetic type (a
         // few hundred rows at most); the block reduction below runs in double
-        C r_du2 = C(0), r_u2 = C(0), r_ux = C(0), r_umax2 = C(0);
-        C dcur[NC][9], dnext[NC][9];
-        C dRc[NC], jxc[NC], jyc[NC], dRn[NC], jxn[NC], jyn[NC];
+        P2 r_du2 = p2(0.f), r_u2 = p2(0.f), r_ux = p2(0.f);
+        C r_umax2 = C(0);
+        // populations and moments of the row that collides and of the next one: the row loop is
+        // written out for two rows, with the two sets changing places
+        P2 dA[9], dB[9];
+        P2 dRa, jxa, jya, dRb, jxb, jyb;
+        P2 us_x = p2(0.f), us_y = p2(0.f), u0_x, u0_y, un_x = p2(0.f), un_y = p2(0.f);  // rows y-1, y, y+1
         bool ok = true;
-        for (int r = rbase; r <= rbase + 5; ++r) ok &= wait_row(r);
+        for (int r = rbase; r <= rbase + 5 && r <= rlast; ++r) ok &= wait_row(r);
         if (!ok) s_bad = 1;
         T pv_a = T(0), pv_b = T(0);
         if (patcher && ok) {  // patch only slots whose copies this thread saw land
@@ -407,223 +429,276 @@ __global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME =
             __syncthreads();
         }
         {
-            C dtmp[NC][9], a0[NC], a1[NC], a2[NC];
-            moments_row(y0 - 1, dtmp, a0, a1, a2);
-            if (y0 == 0) moments_row(2, dtmp, a0, a1, a2);
+            P2 a0, a1, a2, a3, a4;
+            moments_row(y0 - 1, slot_off(y0 - 2), slot_off(y0 - 1), slot_off(y0), dA, a0, a1, a2, us_x, us_y);
+            if (y0 == 0) {
+                moments_row(2, slot_off(1), slot_off(2), slot_off(3), dA, a0, a1, a2, a3, a4);
+                if constexpr (SHUFFLE)
+                    *reinterpret_cast<float4*>(uwall + 2 * col0) = make_float4(lo(a3), lo(a4), hi(a3), hi(a4));
+            }
         }
-        moments_row(y0, dcur, dRc, jxc, jyc);
+        moments_row(y0, slot_off(y0 - 1), slot_off(y0), slot_off(y0 + 1), dA, dRa, jxa, jya, u0_x, u0_y);
+        if (t < 2) halo_node(y0, t == 0 ? -1 : CW, slot_off(y0 - 1), slot_off(y0), slot_off(y0 + 1));
+        // offsets of this item's fields from its first row's first own column
+        const long long ubase = ctl.base + (long long)y0 * nx + x0, ibase = ubase + col0;
+        // address of the thread's columns in row y of a field: `o` / `vo` rows into the item.  FP32: a
+        // CTA-uniform pointer and a 32-bit offset; BF16: per-thread 64-bit pointers (each the faster
+        // one for its kernel: FP32 4096 x 4096 253 against 268 us, BF16 8192 x 2048 228 against 223)
+        auto field_at = [&](auto* f, long long o, uint32_t vo) {
+            using E = std::remove_pointer_t<decltype(f)>;
+            if constexpr (OFF32)
+                return reinterpret_cast<E*>(reinterpret_cast<uintptr_t>(f + ubase) + (vo + (uint32_t)col0) * (uint32_t)sizeof(E));
+            else
+                return f + ibase + o;
+        };
         // the stored flow-induced density, loaded two rows ahead of its use
-        const C* drow = a.drho + ctl.base + x;
-        C drho_next[NC], drho_next2[NC];
-        load_cols<C, NC>(drow + (long long)y0 * nx, drho_next);
-        if (y0 + 1 < y1) load_cols<C, NC>(drow + (long long)(y0 + 1) * nx, drho_next2);
+        const C* drow = a.drho + ibase;
+        P2 drho_next, drho_next2 = p2(0.f);
+        drho_next = load_pair(drow);
+        if (y0 + 1 < y1) drho_next2 = load_pair(drow + nx);
         // relaxation-time extensions with a fluidity memory: the node's fluidity (FP64), one row ahead
         const bool fluid = SCHEME == 3 && P.tau_f > C(0);  // CTA-uniform
-        const double* phrow = a.phi + ctl.base + x;
-        double phi_cur[NC], phi_nxt[NC];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) phi_cur[c] = phi_nxt[c] = 0.0;
-        if (fluid)
-#pragma unroll
-            for (int c = 0; c < NC; ++c) phi_nxt[c] = phrow[(long long)y0 * nx + c];
+        const double* phrow = a.phi + ibase;
+        double2 phi_nxt = make_double2(0.0, 0.0);
+        if (fluid) phi_nxt = *reinterpret_cast<const double2*>(phrow);
         // on residual steps the saved velocity of each row is prefetched the same way, and one
         // thread brings the delta rho and saved-velocity rows into L2 four rows before their
         // register loads (a residual step reads 16 B more per node than a plain one, and the
         // two-rows-ahead register pipeline alone covers about one row of DRAM latency)
-        const bool resid = (a.flags & F_RESID) != 0;
-        const bool mon = (a.flags & (F_RESID | F_MON)) != 0;
-        const C* upx = a.uprev + 2 * ctl.base + x;
-        const C* upy = upx + ctl.plane;
+        const C* upx = a.uprev + ctl.base + ibase;
         auto prefetch_rows = [&](int r) {  // thread TP, residual steps, rows of this item only
             if (r < y1) {
                 const long long o = (long long)r * nx + x0;
                 prefetch_l2(a.drho + ctl.base + o, CW * sizeof(C));
                 prefetch_l2(a.uprev + 2 * ctl.base + o, CW * sizeof(C));
-                prefetch_l2(a.uprev + 2 * ctl.base + ctl.plane + o, CW * sizeof(C));
+                prefetch_l2(a.uprev + 2 * ctl.base + PL + o, CW * sizeof(C));
             }
         };
-        C upx_next[NC], upy_next[NC], upx_next2[NC], upy_next2[NC];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) upx_next[c] = upy_next[c] = upx_next2[c] = upy_next2[c] = C(0);
+        P2 upx_next = p2(0.f), upy_next = p2(0.f), upx_next2 = p2(0.f), upy_next2 = p2(0.f);
         if (resid) {
             if (t == TP)
                 for (int r = y0 + 2; r < y0 + 6; ++r) prefetch_rows(r);
-            load_cols<C, NC>(upx + (long long)y0 * nx, upx_next);
-            load_cols<C, NC>(upy + (long long)y0 * nx, upy_next);
+            upx_next = load_pair(upx);
+            upy_next = load_pair(upx + PL);
             if (y0 + 1 < y1) {
-                load_cols<C, NC>(upx + (long long)(y0 + 1) * nx, upx_next2);
-                load_cols<C, NC>(upy + (long long)(y0 + 1) * nx, upy_next2);
+                upx_next2 = load_pair(upx + nx);
+                upy_next2 = load_pair(upx + PL + nx);
             }
         }
         __syncthreads();
         if (t == TI) {
             fence_proxy_async();
-            for (int r = rbase + K; r < rbase + K + 2 && r <= rlast; ++r) issue(idx_of(r), x0, r);
+            for (int r = rbase + K; r < rbase + K + 2 && r <= rlast; ++r) {
+                issue(slot_off(r), x0, r);
+                issued_end = idx_of(r) + 1;
+            }
         }
 
-        for (int y = y0; y < y1; ++y) {
+        long long o = 0;  // offset of row y from the item's first row
+        uint32_t vo = 0;  // the same in 32 bits (the host keeps an item's rows below 2^30 elements)
+        uint32_t o0 = slot_off(y0), o1 = slot_off(y0 + 1), o2 = slot_off(y0 + 2);  // slots of rows y, y+1, y+2
+        uint32_t par2 = (idx_of(y0 + 2) / K) & 1u;                                  // and row y+2's phase
+        // one row; false: a wait gave up.  EVEN: the first of two rows
+        auto row = [&](const int y, const bool even, P2 (&dcur)[9], P2& dRc, P2& jxc, P2& jyc, P2 (&dnext)[9], P2& dRn, P2& jxn,
+                       P2& jyn) -> bool {
             // 1. moments of row y+1 (its own populations are the next row's collision input);
             //    edge strips patch row y+4, which the moments of iteration y+2 read first
-            if (y + 2 <= rlast && !wait_row(y + 2)) s_bad = 1;
+            //    edge strips' halo columns: HALO2 takes rows y+1 and y+2 in one pass every other row
+            if (!mbar_wait(bar_at(o2), par2, ctl.max_wait_ns)) s_bad = 1;  // (y + 2 <= rlast)
+            const uint32_t o3 = next_slot(o2);
+            const uint32_t par3 = o3 == 0 ? par2 ^ 1u : par2;
             if (patcher && y + 4 <= rlast) {
                 if (!wait_row(y + 4)) s_bad = 1;
                 else patch_store(y + 4, pv_a);
                 pv_a = pv_b;
                 pv_b = patch_load(y + 6);
             }
-            moments_row(y + 1, dnext, dRn, jxn, jyn);
-            C drho_prev[NC], upx_cur[NC], upy_cur[NC];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                drho_prev[c] = drho_next[c];
-                drho_next[c] = drho_next2[c];
-                upx_cur[c] = upx_next[c];
-                upy_cur[c] = upy_next[c];
-            }
-            if (y + 2 < y1) load_cols<C, NC>(drow + (long long)(y + 2) * nx, drho_next2);
-            if (fluid) {
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    phi_cur[c] = phi_nxt[c];
-                    if (y + 1 < y1) phi_nxt[c] = phrow[(long long)(y + 1) * nx + c];
+            moments_row(y + 1, o0, o1, o2, dnext, dRn, jxn, jyn, un_x, un_y);
+            if constexpr (HALO2) {
+                if (even && t < 4) {
+                    const bool second = t >= 2 && y + 2 < y1;
+                    if (second && !mbar_wait(bar_at(o3), par3, ctl.max_wait_ns)) s_bad = 1;
+                    const int r = y + 1 + (t >> 1);
+                    if ((t < 2 || second) && r < ny)
+                        halo_node(r, (t & 1) == 0 ? -1 : CW, second ? o1 : o0, second ? o2 : o1, second ? o3 : o2);
                 }
+            } else {
+                if (t < 2 && y + 1 < ny) halo_node(y + 1, t == 0 ? -1 : CW, o0, o1, o2);
             }
+            const P2 drho_prev = drho_next, upx_cur = upx_next, upy_cur = upy_next;
+            drho_next = drho_next2;
+            if (y + 2 < y1) drho_next2 = load_pair(field_at(a.drho + 2LL * nx, o, vo));
+            double2 phi_cur = phi_nxt;
+            if (fluid && y + 1 < y1) phi_nxt = *reinterpret_cast<const double2*>(phrow + o + nx);
             if (resid) {
                 if (t == TP) prefetch_rows(y + 6);
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    upx_next[c] = upx_next2[c];
-                    upy_next[c] = upy_next2[c];
-                }
+                upx_next = upx_next2;
+                upy_next = upy_next2;
                 if (y + 2 < y1) {
-                    load_cols<C, NC>(upx + (long long)(y + 2) * nx, upx_next2);
-                    load_cols<C, NC>(upy + (long long)(y + 2) * nx, upy_next2);
+                    upx_next2 = load_pair(upx + o + 2 * nx);
+                    upy_next2 = load_pair(upx + PL + o + 2 * nx);
                 }
             }
             __syncthreads();
-            if (s_bad) { bad = true; break; }
+            if (s_bad) return false;
             // 2. refill the slot of row y (no longer read) with row y+K
             if (t == TI && y + K <= rlast) {
                 fence_proxy_async();
-                issue(idx_of(y + K), x0, y + K);
+                issue(o0, x0, y + K);
+                issued_end = idx_of(y + K) + 1;
             }
             // brackets of row y+4: its copy was waited by the shifter lanes (patchers) and its
             // halo patched before the barrier above; the first pull that reads it is that of
             // row y+3, two barriers later
             if (shifter && y + 4 <= rlast) shift_row(y + 4);
-            // 3. collision of row y, node by node, then the row's stores
+            // 3. collision of row y, both nodes together, then the row's stores
             {
-                const long long pn = (long long)y * nx + x;  // first own node
-                C so_xx[NC], so_xy[NC], so_yy[NC];
-#pragma unroll
-                for (int c = 0; c < NC; ++c) so_xx[c] = so_xy[c] = so_yy[c] = C(0);
-                if (SMODE == 1) {
-                    const C* s3 = a.sig3 + 3 * ctl.base + pn;
-                    load_cols<C, NC>(s3, so_xx);
-                    load_cols<C, NC>(s3 + ctl.plane, so_xy);
-                    load_cols<C, NC>(s3 + 2 * ctl.plane, so_yy);
+                // the neighbouring columns' velocities: from the neighbouring lanes (across a warp's
+                // border from shared memory), or from the ring
+                float2 uw, ue;
+                if constexpr (SHUFFLE) {
+                    const float2 bw = edge[4 * (y & 3) + wid], be = edge[4 * (y & 3) + 2 + wid];
+                    uw = make_float2(__shfl_up_sync(0xffffffffu, hi(u0_x), 1), __shfl_up_sync(0xffffffffu, hi(u0_y), 1));
+                    ue = make_float2(__shfl_down_sync(0xffffffffu, lo(u0_x), 1), __shfl_down_sync(0xffffffffu, lo(u0_y), 1));
+                    if (lane == 0) uw = bw;
+                    if (lane == 31) ue = be;
+                } else {
+                    uw = *reinterpret_cast<const float2*>(ring(y, col0 - 1));
+                    ue = *reinterpret_cast<const float2*>(ring(y, col0 + 2));
                 }
-                C D[NC][9], sxx[NC], syy[NC], sxy[NC], drho_new[NC], urx[NC], ury[NC];
+                const P2 Kx = p2(__fsub_rn(hi(u0_x), uw.x), __fsub_rn(ue.x, lo(u0_x)));
+                const P2 Kc = p2(__fsub_rn(hi(u0_y), uw.y), __fsub_rn(ue.y, lo(u0_y)));
+                P2 By, Ey;
+                if (y == 0) {
+                    P2 x2, y2;
+                    wall_pair(2, x2, y2);
+                    By = wall_difference_first(u0_x, un_x, x2);
+                    Ey = wall_difference_first(u0_y, un_y, y2);
+                } else if (y == ny - 1) {
+                    P2 x2, y2;
+                    wall_pair(y - 2, x2, y2);
+                    By = wall_difference_last(u0_x, us_x, x2);
+                    Ey = wall_difference_last(u0_y, us_y, y2);
+                } else {
+                    By = sub(un_x, us_x);
+                    Ey = sub(un_y, us_y);
+                }
+                P2 so_xx = p2(0.f), so_xy = p2(0.f), so_yy = p2(0.f);
+                if (SMODE == 1) {
+                    const C* s3 = a.sig3 + 2 * ctl.base + ibase + o;
+                    so_xx = load_pair(s3);
+                    so_xy = load_pair(s3 + PL);
+                    so_yy = load_pair(s3 + 2 * PL);
+                }
+                PairState s;
+                P2 om = q.om, nom = q.nom, k2 = q.k2;
+                if constexpr (SCHEME == 1) {
+                    s = constitutive_gn(P, q, Kx, By, Kc, Ey, dRc, jxc, jyc, &om);
+                    nom = mul(om, p2(-1.f));
+                    k2 = fma(p2(-0.5f), om, p2(1.f));
+                } else {
+                    P2 tau_M = p2(0.f);
+                    if constexpr (SCHEME == 3) {
+                        double2 phi_new;
+                        const C t0 = relaxation_time_ext<C>(P, 0.5f * lo(Kx), 0.5f * lo(By), 0.5f * lo(Kc), 0.5f * lo(Ey),
+                                                            lo(dRc), lo(drho_prev), phi_cur.x, &phi_new.x);
+                        const C t1 = relaxation_time_ext<C>(P, 0.5f * hi(Kx), 0.5f * hi(By), 0.5f * hi(Kc), 0.5f * hi(Ey),
+                                                            hi(dRc), hi(drho_prev), phi_cur.y, &phi_new.y);
+                        tau_M = p2(t0, t1);
+                        if (fluid) *reinterpret_cast<double2*>(a.phi + ibase + o) = phi_new;
+                    }
+                    s = constitutive<SMODE, BND == 1, SCHEME == 3>(q, Kx, By, Kc, Ey, dRc, jxc, jyc, drho_prev, so_xx, so_xy,
+                                                                   so_yy, tau_M);
+                }
+                const P2 rho_h = sub(add(p2(1.f), s.dReq), s.drho);
+                {  // velocity_ok of both nodes: |u| <= guard without a division (false for NaN)
+                    const P2 j2 = fma(jyc, jyc, mul(jxc, jxc)), g2 = mul(mul(p2(a.guard * a.guard), rho_h), rho_h);
+                    vbad |= !(lo(j2) <= lo(g2)) | !(hi(j2) <= hi(g2));
+                }
+                P2 D[9];
+                collide<SCHEME != 0>(q, s, dcur, D, om, nom, k2);
+                T* po = a.pout + 8 * ctl.base;
+                if (sr) {
+                    const uint32_t node = (uint32_t)((long long)y * nx + x0 + col0);
+                    C d0[9], d1[9], D0[9], D1[9];
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const int col = col0 + c;
-                    const C* uc = uring + 2 * ((y & 3) * UW + col + 1);
-                    const V2 ue = get_u(uc + 2), uw = get_u(uc - 2);  // columns col+1, col-1
-                    const C ka = C(0.5) * (ue.x - uw.x);
-                    const C kc = C(0.5) * (ue.y - uw.y);
-                    C kb, ke;
-                    const V2 un = get_u(uring + 2 * (((y + 1) & 3) * UW + col + 1));  // row y+1
-                    const V2 us = get_u(uring + 2 * (((y + 3) & 3) * UW + col + 1));  // row y-1
-                    if (y == 0) {
-                        const V2 u0 = get_u(uc);
-                        const V2 un2 = get_u(uring + 2 * (((y + 2) & 3) * UW + col + 1));
-                        kb = C(0.5) * (C(-3) * u0.x + C(4) * un.x - un2.x);
-                        ke = C(0.5) * (C(-3) * u0.y + C(4) * un.y - un2.y);
-                    } else if (y == ny - 1) {
-                        const V2 u0 = get_u(uc);
-                        const V2 us2 = get_u(uring + 2 * (((y + 2) & 3) * UW + col + 1));  // row y-2
-                        kb = C(0.5) * (C(3) * u0.x - C(4) * us.x + us2.x);
-                        ke = C(0.5) * (C(3) * u0.y - C(4) * us.y + us2.y);
-                    } else {
-                        kb = C(0.5) * (un.x - us.x);
-                        ke = C(0.5) * (un.y - us.y);
+                    for (int i = 0; i < 9; ++i) {
+                        d0[i] = lo(dcur[i]); d1[i] = hi(dcur[i]);
+                        D0[i] = lo(D[i]); D1[i] = hi(D[i]);
                     }
-                    NodeState<C> s;
-                    C om_n = P.omega;
-                    if constexpr (SCHEME == 1) {
-                        s = constitutive_gn<C>(P, ka, kb, kc, ke, dRc[c], jxc[c], jyc[c], &om_n);
-                    } else if constexpr (SCHEME == 3) {
-                        double phi_new;
-                        const C tau_M = relaxation_time_ext<C>(P, ka, kb, kc, ke, dRc[c], drho_prev[c], phi_cur[c], &phi_new);
-                        s = constitutive<C, SMODE, true>(P, ka, kb, kc, ke, dRc[c], jxc[c], jyc[c], drho_prev[c], so_xx[c],
-                                                         so_xy[c], so_yy[c], tau_M);
-                        if (fluid) a.phi[ctl.base + pn + c] = phi_new;
-                    } else {
-                        s = constitutive<C, SMODE>(P, ka, kb, kc, ke, dRc[c], jxc[c], jyc[c], drho_prev[c], so_xx[c],
-                                                   so_xy[c], so_yy[c]);
-                    }
-                    const C rho_h = C(1) + s.dReq - s.drho;
-                    vbad |= !velocity_ok<C>(jxc[c], jyc[c], rho_h, a.guard);  // NaN or too fast
-                    // the schemes' variants call the collision exactly as the tile kernel's do (the
-                    // same expression, so the same contraction into fused multiply-adds)
-                    if constexpr (SCHEME == 1) collide_impl<C, true>(P, s, dcur[c], D[c], om_n, C(1) - C(0.5) * om_n, P.gx, C(0));
-                    else if constexpr (SCHEME == 3) collide_impl<C, true>(P, s, dcur[c], D[c], P.omega, P.k2, P.gx, C(0));
-                    else collide_node<C>(P, s, dcur[c], D[c]);
-                    sxx[c] = s.sxx;
-                    syy[c] = s.syy;
-                    sxy[c] = s.sxy;
-                    drho_new[c] = s.drho;
-                    urx[c] = ury[c] = C(0);
-                    if (a.flags & (F_SAVE_U | F_RESID | F_MON)) {
-                        const C ih = Arith<C>::div(C(1), rho_h);
-                        urx[c] = jxc[c] * ih;
-                        ury[c] = jyc[c] * ih;
-                        if (mon) {
-                            const C u2 = urx[c] * urx[c] + ury[c] * ury[c];
-                            if (resid) {
-                                const C dx_ = urx[c] - upx_cur[c], dy_ = ury[c] - upy_cur[c];
-                                r_du2 += dx_ * dx_ + dy_ * dy_;
-                            }
-                            r_u2 += u2;
-                            r_ux += urx[c];
-                            r_umax2 = fmax(r_umax2, u2);
+                    store_node<T, C>(field_at(po, o, vo), PL, d0, D0, true, a.sr_key, node);
+                    store_node<T, C>(field_at(po, o, vo) + 1, PL, d1, D1, true, a.sr_key, node + 1);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) store_pop_pair(field_at(po + i * PL, o, vo), add(dcur[i], D[i]));
+                }
+                store_pair(field_at(a.drho, o, vo), s.drho);
+                if (SMODE == 1) {
+                    C* s3 = a.sig3 + 2 * ctl.base + ibase + o;
+                    store_pair(s3, s.sxx);
+                    store_pair(s3 + PL, s.sxy);
+                    store_pair(s3 + 2 * PL, s.syy);
+                }
+                if (store_sigma) {  // (the zz plane holds 0 from lb_create on)
+                    C* s4 = a.sig4 + 3 * ctl.base;
+                    store_pair(field_at(s4, o, vo), s.sxx);
+                    store_pair(field_at(s4 + PL, o, vo), s.syy);
+                    store_pair(field_at(s4 + 3 * PL, o, vo), s.sxy);
+                }
+                if (want_u) {
+                    const P2 ih = rcp(rho_h);
+                    const P2 urx = mul(jxc, ih), ury = mul(jyc, ih);
+                    if (mon) {
+                        const P2 u2 = fma(ury, ury, mul(urx, urx));
+                        if (resid) {
+                            const P2 dx_ = sub(urx, upx_cur), dy_ = sub(ury, upy_cur);
+                            r_du2 = add(r_du2, fma(dy_, dy_, mul(dx_, dx_)));
                         }
+                        r_u2 = add(r_u2, u2);
+                        r_ux = add(r_ux, urx);
+                        r_umax2 = fmaxf(r_umax2, fmaxf(lo(u2), hi(u2)));
                     }
-                }
-                T* po = a.pout + 9 * ctl.base + pn;
-                store_cols_pop<T, C, NC>(po, ctl.plane, dcur, D, (a.flags & F_SR) != 0, a.sr_key, (uint32_t)pn);
-                store_cols<C, NC>(a.drho + ctl.base + pn, drho_new);
-                if (SMODE == 1) {
-                    C* s3 = a.sig3 + 3 * ctl.base + pn;
-                    store_cols<C, NC>(s3, sxx);
-                    store_cols<C, NC>(s3 + ctl.plane, sxy);
-                    store_cols<C, NC>(s3 + 2 * ctl.plane, syy);
-                }
-                if (a.flags & F_STORE_SIGMA) {  // (the zz plane holds 0 from lb_create on)
-                    C* s4 = a.sig4 + 4 * ctl.base + pn;
-                    store_cols<C, NC>(s4, sxx);
-                    store_cols<C, NC>(s4 + ctl.plane, syy);
-                    store_cols<C, NC>(s4 + 3 * ctl.plane, sxy);
-                }
-                if (a.flags & F_SAVE_U) {
-                    C* up_ = a.uprev + 2 * ctl.base + pn;
-                    store_cols<C, NC>(up_, urx);
-                    store_cols<C, NC>(up_ + ctl.plane, ury);
+                    if (save_u) {
+                        C* up_ = a.uprev + ctl.base + ibase + o;
+                        store_pair(up_, urx);
+                        store_pair(up_ + PL, ury);
+                    }
                 }
             }
+            us_x = u0_x;
+            us_y = u0_y;
+            u0_x = un_x;
+            u0_y = un_y;
+            o0 = o1;
+            o1 = o2;
+            o2 = o3;
+            par2 = par3;
+            o += nx;
+            vo += (uint32_t)nx;
+            return true;
+        };
+        if constexpr (!UNROLL2) {
+#pragma unroll 1
+            for (int y = y0; y < y1; ++y) {
+                if (!row(y, ((y - y0) & 1) == 0, dA, dRa, jxa, jya, dB, dRb, jxb, jyb)) { bad = true; break; }
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-#pragma unroll
-                for (int i = 0; i < 9; ++i) dcur[c][i] = dnext[c][i];
-                dRc[c] = dRn[c];
-                jxc[c] = jxn[c];
-                jyc[c] = jyn[c];
+                for (int i = 0; i < 9; ++i) dA[i] = dB[i];
+                dRa = dRb;
+                jxa = jxb;
+                jya = jyb;
+            }
+        } else {
+            for (int y = y0; y < y1; y += 2) {
+                if (!row(y, true, dA, dRa, jxa, jya, dB, dRb, jxb, jyb)) { bad = true; break; }
+                if (y + 1 >= y1) break;
+                if (!row(y + 1, false, dB, dRb, jxb, jyb, dA, dRa, jxa, jya)) { bad = true; break; }
             }
         }
         __syncthreads();  // every slot read of this item is done before the next item's copies
         if (!bad && mon) {
             // block reduction of (sum du^2, sum u^2, sum u_x, max |u|) into this item's partials
-            double v[4] = {(double)r_du2, (double)r_u2, (double)r_ux, (double)r_umax2};
+            double v[4] = {(double)lo(r_du2) + (double)hi(r_du2), (double)lo(r_u2) + (double)hi(r_u2),
+                           (double)lo(r_ux) + (double)hi(r_ux), (double)r_umax2};
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
@@ -631,7 +706,7 @@ __global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME =
                 v[2] += __shfl_xor_sync(0xffffffffu, v[2], o);
                 v[3] = fmax(v[3], __shfl_xor_sync(0xffffffffu, v[3], o));
             }
-            double* red = reinterpret_cast<double*>(uring);  // the velocity ring is free now
+            double* red = reinterpret_cast<double*>(uwall);  // (free now)
             if ((t & 31) == 0)
                 for (int k = 0; k < 4; ++k) red[4 * (t >> 5) + k] = v[k];
             __syncthreads();
@@ -654,8 +729,8 @@ __global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME =
         // into each slot is the only one that can still be in flight (bounded by kMarchDrainNs)
         if (t == TI) {
             atomicOr(ctl.timeout_flag, 2);
-            for (int k = 0; k < K; ++k)
-                if (last_issued[k] != 0xffffffffu) mbar_wait(&bars[k], (last_issued[k] / K) & 1u, kMarchDrainNs);
+            for (uint32_t k = issued_end > (uint32_t)K ? issued_end - K : 0u; k < issued_end; ++k)
+                mbar_wait(bar_at((k % K) * SLOT), (k / K) & 1u, kMarchDrainNs);
         }
         __syncthreads();
     }
@@ -684,41 +759,43 @@ __global__ void __launch_bounds__(CW / NC, NC == 2 ? LBK_MARCH_MINB2 : (SCHEME =
 
 namespace lbk {
 constexpr int kMarchW = 128;  // columns per CTA (one strip)
-constexpr int kMarchK = 8;    // shared-memory row slots (copies run K-2 rows ahead)
-#ifndef LBK_MARCH_NC_BF16
-#define LBK_MARCH_NC_BF16 2
-#endif
-// Adjacent columns per thread.  BF16 storage moves 56 B per node against FP32's 92, so its step is
-// bound by instruction issue: two columns per thread share the per-row address, ring and loop
-// work and pack their stores into bf16x2 words (497 -> 366 instructions per node; with 7 CTAs per
-// SM 57.7 -> 73.8 GLUPS at 4096 x 4096).  The FP32 step is
-// bound by HBM and keeps one column per thread (two measured 4 % slower: a 64-thread CTA at 161
-// registers leaves 10 warps per SM to cover the memory latency).  The BF16 boundary variants
-// take two columns as well (pressure-driven ends 49.8 -> 59.3, moving wall 55.1 -> 72.0 GLUPS).
-template <typename T, int BND>
-constexpr int march_nc() { return std::is_same<T, __nv_bfloat16>::value ? LBK_MARCH_NC_BF16 : 1; }
+// How the kernel is shaped, and what it measured (us per step; FP32 at 4096 x 4096 / 1024 x 1024, BF16
+// at 8192 x 2048 / 1024 x 1024; one column per thread in scalar FP32 before: 274 / 24.8 and 222 / 24.8).
+// Two columns per thread as packed FP32 take the instructions per node from 468 to 268 (FP32) and from
+// 393 to 268 (BF16); what is left is bound by HBM in FP32 at sizes beyond L2 (0.9 of the copy
+// bandwidth) and by the latency of dependent instructions elsewhere: a packed operation holds its
+// warp for about four cycles, and 160 registers leave 12 warps per SM.
+//  - six CTAs of two warps per SM.  Eight (128 registers) spill, or pull the populations twice: BF16
+//    218 / 22.9 against 215 / 20.8.
+//  - seven row slots: with the halo columns of two rows taken together (which waits one row
+//    further ahead) six slots leave too little in flight for HBM (FP32 293 / 20.8 against 253 / 22.4).
+//    Seven fit six CTAs in FP32 without the ring of velocity rows, hence the warp shuffles; BF16 has
+//    the room and keeps the ring (215 / 20.8 against 223 / 20.8 with shuffles).
+//  - the row loop written out for two rows, so that no register moves between them: BF16 230 -> 215;
+//    with pressure-driven ends one row at a time is faster (2048 x 1000: 53.8 against 56.4).
+constexpr int kMarchK = 7;  // shared-memory row slots
 
 template <typename T, typename C, int SMODE, int BND = 0, int SCHEME = 0>
 cudaError_t launch_step_march(const CUtensorMap& map, const StepArgs<T, C>& a, const MarchCtl& ctl, int grid,
                               cudaStream_t s) {
-    constexpr int NC = march_nc<T, BND>();
-    auto k = k_step_march<T, C, SMODE, kMarchW, NC, kMarchK, BND, SCHEME>;
-    const size_t smem = march_smem_bytes<T, C, kMarchW, kMarchK>();
+    constexpr int K = kMarchK;
+    auto k = k_step_march<T, C, SMODE, kMarchW, K, BND, SCHEME>;
+    const size_t smem = march_smem_bytes<T, C, kMarchW, K>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
-    k<<<grid, kMarchW / NC, smem, s>>>(map, a, ctl);
+    k<<<grid, kMarchW / 2, smem, s>>>(map, a, ctl);
     return cudaGetLastError();
 }
 
 template <typename T, typename C, int SMODE, int BND = 0, int SCHEME = 0>
 cudaError_t march_occupancy(int* blocks_per_sm) {
-    constexpr int NC = march_nc<T, BND>();
-    auto k = k_step_march<T, C, SMODE, kMarchW, NC, kMarchK, BND, SCHEME>;
-    const size_t smem = march_smem_bytes<T, C, kMarchW, kMarchK>();
+    constexpr int K = kMarchK;
+    auto k = k_step_march<T, C, SMODE, kMarchW, K, BND, SCHEME>;
+    const size_t smem = march_smem_bytes<T, C, kMarchW, K>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, kMarchW / NC, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, kMarchW / 2, smem);
 }
 }  // namespace lbk
