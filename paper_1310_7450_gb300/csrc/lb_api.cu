@@ -28,13 +28,15 @@
 namespace lbk {
 // learned warm start (lb_warmstart.cu)
 struct WsChan {
-    double g, G, tau0, theta, gamma_c;
+    double G, tau0, theta, gamma_c;
 };
-cudaError_t launch_ws_closed_form(int n_ch, const WsChan* prm, const int* nys, const int* row_off, double* rows,
-                                  double* grid, double* scale, cudaStream_t s);
-cudaError_t launch_ws_decode(int n_ch, const float* pred, const float* t_mu, const float* t_sd, const double* grid,
-                             const double* scale, const double* rows, const int* nys, const int* row_off,
-                             const long long* node_off, int nx, double* u, double* rho, double* drho, cudaStream_t s);
+cudaError_t launch_ws_closed_form(int n_ch, const WsChan* prm, const double* gx, const int* nys, const int* row_off,
+                                  double* rows, double* grid, double* scale, cudaStream_t s);
+template <typename T, typename C>
+cudaError_t launch_ws_start(int n_ch, int max_ny, int n_sm, const float* pred, const float* t_mu, const float* t_sd,
+                            const double* grid, const double* scale, const double* rows, const double* gx, const int* nys,
+                            const int* row_off, const long long* base, const long long* P, int nx, int gpbc, T* pop, C* drho,
+                            C* sig3, cudaStream_t s);
 template <typename F>
 cudaError_t launch_ws_targets(int n_ch, const F* fu, const F* fs, const double* grid, const double* scale, const int* nys,
                               const long long* node_off, int nx, float* targets, cudaStream_t s);
@@ -1922,34 +1924,43 @@ static lb_status ws_closed_form(lb_handle* h) {
         LB_CK(cudaMalloc(&h->ws_rows, sizeof(double) * 3 * (size_t)h->gny));
         LB_CK(cudaMalloc(&h->ws_grid, sizeof(double) * 3 * 256 * (size_t)h->n_ch));
         LB_CK(cudaMalloc(&h->ws_scale, sizeof(double) * 3 * (size_t)h->n_ch));
-        LB_CK(cudaMemcpy(h->ws_row_off, h->row_off.data(), sizeof(int) * h->n_ch, cudaMemcpyHostToDevice));
+        std::vector<WsChan> prm(h->n_ch);
+        for (int c = 0; c < h->n_ch; ++c)
+            prm[c] = WsChan{h->params[c].G_inf, h->params[c].tau0, h->params[c].theta, h->params[c].gamma_c};
+        LB_CK(cudaMemcpyAsync(h->ws_row_off, h->row_off.data(), sizeof(int) * h->n_ch, cudaMemcpyHostToDevice, h->stream));
+        LB_CK(cudaMemcpyAsync(h->ws_prm, prm.data(), sizeof(WsChan) * h->n_ch, cudaMemcpyHostToDevice, h->stream));
+        LB_CK(cudaStreamSynchronize(h->stream));  // (prm goes; the first call only)
     }
-    std::vector<WsChan> prm(h->n_ch);
     for (int c = 0; c < h->n_ch; ++c) {
         const lb_params& p = h->params[c];
         if (!(p.G_inf > 0.0) || !(p.tau0 > 0.0) || !(p.g_x > 0.0))
             return fail(LB_EINVAL, "lb_warmstart: every channel needs G_inf > 0, tau0 > 0 and g_x > 0 (the closed form)%s");
-        prm[c] = WsChan{p.g_x, p.G_inf, p.tau0, p.theta, p.gamma_c};
     }
-    LB_CK(cudaStreamSynchronize(h->stream));
-    LB_CK(cudaMemcpy(h->ws_prm, prm.data(), sizeof(WsChan) * h->n_ch, cudaMemcpyHostToDevice));
-    LB_CK(launch_ws_closed_form(h->n_ch, (const WsChan*)h->ws_prm, h->ny_d, (const int*)h->ws_row_off,
+    // (the body force, the only one that changes, is read from its stream-ordered device copy)
+    LB_CK(launch_ws_closed_form(h->n_ch, (const WsChan*)h->ws_prm, h->gx_d, h->ny_d, (const int*)h->ws_row_off,
                                 (double*)h->ws_rows, (double*)h->ws_grid, (double*)h->ws_scale, h->stream));
     return LB_OK;
 }
 
 lb_status lb_warmstart_apply(lb_handle* h, const float* pred, const float* t_mu, const float* t_sd) {
     if (!h || (!t_mu) != (!t_sd)) return fail(LB_EINVAL, "lb_warmstart_apply: null handle, or only one of t_mu, t_sd%s");
-    const long long N = h->nodes;
-    lb_status st = ensure_hstage(h, (size_t)N * 4 * sizeof(double));
+    lb_status st = ws_closed_form(h);
     if (st != LB_OK) return st;
-    st = ws_closed_form(h);
-    if (st != LB_OK) return st;
-    double* su = (double*)h->hstage;
-    LB_CK(launch_ws_decode(h->n_ch, pred, t_mu, t_sd, (const double*)h->ws_grid, (const double*)h->ws_scale,
-                           (const double*)h->ws_rows, h->ny_d, (const int*)h->ws_row_off, h->node_off_d, h->nx, su,
-                           su + 2 * N, su + 3 * N, h->stream));
-    return set_fields_dev(h, su, su + 2 * N, su + 3 * N);
+    int n_sm = 0, max_ny = 0;
+    LB_CK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->dev));
+    for (int v : h->ny) max_ny = std::max(max_ny, v);
+    const cudaError_t e = with_types(h->prec, [&](auto tt, auto tc) {
+        LB_TYPES(tt, tc);
+        return launch_ws_start<T, C>(h->n_ch, max_ny, n_sm, pred, t_mu, t_sd, (const double*)h->ws_grid,
+                                     (const double*)h->ws_scale, (const double*)h->ws_rows, h->gx_d, h->ny_d,
+                                     (const int*)h->ws_row_off, h->base_d, h->P_d, h->nx, h->gpbc ? 1 : 0, (T*)h->popA,
+                                     (C*)h->drho, h->smode == 1 ? (C*)h->sig3 : nullptr, h->stream);
+    });
+    if (e != cudaSuccess) return cuda_fail(e, "lb_warmstart_apply: start state");
+    if (h->phi) LB_CK(cudaMemsetAsync(h->phi, 0, h->planes * sizeof(double), h->stream));  // fluidity unset
+    LB_CK(cudaStreamSynchronize(h->stream));
+    h->uprev_state = -10;
+    return LB_OK;
 }
 
 lb_status lb_warmstart_targets(lb_handle* h, float* targets) {
