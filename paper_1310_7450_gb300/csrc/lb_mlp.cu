@@ -13,6 +13,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <new>
@@ -40,119 +41,357 @@ lb_status mfail(lb_status s, const char* what) {
         }                                                                    \
     } while (0)
 
-constexpr int TB = 16;  // tile edge of the product kernels
+// ---- the products --------------------------------------------------------------------------------
+// All of them are C[m][n] = sum_k A(m, k) B(k, n) in FP32, with what follows the product done where its
+// sums are formed: the bias and tanh of a forward layer, the loss and its gradient behind the last one, the
+// tanh' factor of a backward layer, Adam behind a weight gradient.
+//
+// A product is 17 to 50 million multiply-adds, 0.4 to 1.3 us of the part's FP32 rate: what bounds it is
+// launching, reaching the operands in L2 and having enough CTAs, not arithmetic.  So a CTA takes a small tile
+// (32 x 32, or 16 x 32 where that leaves fewer than one tile per SM), stages its operands over the whole depth at
+// once, and splits the depth over groups of threads (8 or 16) that keep 4 x 4 sums per thread; the groups' sums are
+// added in a fixed order in shared memory.  The launches of a step are five: the first layer (a few inputs)
+// is evaluated where the second one stages its operand, and a weight gradient shares its launch with the
+// input gradient of the layer below.  Each kernel is set up while the one before it drains (programmatic
+// dependent launch) and stages what that one does not write; see Ready.
+// 4 -> 256 -> 256 -> 768, us per training step / forward pass: batch 24 67.7 / 24.6 -> 25.2 / 9.8, 256 129.6 /
+// 39.0 -> 43.5 / 20.6, 512 213 / 58 -> 68.7 / 26.2 (before: 16 x 16 tiles, 16-deep slabs, ten launches).
+// 16 x 32 tiles at batch 256 take 48.7 / 21.5, 32 x 32 at 512 70.2 / 31.3 (the hidden layers' 128 tiles).
+constexpr int kProdThreads = 512;
+constexpr int kProdTn = 32;                          // tile width
+constexpr int kFirstIn = 8;                          // inputs of a first layer evaluated inside the second
+constexpr size_t kProdSmem = 200 * 1024;             // operand panels of one slab
 
-// Y[b][o] = act( sum_i X[b][i] W[o][i] + bias[o] ), W in BF16, FP32 accumulation.
-// act: 0 = identity, 1 = tanh.  Tiled: a 16x16 output tile per CTA, 16-wide slabs of X and W in
-// shared memory.
-__global__ void k_linear_fwd(const float* __restrict__ X, const __nv_bfloat16* __restrict__ W,
-                             const float* __restrict__ bias, float* __restrict__ Y, int B, int I, int O, int act) {
-    __shared__ float xs[TB][TB + 1], ws[TB][TB + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int b = blockIdx.y * TB + ty, o = blockIdx.x * TB + tx;
-    float acc = 0.f;
-    for (int i0 = 0; i0 < I; i0 += TB) {
-        const int xb = blockIdx.y * TB + ty, xi = i0 + tx;
-        xs[ty][tx] = (xb < B && xi < I) ? X[(long long)xb * I + xi] : 0.f;
-        const int wo = blockIdx.x * TB + ty, wi = i0 + tx;
-        ws[ty][tx] = (wo < O && wi < I) ? __bfloat162float(W[(long long)wo * I + wi]) : 0.f;
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < TB; ++k) acc = fmaf(xs[ty][k], ws[tx][k], acc);
-        __syncthreads();
-    }
-    if (b < B && o < O) {
-        float v = acc + bias[o];
-        if (act == 1) v = tanhf(v);
-        Y[(long long)b * O + o] = v;
-    }
+enum Epilogue { EP_TANH, EP_LINEAR, EP_MSE, EP_DTANH, EP_GRAD };
+
+// What a kernel may read before the grid before it in the stream has finished.  A kernel's blocks start when all
+// blocks of that grid have passed their own wait, so the grids before that one have finished: the weights
+// (written by the last launch of a step, or by the call before) are ready for every launch but the
+// first, and an activation or gradient is when the grid that writes it lies two launches back.
+enum Ready { READY_NONE, READY_B, READY_ALL };  // READY_ALL: both operands; only the results wait
+
+struct Adam {  // Adam (Kingma & Ba 2015) on the FP32 masters, then the BF16 working copy; p == nullptr: no update
+    float *p, *m, *v;
+    __nv_bfloat16* pb;
+    float lr, b1, b2, eps, c1, c2;
+};
+// (pk, mk, vk: the element's parameter and moments, loaded ahead)
+__device__ __forceinline__ void adam_update(const Adam& a, long long k, float gk, float pk, float mk, float vk) {
+    mk = a.b1 * mk + (1.f - a.b1) * gk;
+    vk = a.b2 * vk + (1.f - a.b2) * gk * gk;
+    a.m[k] = mk;
+    a.v[k] = vk;
+    const float upd = a.lr * (mk / a.c1) / (sqrtf(vk / a.c2) + a.eps);
+    pk = pk - upd;
+    a.p[k] = pk;
+    a.pb[k] = __float2bfloat16_rn(pk);
 }
 
-// dX[b][i] = sum_o dY[b][o] W[o][i]   (optionally times tanh'(A[b][i]) = 1 - A^2 of the input A)
-__global__ void k_linear_bwd_x(const float* __restrict__ dY, const __nv_bfloat16* __restrict__ W,
-                               const float* __restrict__ A, float* __restrict__ dX, int B, int I, int O) {
-    __shared__ float gs[TB][TB + 1], ws[TB][TB + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int b = blockIdx.y * TB + ty, i = blockIdx.x * TB + tx;
-    float acc = 0.f;
-    for (int o0 = 0; o0 < O; o0 += TB) {
-        const int gb = blockIdx.y * TB + ty, go = o0 + tx;
-        gs[ty][tx] = (gb < B && go < O) ? dY[(long long)gb * O + go] : 0.f;
-        const int wo = o0 + ty, wi = blockIdx.x * TB + tx;
-        ws[ty][tx] = (wo < O && wi < I) ? __bfloat162float(W[(long long)wo * I + wi]) : 0.f;
-        __syncthreads();
+struct Product {
+    const float* A;       // KMAJ: [m][k], else [k][m]
+    const void* B;        // KMAJ: BF16 [n][k]; else BF16 or FP32 [k][n]
+    float* C;             // [m][n] (EP_GRAD: null with Adam)
+    int M, N, K;
+    const float* bias;    // forward: [n]
+    const float* aux;     // EP_DTANH: activations [m][n]; EP_MSE: targets [m][n]
+    double* partial;      // EP_MSE: one sum of squares per tile
+    float scale;          // EP_MSE: 1 / (number of outputs)
+    float* bias_grad;     // EP_GRAD: row sums of A (null with Adam)
+    Adam w, b;            // EP_GRAD: the weights' and the biases' update
+    int tiles_n, tiles;
+    int slab;             // depth staged at once
+    // first layer evaluated in place of A (x != nullptr): A(m, k) = tanh(sum_i x[m][i] w1[k][i] + b1[k]),
+    // also written to a1 by the first column of tiles
+    const float* x;
+    const __nv_bfloat16* w1;
+    const float* b1;
+    float* a1;
+    int n_in;
+};
+// Wait for the grid before this one in the stream, and let the next one be set up.
+__device__ __forceinline__ void grid_dependency() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+__device__ __forceinline__ void load16(const float* p, float (&v)[4]) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+}
+__device__ __forceinline__ void load16(const __nv_bfloat16* p, float (&v)[8]) {
+    const uint4 q = *reinterpret_cast<const uint4*>(p);  // (a BF16 value is the high half of its FP32 one)
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-        for (int k = 0; k < TB; ++k) acc = fmaf(gs[ty][k], ws[k][tx], acc);
-        __syncthreads();
+    for (int j = 0; j < 4; ++j) {
+        v[2 * j] = __uint_as_float(w[j] << 16);
+        v[2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
     }
-    if (b < B && i < I) {
-        if (A) {
-            const float a = A[(long long)b * I + i];
-            acc *= (1.f - a * a);
+}
+__device__ __forceinline__ float load1(const float* p) { return *p; }
+__device__ __forceinline__ float load1(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+
+// Stage rows [r0, r0 + R) x depth [k0, k0 + kn) of an operand as dst[k][r] (row stride LD), zeros outside, in
+// pieces of 16 bytes.  KMAJ: src[r][k] (depth contiguous): eight rows x four pieces per warp, which reads 64
+// bytes of a row at a time and stores with few bank conflicts; else src[k][r].  U pieces per thread are on
+// their way together.
+template <typename E, int R, int LD, bool KMAJ>
+__device__ __forceinline__ void stage(float* dst, const E* __restrict__ src, int r0, int rows, int k0, int kn, int depth) {
+    const int t = threadIdx.x;
+    constexpr int V = 16 / (int)sizeof(E), U = sizeof(E) == 4 ? 6 : 4;
+    const int kp = (kn + V - 1) / V;  // pieces along the depth
+    const int pieces = KMAJ ? R * ((kp + 3) / 4 * 4) : kn * (R / V);
+    const bool vec = (KMAJ ? depth : rows) % V == 0 && reinterpret_cast<uintptr_t>(src) % 16 == 0;
+    for (int e0 = t; e0 < pieces; e0 += U * kProdThreads) {
+        float v[U][V];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int e = e0 + u * kProdThreads;
+#pragma unroll
+            for (int j = 0; j < V; ++j) v[u][j] = 0.f;
+            if (e >= pieces) continue;
+            if constexpr (KMAJ) {
+                const int r = (e & 7) + 8 * ((e >> 5) % (R / 8)), k = V * (((e >> 3) & 3) + 4 * ((e >> 5) / (R / 8)));
+                if (k >= kn || r0 + r >= rows) continue;
+                const E* p = src + (long long)(r0 + r) * depth + k0 + k;
+                if (vec && k + V <= kn) load16(p, v[u]);
+                else
+#pragma unroll
+                    for (int j = 0; j < V; ++j)
+                        if (k + j < kn) v[u][j] = load1(p + j);
+            } else {
+                const int r = V * (e % (R / V)), k = e / (R / V);
+                const E* p = src + (long long)(k0 + k) * rows + r0 + r;
+                if (vec && r0 + r + V <= rows) load16(p, v[u]);
+                else
+#pragma unroll
+                    for (int j = 0; j < V; ++j)
+                        if (r0 + r + j < rows) v[u][j] = load1(p + j);
+            }
         }
-        dX[(long long)b * I + i] = acc;
-    }
-}
-
-// dW[o][i] = sum_b dY[b][o] X[b][i];  dbias[o] = sum_b dY[b][o] (computed by the blockIdx.x == 0 column)
-__global__ void k_linear_bwd_w(const float* __restrict__ dY, const float* __restrict__ X, float* __restrict__ dW,
-                               float* __restrict__ db, int B, int I, int O) {
-    __shared__ float gs[TB][TB + 1], xs[TB][TB + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int o = blockIdx.y * TB + ty, i = blockIdx.x * TB + tx;
-    float acc = 0.f, accb = 0.f;
-    for (int b0 = 0; b0 < B; b0 += TB) {
-        const int gb = b0 + tx, go = blockIdx.y * TB + ty;
-        gs[ty][tx] = (gb < B && go < O) ? dY[(long long)gb * O + go] : 0.f;  // gs[o][b]
-        const int xb = b0 + ty, xi = blockIdx.x * TB + tx;
-        xs[ty][tx] = (xb < B && xi < I) ? X[(long long)xb * I + xi] : 0.f;   // xs[b][i]
-        __syncthreads();
 #pragma unroll
-        for (int k = 0; k < TB; ++k) {
-            acc = fmaf(gs[ty][k], xs[k][tx], acc);
-            accb += gs[ty][k];
+        for (int u = 0; u < U; ++u) {
+            const int e = e0 + u * kProdThreads;
+            if (e >= pieces) continue;
+            if constexpr (KMAJ) {
+                const int r = (e & 7) + 8 * ((e >> 5) % (R / 8)), k = V * (((e >> 3) & 3) + 4 * ((e >> 5) / (R / 8)));
+#pragma unroll
+                for (int j = 0; j < V; ++j)
+                    if (k + j < kn) dst[(k + j) * LD + r] = v[u][j];
+            } else {
+                const int r = V * (e % (R / V)), k = e / (R / V);
+#pragma unroll
+                for (int j = 0; j < V; j += 4)
+                    *reinterpret_cast<float4*>(dst + k * LD + r + j) = make_float4(v[u][j], v[u][j + 1], v[u][j + 2], v[u][j + 3]);
+            }
         }
-        __syncthreads();
     }
-    if (o < O && i < I) dW[(long long)o * I + i] = acc;
-    if (o < O && blockIdx.x == 0 && tx == 0) db[o] = accb;
 }
 
-// loss = mean (Y - T)^2 over B*O values; dY = 2 (Y - T)/(B*O).  One CTA per row block, partial
-// sums combined by the host in a fixed order.
-__global__ void k_mse(const float* __restrict__ Y, const float* __restrict__ T, float* __restrict__ dY,
-                      double* __restrict__ partial, long long n, float scale) {
-    __shared__ double red[256];
-    double s = 0.0;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const float d = Y[k] - T[k];
-        dY[k] = 2.f * d * scale;
-        s += (double)d * d;
+// One tile of a product.  TM: tile height; AK, BK: operand depth contiguous; E: type of B.
+template <int TM, bool AK, bool BK, typename E, int EP, int READY, bool FIRST = false>
+__device__ __forceinline__ void product_tile(const Product& q, int tile, float* smem) {
+    constexpr int LA = TM + 4, LB = kProdTn + 4;
+    constexpr int GT = (TM / 4) * (kProdTn / 4), G = kProdThreads / GT;  // threads per depth group, groups
+    const int t = threadIdx.x, g = t / GT, l = t % GT;
+    const int tn = 4 * (l % (kProdTn / 4)), tm = 4 * (l / (kProdTn / 4));
+    const int m0 = (tile / q.tiles_n) * TM, n0 = (tile % q.tiles_n) * kProdTn;
+    float* As = smem;
+    float* Bs = smem + (size_t)q.slab * LA;
+    const bool want_rows = EP == EP_GRAD && n0 == 0;  // (uniform) the row sums of A go with the first column of tiles
+    float acc[4][4] = {}, rs[4] = {};
+    // what the results need besides the sums: loaded ahead of the multiply-adds (pre[0]: bias, activation or
+    // parameter; pre[1], pre[2]: target or Adam's moments)
+    constexpr int OUT = TM * kProdTn / kProdThreads;
+    float pre[OUT][3];
+    for (int k0 = 0; k0 < q.K; k0 += q.slab) {
+        const int kn = min(q.slab, q.K - k0);
+        if (k0) __syncthreads();
+        if (READY == READY_NONE && k0 == 0) grid_dependency();
+        stage<E, kProdTn, LB, BK>(Bs, static_cast<const E*>(q.B), n0, q.N, k0, kn, q.K);
+        if (READY == READY_B && k0 == 0) grid_dependency();
+        if constexpr (FIRST) {  // (one slab: k0 = 0, kn = K)
+            // the first layer's weights as FP32 rows of kFirstIn, zero-padded; a thread keeps one row of x
+            float* ws = smem + (size_t)q.slab * (LA + LB);
+            for (int e = t; e < kn * kFirstIn; e += kProdThreads) {
+                const int i = e % kFirstIn, k = e / kFirstIn;
+                ws[e] = i < q.n_in ? __bfloat162float(q.w1[(long long)k * q.n_in + i]) : 0.f;
+            }
+            float* b1 = ws + kn * kFirstIn;
+            for (int k = t; k < kn; k += kProdThreads) b1[k] = q.b1[k];
+            const int r = t % TM;
+            float x[kFirstIn];
+#pragma unroll
+            for (int i = 0; i < kFirstIn; ++i)
+                x[i] = i < q.n_in && m0 + r < q.M ? q.x[(long long)(m0 + r) * q.n_in + i] : 0.f;
+            __syncthreads();
+#pragma unroll 2
+            for (int k = t / TM; k < kn; k += kProdThreads / TM) {
+                float w0[4], w1[4], v = 0.f;
+                load16(ws + k * kFirstIn, w0);
+                load16(ws + k * kFirstIn + 4, w1);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v = fmaf(x[i], w0[i], v);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v = fmaf(x[4 + i], w1[i], v);
+                As[k * LA + r] = m0 + r < q.M ? tanhf(v + b1[k]) : 0.f;
+            }
+            if (n0 == 0) {
+                __syncthreads();
+                for (int e = t; e < TM * kn; e += kProdThreads)
+                    if (m0 + e / kn < q.M) q.a1[(long long)(m0 + e / kn) * kn + e % kn] = As[(e % kn) * LA + e / kn];
+            }
+        } else {
+            stage<float, TM, LA, AK>(As, q.A, m0, q.M, k0, kn, q.K);
+        }
+        if (k0 == 0)
+#pragma unroll
+            for (int u = 0; u < OUT; ++u) {
+                const int e = t + u * kProdThreads, m = m0 + e / kProdTn, n = n0 + e % kProdTn;
+                pre[u][0] = pre[u][1] = pre[u][2] = 0.f;
+                if (m >= q.M || n >= q.N) continue;
+                const long long o = (long long)m * q.N + n;
+                if constexpr (EP == EP_TANH || EP == EP_LINEAR || EP == EP_MSE) pre[u][0] = q.bias[n];
+                if constexpr (EP == EP_MSE) pre[u][1] = q.aux[o];
+                if constexpr (EP == EP_DTANH) pre[u][0] = q.aux[o];
+                if constexpr (EP == EP_GRAD)
+                    if (q.w.p) { pre[u][0] = q.w.p[o]; pre[u][1] = q.w.m[o]; pre[u][2] = q.w.v[o]; }
+            }
+        __syncthreads();
+        const int per = (kn + G - 1) / G, ka = g * per, kb = min(kn, ka + per);
+#pragma unroll 8
+        for (int k = ka; k < kb; ++k) {
+            float a[4], b[4];
+            load16(As + k * LA + tm, a);
+            load16(Bs + k * LB + tn, b);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            if (want_rows)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) rs[i] += a[i];
+        }
     }
-    red[threadIdx.x] = s;
+    // the groups' sums, added in the groups' order
     __syncthreads();
-    for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-        __syncthreads();
+    float* red = smem;                       // [G][TM][kProdTn]
+    float* rred = smem + G * TM * kProdTn;   // [G][TM]
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float4*>(red + (g * TM + tm + i) * kProdTn + tn) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    if (want_rows && tn == 0)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) rred[g * TM + tm + i] = rs[i];
+    __syncthreads();
+    if (READY == READY_ALL) grid_dependency();
+    double sq = 0.0;
+#pragma unroll
+    for (int u = 0; u < OUT; ++u) {
+        const int e = t + u * kProdThreads, m = m0 + e / kProdTn, n = n0 + e % kProdTn;
+        if (m >= q.M || n >= q.N) continue;
+        float v = red[e];
+#pragma unroll
+        for (int k = 1; k < G; ++k) v += red[k * TM * kProdTn + e];
+        const long long o = (long long)m * q.N + n;
+        if constexpr (EP == EP_TANH) q.C[o] = tanhf(v + pre[u][0]);
+        if constexpr (EP == EP_LINEAR) q.C[o] = v + pre[u][0];
+        if constexpr (EP == EP_MSE) {  // loss = mean (y - t)^2, C = 2 (y - t) / n
+            const float d = v + pre[u][0] - pre[u][1];
+            q.C[o] = 2.f * d * q.scale;
+            sq += (double)d * d;
+        }
+        if constexpr (EP == EP_DTANH) q.C[o] = v * (1.f - pre[u][0] * pre[u][0]);
+        if constexpr (EP == EP_GRAD) {
+            if (q.w.p) adam_update(q.w, o, v, pre[u][0], pre[u][1], pre[u][2]);
+            else q.C[o] = v;
+        }
     }
-    if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
+    if (want_rows && t < TM && m0 + t < q.M) {
+        float v = rred[t];
+        for (int k = 1; k < G; ++k) v += rred[k * TM + t];
+        if (q.b.p) adam_update(q.b, m0 + t, v, q.b.p[m0 + t], q.b.m[m0 + t], q.b.v[m0 + t]);
+        else q.bias_grad[m0 + t] = v;
+    }
+    if constexpr (EP == EP_MSE) {
+        __syncthreads();
+        double* dred = reinterpret_cast<double*>(smem);
+        dred[t] = sq;   // (two FP64 additions per SM and clock: one warp adds, not sixteen)
+        __syncthreads();
+        if (t < 32) {
+            for (int k = t + 32; k < kProdThreads; k += 32) sq += dred[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+            if (t == 0) q.partial[tile] = sq;
+        }
+    }
 }
 
-// Adam (Kingma & Ba 2015) on the FP32 masters, then the BF16 working copy.
-__global__ void k_adam(float* __restrict__ p, __nv_bfloat16* __restrict__ pb, const float* __restrict__ g,
-                       float* __restrict__ m, float* __restrict__ v, long long n, float lr, float b1, float b2,
-                       float eps, float c1, float c2) {
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const float gk = g[k];
-        const float mk = b1 * m[k] + (1.f - b1) * gk;
-        const float vk = b2 * v[k] + (1.f - b2) * gk * gk;
-        m[k] = mk;
-        v[k] = vk;
-        const float upd = lr * (mk / c1) / (sqrtf(vk / c2) + eps);
-        const float pk = p[k] - upd;
-        p[k] = pk;
-        pb[k] = __float2bfloat16_rn(pk);
-    }
+template <int TM, int EP, int READY, bool FIRST>
+__global__ void __launch_bounds__(kProdThreads) k_forward(const Product q) {
+    extern __shared__ __align__(16) float prod_smem[];
+    product_tile<TM, true, true, __nv_bfloat16, EP, READY, FIRST>(q, blockIdx.x, prod_smem);
+}
+// input gradient of one layer (x) and weight gradient of the layer above (w, whose operands are older)
+template <int TX, int TW>
+__global__ void __launch_bounds__(kProdThreads) k_backward(const Product x, const Product w) {
+    extern __shared__ __align__(16) float prod_smem[];
+    if ((int)blockIdx.x < x.tiles) product_tile<TX, true, false, __nv_bfloat16, EP_DTANH, READY_B>(x, blockIdx.x, prod_smem);
+    else product_tile<TW, false, false, float, EP_GRAD, READY_ALL>(w, blockIdx.x - x.tiles, prod_smem);
+}
+// the weight gradients of the lower two layers (b: the first layer's, of the gradient just formed)
+template <int TA, int TB>
+__global__ void __launch_bounds__(kProdThreads) k_weights(const Product a, const Product b) {
+    extern __shared__ __align__(16) float prod_smem[];
+    if ((int)blockIdx.x < b.tiles) product_tile<TB, false, false, float, EP_GRAD, READY_NONE>(b, blockIdx.x, prod_smem);
+    else product_tile<TA, false, false, float, EP_GRAD, READY_ALL>(a, blockIdx.x - b.tiles, prod_smem);
+}
+
+// Tile height and tiles of a product; returns its shared memory.
+int tile_height(int M, int N) {
+    const int n = (N + kProdTn - 1) / kProdTn;
+    return (long long)((M + 31) / 32) * n >= 152 ? 32 : 16;
+}
+size_t plan(Product& q, int tm) {
+    q.tiles_n = (q.N + kProdTn - 1) / kProdTn;
+    q.tiles = (q.M + tm - 1) / tm * q.tiles_n;
+    const int row = (tm + 4 + kProdTn + 4) * (int)sizeof(float);
+    q.slab = std::min(q.K, (int)(kProdSmem / row) / 8 * 8);
+    const int G = kProdThreads / ((tm / 4) * (kProdTn / 4));
+    return std::max((size_t)q.slab * row, (size_t)G * tm * (kProdTn + 1) * sizeof(float));
+}
+// Once per handle, on its device: every product kernel may take its shared memory.
+cudaError_t allow_shared_memory() {
+    cudaError_t e = cudaSuccess;
+    auto allow = [&](auto k) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kProdSmem);
+    };
+    allow(k_forward<16, EP_TANH, READY_NONE, true>);
+    allow(k_forward<32, EP_TANH, READY_NONE, true>);
+    allow(k_forward<16, EP_TANH, READY_NONE, false>);
+    allow(k_forward<32, EP_TANH, READY_NONE, false>);
+    allow(k_forward<16, EP_TANH, READY_B, false>);
+    allow(k_forward<32, EP_TANH, READY_B, false>);
+    allow(k_forward<16, EP_LINEAR, READY_B, false>);
+    allow(k_forward<32, EP_LINEAR, READY_B, false>);
+    allow(k_forward<16, EP_MSE, READY_B, false>);
+    allow(k_forward<32, EP_MSE, READY_B, false>);
+    allow(k_backward<16, 32>);
+    allow(k_weights<16, 16>);
+    return e;
+}
+template <typename K, typename... Args>
+cudaError_t launch(K k, int grid, size_t smem, cudaStream_t s, const Args&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kProdThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
 __global__ void k_to_bf16(const float* __restrict__ p, __nv_bfloat16* __restrict__ pb, long long n) {
@@ -188,7 +427,7 @@ struct lb_mlp {
     __nv_bfloat16* pb = nullptr;                                    // BF16 working weights
     float *a1 = nullptr, *a2 = nullptr, *y = nullptr;              // activations [max_batch][..]
     float *d1 = nullptr, *d2 = nullptr, *dy = nullptr;             // their gradients
-    double* partial = nullptr;                                      // loss partial sums
+    double* partial = nullptr;                                      // loss partial sums, one per tile
     long long t = 0;                                                // Adam step
 };
 
@@ -203,35 +442,119 @@ void mlp_free(lb_mlp* m) {
     delete m;
 }
 
-lb_status forward(lb_mlp* m, const float* x, int B) {
-    const dim3 blk(TB, TB);
-    k_linear_fwd<<<dim3((m->H + TB - 1) / TB, (B + TB - 1) / TB), blk, 0, m->stream>>>(x, m->pb + m->o_w1, m->p + m->o_b1, m->a1, B, m->n_in, m->H, 1);
-    k_linear_fwd<<<dim3((m->H + TB - 1) / TB, (B + TB - 1) / TB), blk, 0, m->stream>>>(m->a1, m->pb + m->o_w2, m->p + m->o_b2, m->a2, B, m->H, m->H, 1);
-    k_linear_fwd<<<dim3((m->n_out + TB - 1) / TB, (B + TB - 1) / TB), blk, 0, m->stream>>>(m->a2, m->pb + m->o_w3, m->p + m->o_b3, m->y, B, m->H, m->n_out, 0);
-    MLP_CK(cudaGetLastError());
+template <int EP, int READY, bool FIRST = false>
+cudaError_t run_forward(lb_mlp* m, Product q) {
+    const int tm = tile_height(q.M, q.N);
+    const size_t smem = plan(q, tm) + (FIRST ? sizeof(float) * (kFirstIn + 1) * q.K : 0);
+    return tm == 32 ? launch(k_forward<32, EP, READY, FIRST>, q.tiles, smem, m->stream, q)
+                    : launch(k_forward<16, EP, READY, FIRST>, q.tiles, smem, m->stream, q);
+}
+
+Product forward_product(lb_mlp* m, const float* in, long long o_w, long long o_b, float* out, int B, int I, int O) {
+    Product q{};
+    q.A = in;
+    q.B = m->pb + o_w;
+    q.C = out;
+    q.M = B;
+    q.N = O;
+    q.K = I;
+    q.bias = m->p + o_b;
+    return q;
+}
+
+// The two hidden layers: in one launch when the first has few inputs (every tile of the second evaluates its
+// rows of the first again) and the second's depth fits one slab.
+lb_status forward_hidden(lb_mlp* m, const float* x, int B) {
+    Product q = forward_product(m, m->a1, m->o_w2, m->o_b2, m->a2, B, m->H, m->H);
+    if (m->n_in <= kFirstIn && plan(q, 32) + sizeof(float) * (kFirstIn + 1) * m->H <= kProdSmem && q.slab == m->H) {
+        q.x = x;
+        q.w1 = m->pb + m->o_w1;
+        q.b1 = m->p + m->o_b1;
+        q.a1 = m->a1;
+        q.n_in = m->n_in;
+        MLP_CK((run_forward<EP_TANH, READY_NONE, true>(m, q)));
+    } else {
+        MLP_CK((run_forward<EP_TANH, READY_NONE>(m, forward_product(m, x, m->o_w1, m->o_b1, m->a1, B, m->n_in, m->H))));
+        MLP_CK((run_forward<EP_TANH, READY_B>(m, q)));
+    }
     return LB_OK;
 }
 
-// Forward, loss and the full gradient into m->g; the loss (host) if requested.
-lb_status backward(lb_mlp* m, const float* x, const float* target, int B, double* loss) {
-    lb_status st = forward(m, x, B);
+lb_status forward(lb_mlp* m, const float* x, int B, float* y) {
+    lb_status st = forward_hidden(m, x, B);
+    if (st != LB_OK) return st;
+    MLP_CK((run_forward<EP_LINEAR, READY_B>(m, forward_product(m, m->a2, m->o_w3, m->o_b3, y, B, m->H, m->n_out))));
+    return LB_OK;
+}
+
+// dX[b][i] = sum_o dY[b][o] W[o][i] times tanh' of the input's activations
+Product input_gradient(lb_mlp* m, const float* dy, long long o_w, const float* act, float* dx, int B, int I, int O) {
+    Product q{};
+    q.A = dy;
+    q.B = m->pb + o_w;
+    q.C = dx;
+    q.M = B;
+    q.N = I;
+    q.K = O;
+    q.aux = act;
+    return q;
+}
+// dW[o][i] = sum_b dY[b][o] X[b][i] and db[o] = sum_b dY[b][o]: into m->g, or Adam's update of the layer
+Product weight_gradient(lb_mlp* m, const float* dy, const float* x, long long o_w, long long o_b, int B, int I, int O,
+                        const Adam* adam) {
+    Product q{};
+    q.A = dy;
+    q.B = x;
+    q.M = O;
+    q.N = I;
+    q.K = B;
+    if (adam) {
+        auto at = [&](long long o) {
+            Adam a = *adam;
+            a.p = m->p + o;
+            a.m = m->m + o;
+            a.v = m->v + o;
+            a.pb = m->pb + o;
+            return a;
+        };
+        q.w = at(o_w);
+        q.b = at(o_b);
+    } else {
+        q.C = m->g + o_w;
+        q.bias_grad = m->g + o_b;
+    }
+    return q;
+}
+
+// Forward, loss and the full gradient: into m->g, or (adam) straight into the update of the parameters.  A layer's
+// weights change in a launch after the one whose input gradient reads them.  The loss (host) if
+// requested.
+lb_status backward(lb_mlp* m, const float* x, const float* target, int B, double* loss, const Adam* adam) {
+    lb_status st = forward_hidden(m, x, B);
     if (st != LB_OK) return st;
     const long long n = (long long)B * m->n_out;
-    const int nb = 64;
-    k_mse<<<nb, 256, 0, m->stream>>>(m->y, target, m->dy, m->partial, n, 1.f / (float)n);
-    const dim3 blk(TB, TB);
-    // layer 3
-    k_linear_bwd_w<<<dim3((m->H + TB - 1) / TB, (m->n_out + TB - 1) / TB), blk, 0, m->stream>>>(m->dy, m->a2, m->g + m->o_w3, m->g + m->o_b3, B, m->H, m->n_out);
-    k_linear_bwd_x<<<dim3((m->H + TB - 1) / TB, (B + TB - 1) / TB), blk, 0, m->stream>>>(m->dy, m->pb + m->o_w3, m->a2, m->d2, B, m->H, m->n_out);
-    // layer 2
-    k_linear_bwd_w<<<dim3((m->H + TB - 1) / TB, (m->H + TB - 1) / TB), blk, 0, m->stream>>>(m->d2, m->a1, m->g + m->o_w2, m->g + m->o_b2, B, m->H, m->H);
-    k_linear_bwd_x<<<dim3((m->H + TB - 1) / TB, (B + TB - 1) / TB), blk, 0, m->stream>>>(m->d2, m->pb + m->o_w2, m->a1, m->d1, B, m->H, m->H);
-    // layer 1
-    k_linear_bwd_w<<<dim3((m->n_in + TB - 1) / TB, (m->H + TB - 1) / TB), blk, 0, m->stream>>>(m->d1, x, m->g + m->o_w1, m->g + m->o_b1, B, m->n_in, m->H);
-    MLP_CK(cudaGetLastError());
+    Product y = forward_product(m, m->a2, m->o_w3, m->o_b3, m->dy, B, m->H, m->n_out);
+    y.aux = target;
+    y.partial = m->partial;
+    y.scale = 1.f / (float)n;
+    const int ty = tile_height(y.M, y.N);
+    plan(y, ty);
+    MLP_CK((run_forward<EP_MSE, READY_B>(m, y)));
+    Product none{};
+    Product x3 = input_gradient(m, m->dy, m->o_w3, m->a2, m->d2, B, m->H, m->n_out);
+    Product x2 = input_gradient(m, m->d2, m->o_w2, m->a1, m->d1, B, m->H, m->H);
+    Product w3 = weight_gradient(m, m->dy, m->a2, m->o_w3, m->o_b3, B, m->H, m->n_out, adam);
+    Product w2 = weight_gradient(m, m->d2, m->a1, m->o_w2, m->o_b2, B, m->H, m->H, adam);
+    Product w1 = weight_gradient(m, m->d1, x, m->o_w1, m->o_b1, B, m->n_in, m->H, adam);
+    size_t smem = plan(x3, 16);
+    MLP_CK(launch(k_backward<16, 32>, x3.tiles, smem, m->stream, x3, none));
+    smem = std::max(plan(x2, 16), plan(w3, 32));
+    MLP_CK(launch(k_backward<16, 32>, x2.tiles + w3.tiles, smem, m->stream, x2, w3));
+    smem = std::max(plan(w2, 16), plan(w1, 16));
+    MLP_CK(launch(k_weights<16, 16>, w2.tiles + w1.tiles, smem, m->stream, w2, w1));
     if (loss) {
-        std::vector<double> part(nb);
-        MLP_CK(cudaMemcpyAsync(part.data(), m->partial, sizeof(double) * nb, cudaMemcpyDeviceToHost, m->stream));
+        std::vector<double> part(y.tiles);
+        MLP_CK(cudaMemcpyAsync(part.data(), m->partial, sizeof(double) * y.tiles, cudaMemcpyDeviceToHost, m->stream));
         MLP_CK(cudaStreamSynchronize(m->stream));
         double s = 0.0;
         for (double q : part) s += q;
@@ -263,8 +586,9 @@ lb_status lb_mlp_create(int n_in, int width, int n_out, int max_batch, uint64_t 
     al((void**)&m->pb, P * 2);
     al((void**)&m->a1, B * width * 4); al((void**)&m->a2, B * width * 4); al((void**)&m->y, B * n_out * 4);
     al((void**)&m->d1, B * width * 4); al((void**)&m->d2, B * width * 4); al((void**)&m->dy, B * n_out * 4);
-    al((void**)&m->partial, 64 * sizeof(double));
+    al((void**)&m->partial, (size_t)((B + 15) / 16) * ((n_out + kProdTn - 1) / kProdTn) * sizeof(double));
     if (e != cudaSuccess) { mlp_free(m); return mfail(LB_ENOMEM, "lb_mlp_create: cudaMalloc"); }
+    if (allow_shared_memory() != cudaSuccess) { mlp_free(m); return mfail(LB_ECUDA, "lb_mlp_create: kernel attributes"); }
     e = cudaMemsetAsync(m->p, 0, P * 4, m->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->m, 0, P * 4, m->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->v, 0, P * 4, m->stream);
@@ -286,15 +610,20 @@ long long lb_mlp_num_params(const lb_mlp* m) { return m ? m->n_par : 0; }
 
 lb_status lb_mlp_forward(lb_mlp* m, const float* x, int batch, float* y) {
     if (!m || !x || !y || batch < 1 || batch > m->max_batch) return mfail(LB_EINVAL, "lb_mlp_forward: bad argument");
-    lb_status st = forward(m, x, batch);
-    if (st != LB_OK) return st;
+    // device memory is written by the last layer itself; anything else gets a copy
+    cudaPointerAttributes at{};
+    const bool direct = cudaPointerGetAttributes(&at, y) == cudaSuccess &&
+                        (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
+    (void)cudaGetLastError();
+    lb_status st = forward(m, x, batch, direct ? y : m->y);
+    if (st != LB_OK || direct) return st;
     MLP_CK(cudaMemcpyAsync(y, m->y, sizeof(float) * batch * m->n_out, cudaMemcpyDeviceToDevice, m->stream));
     return LB_OK;
 }
 
 lb_status lb_mlp_gradients(lb_mlp* m, const float* x, const float* target, int batch, float* grads, double* loss) {
     if (!m || !x || !target || batch < 1 || batch > m->max_batch) return mfail(LB_EINVAL, "lb_mlp_gradients: bad argument");
-    lb_status st = backward(m, x, target, batch, loss);
+    lb_status st = backward(m, x, target, batch, loss, nullptr);
     if (st != LB_OK) return st;
     if (grads) MLP_CK(cudaMemcpyAsync(grads, m->g, sizeof(float) * m->n_par, cudaMemcpyDeviceToDevice, m->stream));
     return LB_OK;
@@ -303,14 +632,17 @@ lb_status lb_mlp_gradients(lb_mlp* m, const float* x, const float* target, int b
 lb_status lb_mlp_train_step(lb_mlp* m, const float* x, const float* target, int batch, float lr, double* loss) {
     if (!m || !x || !target || batch < 1 || batch > m->max_batch || !(lr > 0.f))
         return mfail(LB_EINVAL, "lb_mlp_train_step: bad argument");
-    lb_status st = backward(m, x, target, batch, loss);
-    if (st != LB_OK) return st;
-    m->t += 1;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.f - powf(b1, (float)m->t), c2 = 1.f - powf(b2, (float)m->t);
-    k_adam<<<nblocks(m->n_par), 256, 0, m->stream>>>(m->p, m->pb, m->g, m->m, m->v, m->n_par, lr, b1, b2, 1e-8f, c1, c2);
-    MLP_CK(cudaGetLastError());
-    return LB_OK;
+    Adam adam{};
+    const float t = (float)(m->t + 1);
+    adam.lr = lr;
+    adam.b1 = 0.9f;
+    adam.b2 = 0.999f;
+    adam.eps = 1e-8f;
+    adam.c1 = 1.f - powf(adam.b1, t);
+    adam.c2 = 1.f - powf(adam.b2, t);
+    lb_status st = backward(m, x, target, batch, loss, &adam);
+    if (st == LB_OK) m->t += 1;
+    return st;
 }
 
 lb_status lb_mlp_get_params(lb_mlp* m, float* host) {
