@@ -126,6 +126,12 @@ extern template cudaError_t march_occupancy<float, float, 0, 2>(int*);
 extern template cudaError_t march_occupancy<float, float, 1, 2>(int*);
 extern template cudaError_t march_occupancy<__nv_bfloat16, float, 0, 2>(int*);
 extern template cudaError_t march_occupancy<__nv_bfloat16, float, 1, 2>(int*);
+#define LB_MARCH_FIELDS_EXTERN(T, SMODE, BND, SCHEME)                                                                       \
+    extern template cudaError_t launch_step_march<T, float, SMODE, BND, SCHEME, true>(const CUtensorMap&,                       \
+                                                                                      const StepArgs<T, float>&, const MarchCtl&, \
+                                                                                      int, cudaStream_t);
+LB_MARCH_FIELDS_ALL(LB_MARCH_FIELDS_EXTERN)
+#undef LB_MARCH_FIELDS_EXTERN
 }  // namespace lbk
 
 using namespace lbk;
@@ -306,12 +312,6 @@ __global__ void k_reduce_residual(const double* partials, const int* item_begin,
                         with_residual, threadIdx.x);
 }
 
-template <typename A, typename B>
-__global__ void k_convert(const A* src, B* dst, long long n) {
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
-        dst[k] = (B)src[k];
-}
-
 int grid_for(long long n) {
     long long b = (n + 255) / 256;
     return (int)(b < 1 ? 1 : (b > 4096 ? 4096 : b));
@@ -355,6 +355,8 @@ struct NvtxRange {
     NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
+constexpr unsigned long long kDefaultWaitNs = 2000000000ull;
+
 struct lb_handle {
     int dev = 0;
     cudaStream_t stream = nullptr;
@@ -384,8 +386,8 @@ struct lb_handle {
     long long *base_d = nullptr, *P_d = nullptr, *node_off_d = nullptr;
     int* ny_d = nullptr;
     double* gx_d = nullptr;
-    void* fields = nullptr;    // staging for lb_get_fields, 7 values per node in C type
-    void* fconv = nullptr;     // staging for converted fields, 7 values per node
+    void* fields = nullptr;    // staging of fields, 7 values per node (allocated when first needed)
+    size_t fields_bytes = 0;
     void* hstage = nullptr;    // device staging for FP64 host transfers
     size_t hstage_bytes = 0;
     // launch plan
@@ -411,7 +413,7 @@ struct lb_handle {
     bool status_pending = false;
     bool any_unstable = false;
     bool any_timeout = false;
-    unsigned long long wait_ns = 2000000000ull;  // limit of the row-march kernel's mbarrier waits
+    unsigned long long wait_ns = kDefaultWaitNs;  // limit of the row-march kernel's mbarrier waits
     // row-march kernel (wide single channels, FP32 / BF16 storage)
     bool march = false;
     CUtensorMap mapA, mapB;    // tensor maps of the two population buffers ...
@@ -822,7 +824,7 @@ void release(lb_handle* h) {
     free_dev(h->popA); free_dev(h->popB); free_dev(h->drho); free_dev(h->sig3); free_dev(h->sig4); free_dev(h->snn); free_dev(h->phi);
     free_dev(h->uprev); free_dev(h->chan); free_dev(h->items_d); free_dev(h->item_begin_d);
     free_dev(h->partials); free_dev(h->mon_d); free_dev(h->status_d); free_dev(h->base_d); free_dev(h->P_d);
-    free_dev(h->node_off_d); free_dev(h->ny_d); free_dev(h->gx_d); free_dev(h->fields); free_dev(h->fconv);
+    free_dev(h->node_off_d); free_dev(h->ny_d); free_dev(h->gx_d); free_dev(h->fields);
     free_dev(h->hstage);
     free_dev(h->ws_prm); free_dev(h->ws_row_off); free_dev(h->ws_rows); free_dev(h->ws_grid); free_dev(h->ws_scale);
     free_dev(h->march_items_d);
@@ -962,44 +964,34 @@ void march_monitor(lb_handle* h, int flags, MarchCtl& ctl) {
     ctl.with_residual = (flags & F_RESID) ? 1 : 0;
 }
 
-// The row-march kernel takes plain steps (no fields output, no residual reduction).
-template <typename T, typename C>
-cudaError_t launch_march(lb_handle*, const StepArgs<T, C>&) { return cudaErrorNotSupported; }
-template <>
-cudaError_t launch_march<float, float>(lb_handle* h, const StepArgs<float, float>& a) {
-    MarchCtl ctl{h->march_items_d, h->n_march_items, h->status_d, h->P[0], h->base[0], h->wait_ns};
+// The row-march kernel: a step, or (F_FIELDS) the fields of the stored state.
+template <typename T, bool FIELDS>
+cudaError_t launch_march_as(lb_handle* h, const StepArgs<T, float>& a) {
+    // (the fields pass has its own wait limit: lb_set_wait_limit speaks of steps)
+    MarchCtl ctl{h->march_items_d, h->n_march_items, h->status_d, h->P[0], h->base[0], FIELDS ? kDefaultWaitNs : h->wait_ns};
     march_monitor(h, a.flags, ctl);
     const CUtensorMap& m = ((const void*)a.pin == h->mapA_buf) ? h->mapA : h->mapB;
-    if (h->scheme == 1) return launch_step_march<float, float, 0, 0, 1>(m, a, ctl, h->march_grid, h->stream);
+    const int grid = h->march_grid;
+    const cudaStream_t s = h->stream;
+    if (h->scheme == 1) return launch_step_march<T, float, 0, 0, 1, FIELDS>(m, a, ctl, grid, s);
     if (h->scheme == 3)
-        return h->smode ? launch_step_march<float, float, 1, 0, 3>(m, a, ctl, h->march_grid, h->stream)
-                        : launch_step_march<float, float, 0, 0, 3>(m, a, ctl, h->march_grid, h->stream);
+        return h->smode ? launch_step_march<T, float, 1, 0, 3, FIELDS>(m, a, ctl, grid, s)
+                        : launch_step_march<T, float, 0, 0, 3, FIELDS>(m, a, ctl, grid, s);
     if (h->gpbc)
-        return h->smode ? launch_step_march<float, float, 1, 1>(m, a, ctl, h->march_grid, h->stream)
-                        : launch_step_march<float, float, 0, 1>(m, a, ctl, h->march_grid, h->stream);
+        return h->smode ? launch_step_march<T, float, 1, 1, 0, FIELDS>(m, a, ctl, grid, s)
+                        : launch_step_march<T, float, 0, 1, 0, FIELDS>(m, a, ctl, grid, s);
     if (h->moving)
-        return h->smode ? launch_step_march<float, float, 1, 2>(m, a, ctl, h->march_grid, h->stream)
-                        : launch_step_march<float, float, 0, 2>(m, a, ctl, h->march_grid, h->stream);
-    return h->smode ? launch_step_march<float, float, 1>(m, a, ctl, h->march_grid, h->stream)
-                    : launch_step_march<float, float, 0>(m, a, ctl, h->march_grid, h->stream);
+        return h->smode ? launch_step_march<T, float, 1, 2, 0, FIELDS>(m, a, ctl, grid, s)
+                        : launch_step_march<T, float, 0, 2, 0, FIELDS>(m, a, ctl, grid, s);
+    return h->smode ? launch_step_march<T, float, 1, 0, 0, FIELDS>(m, a, ctl, grid, s)
+                    : launch_step_march<T, float, 0, 0, 0, FIELDS>(m, a, ctl, grid, s);
 }
-template <>
-cudaError_t launch_march<__nv_bfloat16, float>(lb_handle* h, const StepArgs<__nv_bfloat16, float>& a) {
-    MarchCtl ctl{h->march_items_d, h->n_march_items, h->status_d, h->P[0], h->base[0], h->wait_ns};
-    march_monitor(h, a.flags, ctl);
-    const CUtensorMap& m = ((const void*)a.pin == h->mapA_buf) ? h->mapA : h->mapB;
-    if (h->scheme == 1) return launch_step_march<__nv_bfloat16, float, 0, 0, 1>(m, a, ctl, h->march_grid, h->stream);
-    if (h->scheme == 3)
-        return h->smode ? launch_step_march<__nv_bfloat16, float, 1, 0, 3>(m, a, ctl, h->march_grid, h->stream)
-                        : launch_step_march<__nv_bfloat16, float, 0, 0, 3>(m, a, ctl, h->march_grid, h->stream);
-    if (h->gpbc)
-        return h->smode ? launch_step_march<__nv_bfloat16, float, 1, 1>(m, a, ctl, h->march_grid, h->stream)
-                        : launch_step_march<__nv_bfloat16, float, 0, 1>(m, a, ctl, h->march_grid, h->stream);
-    if (h->moving)
-        return h->smode ? launch_step_march<__nv_bfloat16, float, 1, 2>(m, a, ctl, h->march_grid, h->stream)
-                        : launch_step_march<__nv_bfloat16, float, 0, 2>(m, a, ctl, h->march_grid, h->stream);
-    return h->smode ? launch_step_march<__nv_bfloat16, float, 1>(m, a, ctl, h->march_grid, h->stream)
-                    : launch_step_march<__nv_bfloat16, float, 0>(m, a, ctl, h->march_grid, h->stream);
+template <typename T, typename C>
+cudaError_t launch_march(lb_handle* h, const StepArgs<T, C>& a) {
+    if constexpr (std::is_same<C, float>::value && (std::is_same<T, float>::value || std::is_same<T, __nv_bfloat16>::value))
+        return (a.flags & F_FIELDS) ? launch_march_as<T, true>(h, a) : launch_march_as<T, false>(h, a);
+    else
+        return cudaErrorNotSupported;
 }
 
 constexpr int kGraphSteps = 32;  // steps per captured graph (even)
@@ -1098,16 +1090,41 @@ lb_status run_steps(lb_handle* h, long n) {
     return LB_OK;
 }
 
-template <typename T, typename C>
-lb_status fields_pass(lb_handle* h, C* fu, C* fs, C* fr) {
-    StepArgs<T, C> a = base_args<T, C>(h);
-    a.flags = F_FIELDS;
-    a.fu = fu;
-    a.fsig = fs;
-    a.frho = fr;
-    LB_CK((gpbc_columns<T, C>(h)));
-    LB_CK((launch<T, C>(h, a)));
+// The fields of the current state into device buffers (any may be null; 16-byte aligned) of type double (out64)
+// or float.
+lb_status fields_pass(lb_handle* h, void* fu, void* fs, void* fr, bool out64) {
+    return with_types(h->prec, [&](auto tt, auto tc) -> lb_status {
+        LB_TYPES(tt, tc);
+        StepArgs<T, C> a = base_args<T, C>(h);
+        a.flags = F_FIELDS | (out64 ? F_OUT64 : 0);
+        a.fu = fu;
+        a.fsig = fs;
+        a.frho = fr;
+        LB_CK((gpbc_columns<T, C>(h)));
+        if (h->march) LB_CK((launch_march<T, C>(h, a)));
+        else LB_CK((launch<T, C>(h, a)));
+        return LB_OK;
+    });
+}
+
+// The handle's staging buffer of 7 values per node (u, sigma, rho one after the other).
+lb_status ensure_fields(lb_handle* h, size_t value_size) {
+    const size_t bytes = 7 * (size_t)h->nodes * value_size + 64;
+    if (h->fields_bytes >= bytes) return LB_OK;
+    free_dev(h->fields);
+    h->fields_bytes = 0;
+    LB_CK(cudaMalloc(&h->fields, bytes));
+    h->fields_bytes = bytes;
     return LB_OK;
+}
+// its parts, each on a 16-byte boundary
+struct FieldParts {
+    char *u, *sigma, *rho;
+};
+FieldParts field_parts(lb_handle* h, size_t value_size) {
+    char* b = (char*)h->fields;
+    const size_t n = (size_t)h->nodes * value_size;
+    return FieldParts{b, b + (2 * n + 15) / 16 * 16, b + (2 * n + 15) / 16 * 16 + 4 * n};
 }
 
 lb_status poll_status(lb_handle* h, bool wait) {
@@ -1793,28 +1810,27 @@ lb_status lb_get_fields(lb_handle* h, void* u, void* sigma, void* rho, int out_d
     if (!h || (out_dtype != 0 && out_dtype != 1)) return fail(LB_EINVAL, "lb_get_fields: bad handle or dtype%s");
     if (!u && !sigma && !rho) return LB_OK;
     const long long N = h->nodes;
-    if (!h->fields) LB_CK(cudaMalloc(&h->fields, 7 * N * h->csize));
-    char* base = (char*)h->fields;
-    void* fu = base;
-    void* fs = base + 2 * N * h->csize;
-    void* fr = base + 6 * N * h->csize;
-    lb_status st;
-    st = with_types(h->prec, [&](auto tt, auto tc) { LB_TYPES(tt, tc); return fields_pass<T, C>(h, (C*)fu, (C*)fs, (C*)fr); });
-    if (st != LB_OK) return st;
     const size_t osize = out_dtype == 0 ? 8 : 4;
-    const void* src = h->fields;
-    if (osize != h->csize) {
-        if (!h->fconv) LB_CK(cudaMalloc(&h->fconv, 7 * N * 8));
-        if (h->csize == 8) k_convert<double, float><<<grid_for(7 * N), 256, 0, h->stream>>>((const double*)h->fields, (float*)h->fconv, 7 * N);
-        else k_convert<float, double><<<grid_for(7 * N), 256, 0, h->stream>>>((const float*)h->fields, (double*)h->fconv, 7 * N);
-        LB_CK(cudaGetLastError());
-        src = h->fconv;
-    }
+    // buffers in device memory on 16-byte boundaries are written by the fields pass itself; anything else
+    // (host memory, odd addresses) goes through the staging buffer
+    auto direct = [h](const void* p) {
+        if (!p) return true;
+        cudaPointerAttributes at{};
+        const bool ok = reinterpret_cast<uintptr_t>(p) % 16 == 0 && cudaPointerGetAttributes(&at, p) == cudaSuccess &&
+                        ((at.type == cudaMemoryTypeDevice && at.device == h->dev) || at.type == cudaMemoryTypeManaged);
+        (void)cudaGetLastError();
+        return ok;
+    };
+    if (on_device && direct(u) && direct(sigma) && direct(rho)) return fields_pass(h, u, sigma, rho, out_dtype == 0);
+    lb_status st = ensure_fields(h, osize);
+    if (st != LB_OK) return st;
+    const FieldParts f = field_parts(h, osize);
+    st = fields_pass(h, u ? f.u : nullptr, sigma ? f.sigma : nullptr, rho ? f.rho : nullptr, out_dtype == 0);
+    if (st != LB_OK) return st;
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    const char* s = (const char*)src;
-    if (u) LB_CK(cudaMemcpyAsync(u, s, 2 * N * osize, kind, h->stream));
-    if (sigma) LB_CK(cudaMemcpyAsync(sigma, s + 2 * N * osize, 4 * N * osize, kind, h->stream));
-    if (rho) LB_CK(cudaMemcpyAsync(rho, s + 6 * N * osize, N * osize, kind, h->stream));
+    if (u) LB_CK(cudaMemcpyAsync(u, f.u, 2 * N * osize, kind, h->stream));
+    if (sigma) LB_CK(cudaMemcpyAsync(sigma, f.sigma, 4 * N * osize, kind, h->stream));
+    if (rho) LB_CK(cudaMemcpyAsync(rho, f.rho, N * osize, kind, h->stream));
     if (!on_device) LB_CK(cudaStreamSynchronize(h->stream));
     return LB_OK;
 }
@@ -1967,13 +1983,11 @@ lb_status lb_warmstart_targets(lb_handle* h, float* targets) {
     if (!h || !targets) return fail(LB_EINVAL, "lb_warmstart_targets: null argument%s");
     lb_status st = ws_closed_form(h);
     if (st != LB_OK) return st;
-    const long long N = h->nodes;
-    if (!h->fields) LB_CK(cudaMalloc(&h->fields, 7 * N * h->csize));
-    char* base = (char*)h->fields;
-    void* fu = base;
-    void* fs = base + 2 * N * h->csize;
-    void* fr = base + 6 * N * h->csize;
-    st = with_types(h->prec, [&](auto tt, auto tc) { LB_TYPES(tt, tc); return fields_pass<T, C>(h, (C*)fu, (C*)fs, (C*)fr); });
+    st = ensure_fields(h, h->csize);
+    if (st != LB_OK) return st;
+    const FieldParts f = field_parts(h, h->csize);
+    void *fu = f.u, *fs = f.sigma;
+    st = fields_pass(h, fu, fs, nullptr, h->csize == 8);
     if (st != LB_OK) return st;
     if (h->csize == 8)
         LB_CK(launch_ws_targets<double>(h->n_ch, (const double*)fu, (const double*)fs, (const double*)h->ws_grid,

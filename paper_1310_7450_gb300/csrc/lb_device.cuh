@@ -150,6 +150,7 @@ enum : int {
     F_MON = 32,         // accumulate flux and max |u| only (block partials; no u_prev read)
     F_SNN = 64,         // scheme 2, first pass: write Sigma^nN (xx, xy, yy) only (no state writes)
     F_DIV = 128,        // scheme 2, second pass: add div Sigma^nN of the written planes as a force
+    F_OUT64 = 256,      // F_FIELDS: the outputs are double, else float (whatever the arithmetic type)
 };
 
 template <typename T, typename C>
@@ -160,9 +161,9 @@ struct StepArgs {
     C* __restrict__ sig3;          // carried stress (xx, xy, yy) [3 planes], stress mode 1
     C* __restrict__ sig4;          // stress output (xx, yy, zz, xy) [4 planes]
     C* __restrict__ uprev;         // saved velocity [2 planes]
-    C* __restrict__ fu;            // fields-only outputs, compact node order: u [node][2]
-    C* __restrict__ fsig;          //   sigma [node][4]
-    C* __restrict__ frho;          //   rho [node]
+    void* __restrict__ fu;         // fields-only outputs, compact node order: u [node][2]
+    void* __restrict__ fsig;       //   sigma [node][4] as xx, yy, zz, xy
+    void* __restrict__ frho;       //   rho [node]; any may be null; 16-byte aligned; float or double (F_OUT64)
     double* __restrict__ partials; // residual partials [item][4]
     C* __restrict__ snn;           // scheme 2: Sigma^nN (xx, xy, yy) of this step [3 planes]
     double* __restrict__ phi;      // scheme 3: fluidity 1/tau_M of the last step [plane] (0: unset),
@@ -179,6 +180,25 @@ struct StepArgs {
                                    // the column means of rho - 1 [channel][col]
     int gny;                       // rows of all channels (the row stride of gcol)
 };
+
+// The fields of one node, in the caller's type and layout: one vector store per field, so that no pass has to
+// convert or rearrange them afterwards.
+template <typename C, typename T>
+__device__ __forceinline__ void store_fields(const StepArgs<T, C>& a, long long node, C ux, C uy, C sxx, C syy, C sxy, C rho) {
+    if (a.flags & F_OUT64) {
+        if (a.fu) static_cast<double2*>(a.fu)[node] = make_double2((double)ux, (double)uy);
+        if (a.fsig) {
+            double2* q = static_cast<double2*>(a.fsig) + 2 * node;
+            q[0] = make_double2((double)sxx, (double)syy);
+            q[1] = make_double2(0.0, (double)sxy);
+        }
+        if (a.frho) static_cast<double*>(a.frho)[node] = (double)rho;
+    } else {
+        if (a.fu) static_cast<float2*>(a.fu)[node] = make_float2((float)ux, (float)uy);
+        if (a.fsig) static_cast<float4*>(a.fsig)[node] = make_float4((float)sxx, (float)syy, 0.f, (float)sxy);
+        if (a.frho) static_cast<float*>(a.frho)[node] = (float)rho;
+    }
+}
 
 // ---- per-node arithmetic -------------------------------------------------------------------
 

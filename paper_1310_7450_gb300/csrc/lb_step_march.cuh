@@ -163,7 +163,9 @@ __device__ __forceinline__ P2 slot_pair_odd(const T* p) {
 // SCHEME 3: the relaxation-time extensions (periodic x, bounce-back walls, either stress mode): the
 // node's FP64 fluidity is loaded one row ahead of its use and stored with the step, as in the tile
 // kernel's scheme-3 variant.
-template <typename T, typename C, int SMODE, int CW, int K, int BND = 0, int SCHEME = 0>
+// FIELDS: the fields of the stored state (F_FIELDS) instead of a step: everything up to the stress, then
+// u, sigma and rho in node order.
+template <typename T, typename C, int SMODE, int CW, int K, int BND = 0, int SCHEME = 0, bool FIELDS = false>
 __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant__ CUtensorMap tmap,
                                                                                   const StepArgs<T, C> a,
                                                                                   const MarchCtl ctl) {
@@ -605,16 +607,23 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                         const C t1 = relaxation_time_ext<C>(P, 0.5f * hi(Kx), 0.5f * hi(By), 0.5f * hi(Kc), 0.5f * hi(Ey),
                                                             hi(dRc), hi(drho_prev), phi_cur.y, &phi_new.y);
                         tau_M = p2(t0, t1);
-                        if (fluid) *reinterpret_cast<double2*>(a.phi + ibase + o) = phi_new;
+                        if (!FIELDS && fluid) *reinterpret_cast<double2*>(a.phi + ibase + o) = phi_new;
                     }
                     s = constitutive<SMODE, BND == 1, SCHEME == 3>(q, Kx, By, Kc, Ey, dRc, jxc, jyc, drho_prev, so_xx, so_xy,
                                                                    so_yy, tau_M);
                 }
                 const P2 rho_h = sub(add(p2(1.f), s.dReq), s.drho);
+                if constexpr (FIELDS) {
+                    const P2 ih = rcp(rho_h), urx = mul(jxc, ih), ury = mul(jyc, ih);
+                    const long long node = (long long)y * nx + x0 + col0;
+                    store_fields<C>(a, node, lo(urx), lo(ury), lo(s.sxx), lo(s.syy), lo(s.sxy), lo(rho_h));
+                    store_fields<C>(a, node + 1, hi(urx), hi(ury), hi(s.sxx), hi(s.syy), hi(s.sxy), hi(rho_h));
+                }
                 {  // velocity_ok of both nodes: |u| <= guard without a division (false for NaN)
                     const P2 j2 = fma(jyc, jyc, mul(jxc, jxc)), g2 = mul(mul(p2(a.guard * a.guard), rho_h), rho_h);
                     vbad |= !(lo(j2) <= lo(g2)) | !(hi(j2) <= hi(g2));
                 }
+                if constexpr (!FIELDS) {
                 P2 D[9];
                 collide<SCHEME != 0>(q, s, dcur, D, om, nom, k2);
                 T* po = a.pout + 8 * ctl.base;
@@ -664,6 +673,7 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                         store_pair(up_ + PL, ury);
                     }
                 }
+                }  // not the fields pass
             }
             us_x = u0_x;
             us_y = u0_y;
@@ -775,11 +785,11 @@ constexpr int kMarchW = 128;  // columns per CTA (one strip)
 //    with pressure-driven ends one row at a time is faster (2048 x 1000: 53.8 against 56.4).
 constexpr int kMarchK = 7;  // shared-memory row slots
 
-template <typename T, typename C, int SMODE, int BND = 0, int SCHEME = 0>
+template <typename T, typename C, int SMODE, int BND = 0, int SCHEME = 0, bool FIELDS = false>
 cudaError_t launch_step_march(const CUtensorMap& map, const StepArgs<T, C>& a, const MarchCtl& ctl, int grid,
                               cudaStream_t s) {
     constexpr int K = kMarchK;
-    auto k = k_step_march<T, C, SMODE, kMarchW, K, BND, SCHEME>;
+    auto k = k_step_march<T, C, SMODE, kMarchW, K, BND, SCHEME, FIELDS>;
     const size_t smem = march_smem_bytes<T, C, kMarchW, K>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
@@ -799,3 +809,10 @@ cudaError_t march_occupancy(int* blocks_per_sm) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, kMarchW / 2, smem);
 }
 }  // namespace lbk
+// Every variant (storage type, stress mode, boundary, scheme) of the kernel.
+#define LB_MARCH_FIELDS_ALL(X)                                                                      \
+    X(float, 0, 0, 0) X(float, 1, 0, 0) X(float, 0, 1, 0) X(float, 1, 1, 0) X(float, 0, 2, 0) X(float, 1, 2, 0) \
+    X(float, 0, 0, 1) X(float, 0, 0, 3) X(float, 1, 0, 3)                                               \
+    X(__nv_bfloat16, 0, 0, 0) X(__nv_bfloat16, 1, 0, 0) X(__nv_bfloat16, 0, 1, 0) X(__nv_bfloat16, 1, 1, 0) \
+    X(__nv_bfloat16, 0, 2, 0) X(__nv_bfloat16, 1, 2, 0) X(__nv_bfloat16, 0, 0, 1) X(__nv_bfloat16, 0, 0, 3) \
+    X(__nv_bfloat16, 1, 0, 3)

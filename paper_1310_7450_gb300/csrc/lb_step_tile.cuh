@@ -227,14 +227,7 @@ __global__ void __launch_bounds__(NT) k_step_tile(const StepArgs<T, C> a) {
         }
 
         if (a.flags & F_FIELDS) {
-            const long long node = P.node_off + pn;
-            a.fu[2 * node] = urx;
-            a.fu[2 * node + 1] = ury;
-            a.fsig[4 * node + 0] = s.sxx;
-            a.fsig[4 * node + 1] = s.syy;
-            a.fsig[4 * node + 2] = C(0);
-            a.fsig[4 * node + 3] = s.sxy;
-            a.frho[node] = rho_h;
+            store_fields<C>(a, P.node_off + pn, urx, ury, s.sxx, s.syy, s.sxy, rho_h);
         } else {
             C D[9];
             if constexpr (SCHEME != 0) collide_impl<C, true>(P, s, d, D, om, k2, fx, fy);
