@@ -29,7 +29,8 @@ sys.path.insert(0, ROOT)
 METRIC = "GLUPS & % HBM roofline; batched-sweep time-to-steady, plain vs warm-start"
 UNIT = "GLUPS"
 KERNEL_SOURCES = {
-    "k_step_march": ["paper_1310_7450_gb300/csrc/lb_step_march.cuh", "paper_1310_7450_gb300/csrc/lb_device.cuh"],
+    "k_step_march": ["paper_1310_7450_gb300/csrc/lb_step_march.cuh", "paper_1310_7450_gb300/csrc/lb_pair.cuh",
+                     "paper_1310_7450_gb300/csrc/lb_device.cuh"],
     "k_step_tile": ["paper_1310_7450_gb300/csrc/lb_step_tile.cuh", "paper_1310_7450_gb300/csrc/lb_device.cuh"],
 }
 

@@ -66,10 +66,6 @@ extern template cudaError_t launch_step_tile<__nv_bfloat16, float, 0, 1>(const S
                                                                          cudaStream_t);
 extern template cudaError_t launch_step_tile<__nv_bfloat16, float, 0, 2>(const StepArgs<__nv_bfloat16, float>&, int, size_t,
                                                                          cudaStream_t);
-extern template cudaError_t launch_step_march<float, float, 0>(const CUtensorMap&, const StepArgs<float, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<float, float, 1>(const CUtensorMap&, const StepArgs<float, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<__nv_bfloat16, float, 0>(const CUtensorMap&, const StepArgs<__nv_bfloat16, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<__nv_bfloat16, float, 1>(const CUtensorMap&, const StepArgs<__nv_bfloat16, float>&, const MarchCtl&, int, cudaStream_t);
 #define LB_SWEEP_EXTERN(T, C, NX)                                                                                   \
     extern template cudaError_t launch_sweep<T, C, 128, 4, NX>(const SweepArgs<T, C>&, int, int, size_t, cudaStream_t); \
     extern template cudaError_t launch_sweep<T, C, 256, 4, NX>(const SweepArgs<T, C>&, int, int, size_t, cudaStream_t); \
@@ -94,44 +90,13 @@ LB_SWEEP_SMEM_EXTERN(float, float, 4)
 LB_SWEEP_SMEM_EXTERN(__nv_bfloat16, float, 4)
 LB_SWEEP_SMEM_EXTERN(double, double, 4)
 #undef LB_SWEEP_SMEM_EXTERN
-extern template cudaError_t march_occupancy<float, float, 0>(int*);
-extern template cudaError_t march_occupancy<float, float, 1>(int*);
-extern template cudaError_t march_occupancy<__nv_bfloat16, float, 0>(int*);
-extern template cudaError_t march_occupancy<__nv_bfloat16, float, 1>(int*);
-extern template cudaError_t launch_step_march<float, float, 0, 0, 1>(const CUtensorMap&, const StepArgs<float, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<__nv_bfloat16, float, 0, 0, 1>(const CUtensorMap&, const StepArgs<__nv_bfloat16, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t march_occupancy<float, float, 0, 0, 1>(int*);
-extern template cudaError_t march_occupancy<__nv_bfloat16, float, 0, 0, 1>(int*);
-extern template cudaError_t launch_step_march<float, float, 0, 0, 3>(const CUtensorMap&, const StepArgs<float, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<float, float, 1, 0, 3>(const CUtensorMap&, const StepArgs<float, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<__nv_bfloat16, float, 0, 0, 3>(const CUtensorMap&, const StepArgs<__nv_bfloat16, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<__nv_bfloat16, float, 1, 0, 3>(const CUtensorMap&, const StepArgs<__nv_bfloat16, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t march_occupancy<float, float, 0, 0, 3>(int*);
-extern template cudaError_t march_occupancy<float, float, 1, 0, 3>(int*);
-extern template cudaError_t march_occupancy<__nv_bfloat16, float, 0, 0, 3>(int*);
-extern template cudaError_t march_occupancy<__nv_bfloat16, float, 1, 0, 3>(int*);
-extern template cudaError_t launch_step_march<float, float, 0, 1>(const CUtensorMap&, const StepArgs<float, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<float, float, 1, 1>(const CUtensorMap&, const StepArgs<float, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<__nv_bfloat16, float, 0, 1>(const CUtensorMap&, const StepArgs<__nv_bfloat16, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<__nv_bfloat16, float, 1, 1>(const CUtensorMap&, const StepArgs<__nv_bfloat16, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t march_occupancy<float, float, 0, 1>(int*);
-extern template cudaError_t march_occupancy<float, float, 1, 1>(int*);
-extern template cudaError_t march_occupancy<__nv_bfloat16, float, 0, 1>(int*);
-extern template cudaError_t march_occupancy<__nv_bfloat16, float, 1, 1>(int*);
-extern template cudaError_t launch_step_march<float, float, 0, 2>(const CUtensorMap&, const StepArgs<float, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<float, float, 1, 2>(const CUtensorMap&, const StepArgs<float, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<__nv_bfloat16, float, 0, 2>(const CUtensorMap&, const StepArgs<__nv_bfloat16, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t launch_step_march<__nv_bfloat16, float, 1, 2>(const CUtensorMap&, const StepArgs<__nv_bfloat16, float>&, const MarchCtl&, int, cudaStream_t);
-extern template cudaError_t march_occupancy<float, float, 0, 2>(int*);
-extern template cudaError_t march_occupancy<float, float, 1, 2>(int*);
-extern template cudaError_t march_occupancy<__nv_bfloat16, float, 0, 2>(int*);
-extern template cudaError_t march_occupancy<__nv_bfloat16, float, 1, 2>(int*);
-#define LB_MARCH_FIELDS_EXTERN(T, SMODE, BND, SCHEME)                                                                       \
-    extern template cudaError_t launch_step_march<T, float, SMODE, BND, SCHEME, true>(const CUtensorMap&,                       \
-                                                                                      const StepArgs<T, float>&, const MarchCtl&, \
-                                                                                      int, cudaStream_t);
-LB_MARCH_FIELDS_ALL(LB_MARCH_FIELDS_EXTERN)
-#undef LB_MARCH_FIELDS_EXTERN
+#define X(T, SMODE, BND, SCHEME)                                                                              \
+    LB_MARCH_STEP(extern, T, SMODE, BND, SCHEME, kFull) LB_MARCH_FIELDS(extern, T, SMODE, BND, SCHEME, kFull) \
+    LB_MARCH_STEP(extern, T, SMODE, BND, SCHEME, kPart) LB_MARCH_FIELDS(extern, T, SMODE, BND, SCHEME, kPart) \
+    LB_MARCH_STEP(extern, T, SMODE, BND, SCHEME, kOdd) LB_MARCH_FIELDS(extern, T, SMODE, BND, SCHEME, kOdd)
+LB_MARCH_VARIANTS(X, float)
+LB_MARCH_VARIANTS(X, __nv_bfloat16)
+#undef X
 }  // namespace lbk
 
 using namespace lbk;
@@ -416,6 +381,7 @@ struct lb_handle {
     unsigned long long wait_ns = kDefaultWaitNs;  // limit of the row-march kernel's mbarrier waits
     // row-march kernel (wide single channels, FP32 / BF16 storage)
     bool march = false;
+    int march_strip = kFull;   // its strips: whole, partial, or rows of any length
     CUtensorMap mapA, mapB;    // tensor maps of the two population buffers ...
     const void* mapA_buf = nullptr;  // ... and the buffers they describe (the pointers swap)
     const void* mapB_buf = nullptr;
@@ -562,16 +528,17 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// 3-D map over the 9 population planes of channel 0: dims (nx, ny, 9), box (W + 2 HP, 1, 9).
+// 3-D map over the 9 population planes of channel 0: dims (nx, ny, 9), box (strip, 1, 9); where the row length is
+// no multiple of 16 bytes the planes are one row each: dims (nx ny, 1, 9).
 bool make_pop_map(const lb_handle* h, void* base, CUtensorMap* map) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
-    const bool bf = h->prec == LB_PREC_BF16;
-    const cuuint64_t es = bf ? 2 : 4;
-    const cuuint32_t hp = (cuuint32_t)(16 / es);
-    cuuint64_t dims[3] = {(cuuint64_t)h->nx, (cuuint64_t)h->ny[0], 9};
-    cuuint64_t strides[2] = {(cuuint64_t)h->nx * es, (cuuint64_t)h->P[0] * es};
-    cuuint32_t box[3] = {(cuuint32_t)kMarchW + 2 * hp, 1, 9};
+    const bool bf = h->prec == LB_PREC_BF16, odd = h->march_strip == kOdd;
+    const cuuint64_t es = bf ? 2 : 4, plane = (cuuint64_t)h->P[0] * es;
+    const int width = bf ? march_slot_width<__nv_bfloat16>(kMarchW, odd) : march_slot_width<float>(kMarchW, odd);
+    cuuint64_t dims[3] = {(cuuint64_t)h->nx * (odd ? h->ny[0] : 1), odd ? 1 : (cuuint64_t)h->ny[0], 9};
+    cuuint64_t strides[2] = {odd ? plane : (cuuint64_t)h->nx * es, plane};
+    cuuint32_t box[3] = {(cuuint32_t)width, 1, 9};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = enc(map, bf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides,
                      box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -613,7 +580,13 @@ static MarchModel march_model(int prec, bool gpbc) {
 }
 
 static std::vector<MarchItem> march_plan(int nx, int ny, int R, int nsm, MarchModel m) {
-    const int strips = nx / kMarchW;
+    // strips of one width (a multiple of 8 columns) but the last, which has two at least (a halo column's
+    // populations come from one column further on)
+    const int least = (nx + kMarchW - 1) / kMarchW;
+    int W = std::min(kMarchW, ((nx + least - 1) / least + 7) / 8 * 8);
+    while (nx % W == 1) W -= 8;
+    const int strips = (nx + W - 1) / W;
+    auto width = [&](int x0) { return std::min(W, nx - x0); };
     const int slots = R * nsm;
     const int maxn = std::max(1, ny / 8);
     auto speed = [&](int b) {
@@ -634,6 +607,7 @@ static std::vector<MarchItem> march_plan(int nx, int ny, int R, int nsm, MarchMo
             it.x0 = x0;
             it.y0 = y;
             it.y1 = y1;
+            it.w = width(x0);
             out.push_back(it);
             y = y1;
         }
@@ -686,7 +660,7 @@ static std::vector<MarchItem> march_plan(int nx, int ny, int R, int nsm, MarchMo
     auto strip_items = [&](int s, int cnt) {
         std::vector<double> w(cnt);
         for (int k = 0; k < cnt; ++k) w[k] = speed(b + k);
-        split(items, s * kMarchW, w);
+        split(items, s * W, w);
         b += cnt;
     };
     if (!cm) {
@@ -703,10 +677,53 @@ static std::vector<MarchItem> march_plan(int nx, int ny, int R, int nsm, MarchMo
     for (int c = 0; c < C; ++c)
         for (int s = 1; s <= I; ++s) {
             MarchItem it = chunk[c];
-            it.x0 = s * kMarchW;
+            it.x0 = s * W;
+            it.w = width(it.x0);
             items.push_back(it);
         }
     return items;
+}
+
+// The row-march variant of a handle: f(stress mode, boundary, scheme, strips) as constants.
+template <int V> using Num = std::integral_constant<int, V>;
+template <typename F>
+auto march_variant(const lb_handle* h, F&& f) {
+    auto with_strip = [&](auto sm, auto bnd, auto sch) {
+        if (h->march_strip == kOdd) return f(sm, bnd, sch, Num<kOdd>{});
+        return h->march_strip == kPart ? f(sm, bnd, sch, Num<kPart>{}) : f(sm, bnd, sch, Num<kFull>{});
+    };
+    auto with_mode = [&](auto bnd, auto sch) {
+        return h->smode ? with_strip(Num<1>{}, bnd, sch) : with_strip(Num<0>{}, bnd, sch);
+    };
+    if (h->scheme == 1) return with_strip(Num<0>{}, Num<0>{}, Num<1>{});
+    if (h->scheme == 3) return with_mode(Num<0>{}, Num<3>{});
+    if (h->gpbc) return with_mode(Num<1>{}, Num<0>{});
+    if (h->moving) return with_mode(Num<2>{}, Num<0>{});
+    return with_mode(Num<0>{}, Num<0>{});
+}
+
+// A grid too small to give every resident CTA an 8-row item is cut finer, down to 2 rows: a row takes about 1.5 us
+// whatever the chip's load (its instructions wait for one another), so the launch lasts as long as its
+// longest item.  128 x 512 FP32: 18.8 us with 8-row items, 9.6 with 2-row ones.
+static std::vector<MarchItem> fine_items(std::vector<MarchItem> in, int nx, int ny, int slots) {
+    int strips = 0, W = in[0].w;
+    for (const MarchItem& it : in) {
+        strips += it.y0 == 0;
+        W = std::max(W, it.w);
+    }
+    if ((long long)strips * (ny / 8) >= slots) return in;
+    const int n = std::min(ny / 2, std::max(1, slots / strips));
+    std::vector<MarchItem> out;
+    for (int k = 0; k < n; ++k)
+        for (int s = 0; s < strips; ++s) {
+            MarchItem it{};
+            it.x0 = s * W;
+            it.w = std::min(W, nx - it.x0);
+            it.y0 = (int)((long long)ny * k / n);
+            it.y1 = (int)((long long)ny * (k + 1) / n);
+            out.push_back(it);
+        }
+    return out;
 }
 
 // The kernel addresses an item's rows with 32-bit offsets: items of 2^29 elements or more are halved.
@@ -731,37 +748,39 @@ static std::vector<MarchItem> short_items(const std::vector<MarchItem>& in, int 
     return out;
 }
 
+// Whole strips always march; other widths where that is the faster kernel.  A march step lasts 10 us at least (a
+// chain of rows), a tile step 5, but the tile kernel takes 1.3 to 2 times as long per node.  Tile / march, us:
+// FP32 100 x 1600 10.1 / 12.7, 200 x 1600 15.8 / 16.8, 500 x 800 17.5 / 16.8, 1000 x 777 30.1 / 23.0, 1001 x 777
+// 30.7 / 25.0, 2049 x 600 52.3 / 35.0; BF16 200 x 400 9.4 / 10.6, 70 x 2000 16.2 / 15.7, 100 x 1600 16.0 / 13.3,
+// 1000 x 300 18.1 / 13.5, 1001 x 777 44.8 / 26.8.  Below 96 columns half of a strip's threads have none.
+static bool march_pays(const lb_handle* h) {
+    if (h->nx % kMarchW == 0) return true;
+    return h->nx >= 96 && (long long)h->nx * h->ny[0] >= (h->prec == LB_PREC_BF16 ? 150000 : 400000);
+}
+
 lb_status plan_march(lb_handle* h) {
     h->march = false;
-    if (h->n_ch != 1 || (h->prec != LB_PREC_F32 && h->prec != LB_PREC_BF16) || h->nx % kMarchW != 0 ||
-        h->ny[0] < 16 || (h->flags & LB_GRID_TILE_ONLY) || h->scheme == 2 ||
-        (h->scheme == 3 && (h->gpbc || h->moving)))
+    if (h->n_ch != 1 || (h->prec != LB_PREC_F32 && h->prec != LB_PREC_BF16) || h->ny[0] < 16 ||
+        (h->flags & LB_GRID_TILE_ONLY) || h->scheme == 2 || (h->scheme == 3 && (h->gpbc || h->moving)) || !march_pays(h))
         return LB_OK;
+    h->march_strip = h->nx % kMarchW == 0 ? kFull : (h->nx % (h->prec == LB_PREC_BF16 ? 8 : 4) == 0 ? kPart : kOdd);
+    if (h->march_strip == kOdd && (long long)h->nx * (h->ny[0] + 4) >= (1ll << 31) - 4096) return LB_OK;  // (copy coordinates)
     if (!make_pop_map(h, h->popA, &h->mapA) || !make_pop_map(h, h->popB, &h->mapB)) return LB_OK;
     h->mapA_buf = h->popA;
     h->mapB_buf = h->popB;
     int bps = 0, nsm = 0;
     cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->dev);
-    if (e == cudaSuccess) {
-        const bool bnd = h->gpbc || h->moving;
-        if (h->prec == LB_PREC_F32) {
-            if (h->scheme == 1) e = march_occupancy<float, float, 0, 0, 1>(&bps);
-            else if (h->scheme == 3) e = h->smode ? march_occupancy<float, float, 1, 0, 3>(&bps) : march_occupancy<float, float, 0, 0, 3>(&bps);
-            else if (h->gpbc) e = h->smode ? march_occupancy<float, float, 1, 1>(&bps) : march_occupancy<float, float, 0, 1>(&bps);
-            else if (bnd) e = h->smode ? march_occupancy<float, float, 1, 2>(&bps) : march_occupancy<float, float, 0, 2>(&bps);
-            else e = h->smode ? march_occupancy<float, float, 1>(&bps) : march_occupancy<float, float, 0>(&bps);
-        } else {
-            if (h->scheme == 1) e = march_occupancy<__nv_bfloat16, float, 0, 0, 1>(&bps);
-            else if (h->scheme == 3) e = h->smode ? march_occupancy<__nv_bfloat16, float, 1, 0, 3>(&bps) : march_occupancy<__nv_bfloat16, float, 0, 0, 3>(&bps);
-            else if (h->gpbc) e = h->smode ? march_occupancy<__nv_bfloat16, float, 1, 1>(&bps) : march_occupancy<__nv_bfloat16, float, 0, 1>(&bps);
-            else if (bnd) e = h->smode ? march_occupancy<__nv_bfloat16, float, 1, 2>(&bps) : march_occupancy<__nv_bfloat16, float, 0, 2>(&bps);
-            else e = h->smode ? march_occupancy<__nv_bfloat16, float, 1>(&bps) : march_occupancy<__nv_bfloat16, float, 0>(&bps);
-        }
-    }
+    if (e == cudaSuccess)
+        e = march_variant(h, [&](auto sm, auto bnd, auto sch, auto strip) {
+            constexpr int SM = decltype(sm)::value, B = decltype(bnd)::value, S = decltype(sch)::value;
+            return h->prec == LB_PREC_F32 ? march_occupancy<float, float, SM, B, S, decltype(strip)::value>(&bps)
+                                          : march_occupancy<__nv_bfloat16, float, SM, B, S, decltype(strip)::value>(&bps);
+        });
     if (e != cudaSuccess) return cuda_fail(e, "lb_create: march occupancy");
     if (bps < 1) return LB_OK;
     const int slots = bps * nsm;
-    const std::vector<MarchItem> items = short_items(march_plan(h->nx, h->ny[0], bps, nsm, march_model(h->prec, h->gpbc)), h->nx);
+    const std::vector<MarchItem> items = short_items(
+        fine_items(march_plan(h->nx, h->ny[0], bps, nsm, march_model(h->prec, h->gpbc)), h->nx, h->ny[0], slots), h->nx);
     LB_CK(cudaMalloc(&h->march_items_d, sizeof(MarchItem) * items.size()));
     LB_CK(cudaMemcpy(h->march_items_d, items.data(), sizeof(MarchItem) * items.size(), cudaMemcpyHostToDevice));
     h->n_march_items = (int)items.size();
@@ -971,20 +990,10 @@ cudaError_t launch_march_as(lb_handle* h, const StepArgs<T, float>& a) {
     MarchCtl ctl{h->march_items_d, h->n_march_items, h->status_d, h->P[0], h->base[0], FIELDS ? kDefaultWaitNs : h->wait_ns};
     march_monitor(h, a.flags, ctl);
     const CUtensorMap& m = ((const void*)a.pin == h->mapA_buf) ? h->mapA : h->mapB;
-    const int grid = h->march_grid;
-    const cudaStream_t s = h->stream;
-    if (h->scheme == 1) return launch_step_march<T, float, 0, 0, 1, FIELDS>(m, a, ctl, grid, s);
-    if (h->scheme == 3)
-        return h->smode ? launch_step_march<T, float, 1, 0, 3, FIELDS>(m, a, ctl, grid, s)
-                        : launch_step_march<T, float, 0, 0, 3, FIELDS>(m, a, ctl, grid, s);
-    if (h->gpbc)
-        return h->smode ? launch_step_march<T, float, 1, 1, 0, FIELDS>(m, a, ctl, grid, s)
-                        : launch_step_march<T, float, 0, 1, 0, FIELDS>(m, a, ctl, grid, s);
-    if (h->moving)
-        return h->smode ? launch_step_march<T, float, 1, 2, 0, FIELDS>(m, a, ctl, grid, s)
-                        : launch_step_march<T, float, 0, 2, 0, FIELDS>(m, a, ctl, grid, s);
-    return h->smode ? launch_step_march<T, float, 1, 0, 0, FIELDS>(m, a, ctl, grid, s)
-                    : launch_step_march<T, float, 0, 0, 0, FIELDS>(m, a, ctl, grid, s);
+    return march_variant(h, [&](auto sm, auto bnd, auto sch, auto strip) {
+        return launch_step_march<T, float, decltype(sm)::value, decltype(bnd)::value, decltype(sch)::value, FIELDS,
+                                 decltype(strip)::value>(m, a, ctl, h->march_grid, h->stream);
+    });
 }
 template <typename T, typename C>
 cudaError_t launch_march(lb_handle* h, const StepArgs<T, C>& a) {

@@ -28,8 +28,11 @@
 
 namespace lbk {
 
+enum : int { kFull = 0, kPart = 1, kOdd = 2 };  // strips of a channel, see k_step_march
+
 struct MarchItem {
-    int x0, y0, y1, pad_;
+    int x0, y0, y1;  // first column, rows [y0, y1)
+    int w;           // columns (kMarchW at most)
 };
 
 struct MarchCtl {
@@ -122,11 +125,15 @@ struct MarchGeom {
     static constexpr int HP = 16 / (int)sizeof(T);  // halo columns per side (16 bytes)
 };
 
+// Elements of a slot row: the strip and its halo; ODD: and up to HP - 1 elements before them, since a copy starts
+// on a 16-byte boundary and the rows of a channel whose width is no multiple of 16 bytes do not.
+template <typename T>
+__host__ __device__ constexpr int march_slot_width(int W, bool odd) { return W + (odd ? 3 : 2) * MarchGeom<T>::HP; }
+
 // Shared-memory footprint of the march kernel (bytes).
-template <typename T, typename C, int W, int K>
+template <typename T, typename C, int W, int K, bool ODD>
 constexpr size_t march_smem_bytes() {
-    constexpr int HP = MarchGeom<T>::HP;
-    constexpr size_t slot = ((size_t)9 * (W + 2 * HP) * sizeof(T) + 8 + 127) / 128 * 128;
+    constexpr size_t slot = ((size_t)9 * march_slot_width<T>(W, ODD) * sizeof(T) + 8 + 127) / 128 * 128;
     return K * slot + (std::is_same<T, float>::value ? (size_t)W * 2 * sizeof(C) + 4 * 4 * 2 * sizeof(C)
                                                      : (size_t)4 * (W + 4) * 2 * sizeof(C));
 }
@@ -163,16 +170,22 @@ __device__ __forceinline__ P2 slot_pair_odd(const T* p) {
 // SCHEME 3: the relaxation-time extensions (periodic x, bounce-back walls, either stress mode): the
 // node's FP64 fluidity is loaded one row ahead of its use and stored with the step, as in the tile
 // kernel's scheme-3 variant.
+// STRIP: kFull, the width is a multiple of CW; kPart, strips of another width, rows a multiple of 16 bytes; kOdd,
+// rows of any length.  kOdd's copies come from a map of the planes as one long row each, start on the
+// 16-byte boundary before the strip, and the pulls add the remainder of each row; its global loads and
+// stores go column by column.  (Variants of their own: the masks of a partial strip cost whole strips 13 % in
+// FP32 and 22 % in BF16.)
 // FIELDS: the fields of the stored state (F_FIELDS) instead of a step: everything up to the stress, then
 // u, sigma and rho in node order.
-template <typename T, typename C, int SMODE, int CW, int K, int BND = 0, int SCHEME = 0, bool FIELDS = false>
+template <typename T, typename C, int SMODE, int CW, int K, int BND = 0, int SCHEME = 0, bool FIELDS = false, int STRIP = 0>
 __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant__ CUtensorMap tmap,
                                                                                   const StepArgs<T, C> a,
                                                                                   const MarchCtl ctl) {
     static_assert(std::is_same<C, float>::value, "the pair arithmetic is FP32");
     constexpr int NT = CW / 2;                                       // threads per CTA
+    constexpr bool ODD = STRIP == kOdd;
     constexpr int HP = MarchGeom<T>::HP;
-    constexpr int SW = CW + 2 * HP;                                  // slot row width (elements)
+    constexpr int SW = march_slot_width<T>(CW, ODD);                 // slot row width (elements)
     constexpr uint32_t TX = 9u * SW * sizeof(T);                     // bytes per copy
     constexpr uint32_t SLOT = (TX + 8 + 127) / 128 * 128;            // a slot: the copy, then its mbarrier
     // measured choices, see the note above the launchers
@@ -238,7 +251,12 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
 
     auto issue = [&](uint32_t off, int x0, int row) {  // issuing thread (TI) only
         mbar_expect_tx(bar_at(off), TX);
-        tma_load_3d(slots + off, &tmap, bar_at(off), x0 - HP, row, 0);
+        if constexpr (ODD) {
+            const int x = row * nx + x0 - HP;  // (the host keeps planes below 2^31 elements)
+            tma_load_3d(slots + off, &tmap, bar_at(off), x - (x & (HP - 1)), 0, 0);
+        } else {
+            tma_load_3d(slots + off, &tmap, bar_at(off), x0 - HP, row, 0);
+        }
     };
     // the slot after the one at `off`
     auto next_slot = [&](uint32_t off) -> uint32_t { return off == (K - 1) * SLOT ? 0u : off + SLOT; };
@@ -246,32 +264,40 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
 
     for (int item = blockIdx.x; item < ctl.n_items && !bad && !halted; item += gridDim.x) {
         const MarchItem it = ctl.items[item];
-        const int x0 = it.x0, y0 = it.y0, y1 = it.y1;
+        const int x0 = it.x0, y0 = it.y0, y1 = it.y1, sw = STRIP == kFull ? CW : it.w;
         const int rbase = y0 - 2;                 // first source row of this item
         const int rlast = y1 + 1;                 // last source row
         const uint32_t L0 = nload;                // load index of row rbase
-        const bool left_edge = (x0 == 0), right_edge = (x0 + CW == nx);
-        const int col0 = 2 * t;                   // first own column (relative to x0)
+        const bool left_edge = (x0 == 0), right_edge = (x0 + sw == nx);
+        // first own column (relative to x0).  Threads beyond a narrower strip repeat its last pair and
+        // store nothing; with an odd width the last pair's second column is the halo column
+        const int col0 = STRIP == kFull ? 2 * t : min(2 * t, ODD ? (sw - 1) & ~1 : sw - 2);
+        const bool own0 = STRIP == kFull || 2 * t < sw, own1 = STRIP == kFull || 2 * t + 1 < sw;
+        const bool last_pair = STRIP == kFull ? t == NT - 1 : col0 + 2 == sw;
 
         // index of the copy holding source row r, its slot, and the wait for it
         auto idx_of = [&](int r) -> uint32_t { return L0 + (uint32_t)(r - rbase); };
         auto slot_off = [&](int r) -> uint32_t { return (idx_of(r) % K) * SLOT; };
+        // offset of column x0 - HP of row r inside the slots, given its slot
+        auto row_at = [&](uint32_t off, int r) -> uint32_t {
+            return ODD ? off + ((uint32_t)(r * nx + x0) & (HP - 1)) * (uint32_t)sizeof(T) : off;
+        };
         auto wait_row = [&](int r) -> bool {
             const uint32_t i = idx_of(r);
             return mbar_wait(bar_at((i % K) * SLOT), (i / K) & 1u, ctl.max_wait_ns);
         };
-        // periodic wrap: the edge strips' halo columns x0-2, x0-1 (left) or x0+CW, x0+CW+1 (right)
+        // periodic wrap: the edge strips' halo columns x0-2, x0-1 (left) or x0+sw, x0+sw+1 (right)
         // come from the other end of the row; threads 0..17 (left) and 32..49 (right) each own
         // one (direction, column) value, loaded two rows before it is patched into its slot
         const bool patcher = (left_edge && t < 18) || (right_edge && t >= 32 && t < 50);
         const int pi = left_edge && t < 18 ? (t >> 1) : ((t - 32) >> 1);             // direction
         const int pc = left_edge && t < 18 ? (nx - 2 + (t & 1)) : ((t - 32) & 1);     // global column
-        const int ps = left_edge && t < 18 ? (HP - 2 + (t & 1)) : (HP + CW + ((t - 32) & 1));  // slot column
+        const int ps = left_edge && t < 18 ? (HP - 2 + (t & 1)) : (HP + sw + ((t - 32) & 1));  // slot column
         auto patch_load = [&](int r) -> T {
             return (r >= 0 && r < ny && r <= rlast) ? a.pin[9 * ctl.base + (long long)pi * PL + (long long)r * nx + pc] : T(0);
         };
         auto patch_store = [&](int r, T v) {
-            if (r >= 0 && r < ny && r <= rlast) reinterpret_cast<T*>(slots + slot_off(r))[pi * SW + ps] = v;
+            if (r >= 0 && r < ny && r <= rlast) reinterpret_cast<T*>(slots + row_at(slot_off(r), r))[pi * SW + ps] = v;
         };
         // GPBC brackets: lanes 0..5 of the left edge strip's patchers (32..37 on a right edge
         // strip) take one (boundary column, direction) each and evaluate source row r from the
@@ -284,8 +310,8 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
             if (r < 0 || r >= ny || r > rlast) return;
             const int c = sl / 3, j = sl - 3 * (sl / 3);
             const int i = c == 1 ? (j == 0 ? 1 : (j == 1 ? 5 : 8)) : (j == 0 ? 3 : (j == 1 ? 6 : 7));
-            const int bcol = c == 1 ? (right_edge ? CW - 1 : -1) : (left_edge ? 0 : CW);
-            const T* sb = reinterpret_cast<const T*>(slots + slot_off(r)) + HP + bcol;
+            const int bcol = c == 1 ? (right_edge ? sw - 1 : -1) : (left_edge ? 0 : sw);
+            const T* sb = reinterpret_cast<const T*>(slots + row_at(slot_off(r), r)) + HP + bcol;
             C e[9], mR, mx, my;
 #pragma unroll
             for (int k = 0; k < 9; ++k) e[k] = (C)Store<T>::cvt(sb[k * SW]);
@@ -323,9 +349,9 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
         // direction i comes from source row r - cy_i, column col - cx_i.  om, o0, op: slot offsets of
         // the source rows r-1, r, r+1
         auto pull_one = [&](int col, int r, uint32_t om, uint32_t o0, uint32_t op, C (&d)[9]) {
-            const T* sm = reinterpret_cast<const T*>(slots + om) + HP + col;
-            const T* s0 = reinterpret_cast<const T*>(slots + o0) + HP + col;
-            const T* sp = reinterpret_cast<const T*>(slots + op) + HP + col;
+            const T* sm = reinterpret_cast<const T*>(slots + row_at(om, r - 1)) + HP + col;
+            const T* s0 = reinterpret_cast<const T*>(slots + row_at(o0, r)) + HP + col;
+            const T* sp = reinterpret_cast<const T*>(slots + row_at(op, r + 1)) + HP + col;
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
                 const bool wall = (cy(i) == 1 && r == 0) || (cy(i) == -1 && r == ny - 1);
@@ -336,21 +362,25 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
         };
         // the same for the thread's two columns
         auto pull_pair = [&](int r, uint32_t om, uint32_t o0, uint32_t op, P2 (&d)[9]) {
-            const T* sm = reinterpret_cast<const T*>(slots + om) + HP + col0;
-            const T* s0 = reinterpret_cast<const T*>(slots + o0) + HP + col0;
-            const T* sp = reinterpret_cast<const T*>(slots + op) + HP + col0;
+            const T* sm = reinterpret_cast<const T*>(slots + row_at(om, r - 1)) + HP + col0;
+            const T* s0 = reinterpret_cast<const T*>(slots + row_at(o0, r)) + HP + col0;
+            const T* sp = reinterpret_cast<const T*>(slots + row_at(op, r + 1)) + HP + col0;
+            auto even_pair = [&](const T* p) -> P2 {  // (columns of even index: one access where rows are aligned)
+                if constexpr (ODD) return slot_pair_odd<T>(p);
+                else return slot_pair(p);
+            };
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
                 const T* sr = cy(i) == 1 ? sm : (cy(i) == -1 ? sp : s0);
-                d[i] = cx(i) == 0 ? slot_pair(sr + i * SW) : slot_pair_odd<T>(sr + i * SW - cx(i));
+                d[i] = cx(i) == 0 ? even_pair(sr + i * SW) : slot_pair_odd<T>(sr + i * SW - cx(i));
             }
             if (r == 0 || r == ny - 1) {  // bounce-back at the wall (uniform over the CTA)
 #pragma unroll
                 for (int i = 0; i < 9; ++i)
-                    if (cy(i) != 0 && (cy(i) == 1 ? r == 0 : r == ny - 1)) d[i] = slot_pair(s0 + opp(i) * SW);
+                    if (cy(i) != 0 && (cy(i) == 1 ? r == 0 : r == ny - 1)) d[i] = even_pair(s0 + opp(i) * SW);
             }
             if (BND >= 1) {
-                const bool near_end = gpbc_edge && ((left_edge && t == 0) || (right_edge && t == NT - 1));
+                const bool near_end = gpbc_edge && ((left_edge && col0 == 0) || (right_edge && col0 + 2 >= sw));
                 if (near_end || r == ny - 1) {
                     C e0[9], e1[9];
 #pragma unroll
@@ -440,7 +470,7 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
             }
         }
         moments_row(y0, slot_off(y0 - 1), slot_off(y0), slot_off(y0 + 1), dA, dRa, jxa, jya, u0_x, u0_y);
-        if (t < 2) halo_node(y0, t == 0 ? -1 : CW, slot_off(y0 - 1), slot_off(y0), slot_off(y0 + 1));
+        if (t < 2) halo_node(y0, t == 0 ? -1 : sw, slot_off(y0 - 1), slot_off(y0), slot_off(y0 + 1));
         // offsets of this item's fields from its first row's first own column
         const long long ubase = ctl.base + (long long)y0 * nx + x0, ibase = ubase + col0;
         // address of the thread's columns in row y of a field: `o` / `vo` rows into the item.  FP32: a
@@ -453,16 +483,41 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
             else
                 return f + ibase + o;
         };
+        // the thread's own columns of a field: one access for both, or (ODD) one each
+        auto ld = [&](const C* p) -> P2 {
+            if constexpr (ODD) return p2(p[0], own1 ? p[1] : 0.f);
+            else return load_pair(p);
+        };
+        auto st = [&](C* p, P2 v) {
+            if constexpr (ODD) {
+                if (own0) p[0] = lo(v);
+                if (own1) p[1] = hi(v);
+            } else if (own0) {
+                store_pair(p, v);
+            }
+        };
+        auto st_pop = [&](T* p, P2 v) {
+            if constexpr (ODD) {
+                if (own0) Store<T>::st(p, lo(v));
+                if (own1) Store<T>::st(p + 1, hi(v));
+            } else if (own0) {
+                store_pop_pair(p, v);
+            }
+        };
+        auto ld_phi = [&](const double* p) -> double2 {
+            if constexpr (ODD) return make_double2(p[0], own1 ? p[1] : 0.0);
+            else return *reinterpret_cast<const double2*>(p);
+        };
         // the stored flow-induced density, loaded two rows ahead of its use
         const C* drow = a.drho + ibase;
         P2 drho_next, drho_next2 = p2(0.f);
-        drho_next = load_pair(drow);
-        if (y0 + 1 < y1) drho_next2 = load_pair(drow + nx);
+        drho_next = ld(drow);
+        if (y0 + 1 < y1) drho_next2 = ld(drow + nx);
         // relaxation-time extensions with a fluidity memory: the node's fluidity (FP64), one row ahead
         const bool fluid = SCHEME == 3 && P.tau_f > C(0);  // CTA-uniform
         const double* phrow = a.phi + ibase;
         double2 phi_nxt = make_double2(0.0, 0.0);
-        if (fluid) phi_nxt = *reinterpret_cast<const double2*>(phrow);
+        if (fluid) phi_nxt = ld_phi(phrow);
         // on residual steps the saved velocity of each row is prefetched the same way, and one
         // thread brings the delta rho and saved-velocity rows into L2 four rows before their
         // register loads (a residual step reads 16 B more per node than a plain one, and the
@@ -470,21 +525,26 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
         const C* upx = a.uprev + ctl.base + ibase;
         auto prefetch_rows = [&](int r) {  // thread TP, residual steps, rows of this item only
             if (r < y1) {
+                // (whole 16-byte pieces: at an odd width the row's first and last ones are left out)
                 const long long o = (long long)r * nx + x0;
-                prefetch_l2(a.drho + ctl.base + o, CW * sizeof(C));
-                prefetch_l2(a.uprev + 2 * ctl.base + o, CW * sizeof(C));
-                prefetch_l2(a.uprev + 2 * ctl.base + PL + o, CW * sizeof(C));
+                const int lead = ODD ? (int)((4 - (o & 3)) & 3) : 0;
+                const uint32_t bytes = (uint32_t)max(0, (sw - lead) / 4) * 16u;
+                if (bytes) {
+                    prefetch_l2(a.drho + ctl.base + o + lead, bytes);
+                    prefetch_l2(a.uprev + 2 * ctl.base + o + lead, bytes);
+                    prefetch_l2(a.uprev + 2 * ctl.base + PL + o + lead, bytes);
+                }
             }
         };
         P2 upx_next = p2(0.f), upy_next = p2(0.f), upx_next2 = p2(0.f), upy_next2 = p2(0.f);
         if (resid) {
             if (t == TP)
                 for (int r = y0 + 2; r < y0 + 6; ++r) prefetch_rows(r);
-            upx_next = load_pair(upx);
-            upy_next = load_pair(upx + PL);
+            upx_next = ld(upx);
+            upy_next = ld(upx + PL);
             if (y0 + 1 < y1) {
-                upx_next2 = load_pair(upx + nx);
-                upy_next2 = load_pair(upx + PL + nx);
+                upx_next2 = ld(upx + nx);
+                upy_next2 = ld(upx + PL + nx);
             }
         }
         __syncthreads();
@@ -522,23 +582,23 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                     if (second && !mbar_wait(bar_at(o3), par3, ctl.max_wait_ns)) s_bad = 1;
                     const int r = y + 1 + (t >> 1);
                     if ((t < 2 || second) && r < ny)
-                        halo_node(r, (t & 1) == 0 ? -1 : CW, second ? o1 : o0, second ? o2 : o1, second ? o3 : o2);
+                        halo_node(r, (t & 1) == 0 ? -1 : sw, second ? o1 : o0, second ? o2 : o1, second ? o3 : o2);
                 }
             } else {
-                if (t < 2 && y + 1 < ny) halo_node(y + 1, t == 0 ? -1 : CW, o0, o1, o2);
+                if (t < 2 && y + 1 < ny) halo_node(y + 1, t == 0 ? -1 : sw, o0, o1, o2);
             }
             const P2 drho_prev = drho_next, upx_cur = upx_next, upy_cur = upy_next;
             drho_next = drho_next2;
-            if (y + 2 < y1) drho_next2 = load_pair(field_at(a.drho + 2LL * nx, o, vo));
+            if (y + 2 < y1) drho_next2 = ld(field_at(a.drho + 2LL * nx, o, vo));
             double2 phi_cur = phi_nxt;
-            if (fluid && y + 1 < y1) phi_nxt = *reinterpret_cast<const double2*>(phrow + o + nx);
+            if (fluid && y + 1 < y1) phi_nxt = ld_phi(phrow + o + nx);
             if (resid) {
                 if (t == TP) prefetch_rows(y + 6);
                 upx_next = upx_next2;
                 upy_next = upy_next2;
                 if (y + 2 < y1) {
-                    upx_next2 = load_pair(upx + o + 2 * nx);
-                    upy_next2 = load_pair(upx + PL + o + 2 * nx);
+                    upx_next2 = ld(upx + o + 2 * nx);
+                    upy_next2 = ld(upx + PL + o + 2 * nx);
                 }
             }
             __syncthreads();
@@ -559,11 +619,12 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                 // border from shared memory), or from the ring
                 float2 uw, ue;
                 if constexpr (SHUFFLE) {
-                    const float2 bw = edge[4 * (y & 3) + wid], be = edge[4 * (y & 3) + 2 + wid];
+                    const float2 bw = edge[4 * (y & 3) + wid];
+                    const float2 be = edge[4 * (y & 3) + (STRIP == kFull ? 2 + wid : (last_pair ? 3 : 2))];
                     uw = make_float2(__shfl_up_sync(0xffffffffu, hi(u0_x), 1), __shfl_up_sync(0xffffffffu, hi(u0_y), 1));
                     ue = make_float2(__shfl_down_sync(0xffffffffu, lo(u0_x), 1), __shfl_down_sync(0xffffffffu, lo(u0_y), 1));
                     if (lane == 0) uw = bw;
-                    if (lane == 31) ue = be;
+                    if (lane == 31 || (STRIP != kFull && last_pair)) ue = be;
                 } else {
                     uw = *reinterpret_cast<const float2*>(ring(y, col0 - 1));
                     ue = *reinterpret_cast<const float2*>(ring(y, col0 + 2));
@@ -588,9 +649,9 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                 P2 so_xx = p2(0.f), so_xy = p2(0.f), so_yy = p2(0.f);
                 if (SMODE == 1) {
                     const C* s3 = a.sig3 + 2 * ctl.base + ibase + o;
-                    so_xx = load_pair(s3);
-                    so_xy = load_pair(s3 + PL);
-                    so_yy = load_pair(s3 + 2 * PL);
+                    so_xx = ld(s3);
+                    so_xy = ld(s3 + PL);
+                    so_yy = ld(s3 + 2 * PL);
                 }
                 PairState s;
                 P2 om = q.om, nom = q.nom, k2 = q.k2;
@@ -607,7 +668,15 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                         const C t1 = relaxation_time_ext<C>(P, 0.5f * hi(Kx), 0.5f * hi(By), 0.5f * hi(Kc), 0.5f * hi(Ey),
                                                             hi(dRc), hi(drho_prev), phi_cur.y, &phi_new.y);
                         tau_M = p2(t0, t1);
-                        if (!FIELDS && fluid) *reinterpret_cast<double2*>(a.phi + ibase + o) = phi_new;
+                        if (!FIELDS && fluid) {
+                            double* ph = a.phi + ibase + o;
+                            if constexpr (ODD) {
+                                if (own0) ph[0] = phi_new.x;
+                                if (own1) ph[1] = phi_new.y;
+                            } else if (own0) {
+                                *reinterpret_cast<double2*>(ph) = phi_new;
+                            }
+                        }
                     }
                     s = constitutive<SMODE, BND == 1, SCHEME == 3>(q, Kx, By, Kc, Ey, dRc, jxc, jyc, drho_prev, so_xx, so_xy,
                                                                    so_yy, tau_M);
@@ -616,12 +685,12 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                 if constexpr (FIELDS) {
                     const P2 ih = rcp(rho_h), urx = mul(jxc, ih), ury = mul(jyc, ih);
                     const long long node = (long long)y * nx + x0 + col0;
-                    store_fields<C>(a, node, lo(urx), lo(ury), lo(s.sxx), lo(s.syy), lo(s.sxy), lo(rho_h));
-                    store_fields<C>(a, node + 1, hi(urx), hi(ury), hi(s.sxx), hi(s.syy), hi(s.sxy), hi(rho_h));
+                    if (own0) store_fields<C>(a, node, lo(urx), lo(ury), lo(s.sxx), lo(s.syy), lo(s.sxy), lo(rho_h));
+                    if (own1) store_fields<C>(a, node + 1, hi(urx), hi(ury), hi(s.sxx), hi(s.syy), hi(s.sxy), hi(rho_h));
                 }
                 {  // velocity_ok of both nodes: |u| <= guard without a division (false for NaN)
                     const P2 j2 = fma(jyc, jyc, mul(jxc, jxc)), g2 = mul(mul(p2(a.guard * a.guard), rho_h), rho_h);
-                    vbad |= !(lo(j2) <= lo(g2)) | !(hi(j2) <= hi(g2));
+                    vbad |= (own0 & !(lo(j2) <= lo(g2))) | (own1 & !(hi(j2) <= hi(g2)));
                 }
                 if constexpr (!FIELDS) {
                 P2 D[9];
@@ -635,42 +704,44 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                         d0[i] = lo(dcur[i]); d1[i] = hi(dcur[i]);
                         D0[i] = lo(D[i]); D1[i] = hi(D[i]);
                     }
-                    store_node<T, C>(field_at(po, o, vo), PL, d0, D0, true, a.sr_key, node);
-                    store_node<T, C>(field_at(po, o, vo) + 1, PL, d1, D1, true, a.sr_key, node + 1);
+                    if (own0) store_node<T, C>(field_at(po, o, vo), PL, d0, D0, true, a.sr_key, node);
+                    if (own1) store_node<T, C>(field_at(po, o, vo) + 1, PL, d1, D1, true, a.sr_key, node + 1);
                 } else {
 #pragma unroll
-                    for (int i = 0; i < 9; ++i) store_pop_pair(field_at(po + i * PL, o, vo), add(dcur[i], D[i]));
+                    for (int i = 0; i < 9; ++i) st_pop(field_at(po + i * PL, o, vo), add(dcur[i], D[i]));
                 }
-                store_pair(field_at(a.drho, o, vo), s.drho);
+                st(field_at(a.drho, o, vo), s.drho);
                 if (SMODE == 1) {
                     C* s3 = a.sig3 + 2 * ctl.base + ibase + o;
-                    store_pair(s3, s.sxx);
-                    store_pair(s3 + PL, s.sxy);
-                    store_pair(s3 + 2 * PL, s.syy);
+                    st(s3, s.sxx);
+                    st(s3 + PL, s.sxy);
+                    st(s3 + 2 * PL, s.syy);
                 }
                 if (store_sigma) {  // (the zz plane holds 0 from lb_create on)
                     C* s4 = a.sig4 + 3 * ctl.base;
-                    store_pair(field_at(s4, o, vo), s.sxx);
-                    store_pair(field_at(s4 + PL, o, vo), s.syy);
-                    store_pair(field_at(s4 + 3 * PL, o, vo), s.sxy);
+                    st(field_at(s4, o, vo), s.sxx);
+                    st(field_at(s4 + PL, o, vo), s.syy);
+                    st(field_at(s4 + 3 * PL, o, vo), s.sxy);
                 }
                 if (want_u) {
                     const P2 ih = rcp(rho_h);
                     const P2 urx = mul(jxc, ih), ury = mul(jyc, ih);
                     if (mon) {
-                        const P2 u2 = fma(ury, ury, mul(urx, urx));
+                        // (threads and halves without a column of their own add zeros, whatever they hold)
+                        auto mask = [&](P2 v) { return STRIP == kFull ? v : p2(own0 ? lo(v) : 0.f, own1 ? hi(v) : 0.f); };
+                        const P2 u2 = mask(fma(ury, ury, mul(urx, urx)));
                         if (resid) {
                             const P2 dx_ = sub(urx, upx_cur), dy_ = sub(ury, upy_cur);
-                            r_du2 = add(r_du2, fma(dy_, dy_, mul(dx_, dx_)));
+                            r_du2 = add(r_du2, mask(fma(dy_, dy_, mul(dx_, dx_))));
                         }
                         r_u2 = add(r_u2, u2);
-                        r_ux = add(r_ux, urx);
+                        r_ux = add(r_ux, mask(urx));
                         r_umax2 = fmaxf(r_umax2, fmaxf(lo(u2), hi(u2)));
                     }
                     if (save_u) {
                         C* up_ = a.uprev + ctl.base + ibase + o;
-                        store_pair(up_, urx);
-                        store_pair(up_ + PL, ury);
+                        st(up_, urx);
+                        st(up_ + PL, ury);
                     }
                 }
                 }  // not the fields pass
@@ -785,12 +856,12 @@ constexpr int kMarchW = 128;  // columns per CTA (one strip)
 //    with pressure-driven ends one row at a time is faster (2048 x 1000: 53.8 against 56.4).
 constexpr int kMarchK = 7;  // shared-memory row slots
 
-template <typename T, typename C, int SMODE, int BND = 0, int SCHEME = 0, bool FIELDS = false>
+template <typename T, typename C, int SMODE, int BND = 0, int SCHEME = 0, bool FIELDS = false, int STRIP = 0>
 cudaError_t launch_step_march(const CUtensorMap& map, const StepArgs<T, C>& a, const MarchCtl& ctl, int grid,
                               cudaStream_t s) {
     constexpr int K = kMarchK;
-    auto k = k_step_march<T, C, SMODE, kMarchW, K, BND, SCHEME, FIELDS>;
-    const size_t smem = march_smem_bytes<T, C, kMarchW, K>();
+    auto k = k_step_march<T, C, SMODE, kMarchW, K, BND, SCHEME, FIELDS, STRIP>;
+    const size_t smem = march_smem_bytes<T, C, kMarchW, K, STRIP == kOdd>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
@@ -798,21 +869,26 @@ cudaError_t launch_step_march(const CUtensorMap& map, const StepArgs<T, C>& a, c
     return cudaGetLastError();
 }
 
-template <typename T, typename C, int SMODE, int BND = 0, int SCHEME = 0>
+template <typename T, typename C, int SMODE, int BND = 0, int SCHEME = 0, int STRIP = 0>
 cudaError_t march_occupancy(int* blocks_per_sm) {
     constexpr int K = kMarchK;
-    auto k = k_step_march<T, C, SMODE, kMarchW, K, BND, SCHEME>;
-    const size_t smem = march_smem_bytes<T, C, kMarchW, K>();
+    auto k = k_step_march<T, C, SMODE, kMarchW, K, BND, SCHEME, false, STRIP>;
+    const size_t smem = march_smem_bytes<T, C, kMarchW, K, STRIP == kOdd>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, kMarchW / 2, smem);
 }
 }  // namespace lbk
-// Every variant (storage type, stress mode, boundary, scheme) of the kernel.
-#define LB_MARCH_FIELDS_ALL(X)                                                                      \
-    X(float, 0, 0, 0) X(float, 1, 0, 0) X(float, 0, 1, 0) X(float, 1, 1, 0) X(float, 0, 2, 0) X(float, 1, 2, 0) \
-    X(float, 0, 0, 1) X(float, 0, 0, 3) X(float, 1, 0, 3)                                               \
-    X(__nv_bfloat16, 0, 0, 0) X(__nv_bfloat16, 1, 0, 0) X(__nv_bfloat16, 0, 1, 0) X(__nv_bfloat16, 1, 1, 0) \
-    X(__nv_bfloat16, 0, 2, 0) X(__nv_bfloat16, 1, 2, 0) X(__nv_bfloat16, 0, 0, 1) X(__nv_bfloat16, 0, 0, 3) \
-    X(__nv_bfloat16, 1, 0, 3)
+// Every variant (stress mode, boundary, scheme) of the kernel for storage type T; X(T, SMODE, BND, SCHEME).
+#define LB_MARCH_VARIANTS(X, T)                                                          \
+    X(T, 0, 0, 0) X(T, 1, 0, 0) X(T, 0, 1, 0) X(T, 1, 1, 0) X(T, 0, 2, 0) X(T, 1, 2, 0) \
+    X(T, 0, 0, 1) X(T, 0, 0, 3) X(T, 1, 0, 3)
+// Its instantiations for steps (with the occupancy query) and for the fields pass.
+#define LB_MARCH_STEP(PREFIX, T, SMODE, BND, SCHEME, STRIP)                                                                  \
+    PREFIX template cudaError_t launch_step_march<T, float, SMODE, BND, SCHEME, false, STRIP>(                              \
+        const CUtensorMap&, const StepArgs<T, float>&, const MarchCtl&, int, cudaStream_t);                                \
+    PREFIX template cudaError_t march_occupancy<T, float, SMODE, BND, SCHEME, STRIP>(int*);
+#define LB_MARCH_FIELDS(PREFIX, T, SMODE, BND, SCHEME, STRIP)                                                                \
+    PREFIX template cudaError_t launch_step_march<T, float, SMODE, BND, SCHEME, true, STRIP>(                               \
+        const CUtensorMap&, const StepArgs<T, float>&, const MarchCtl&, int, cudaStream_t);
