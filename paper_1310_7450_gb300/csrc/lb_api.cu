@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "lb_step_march.cuh"
+#include "lb_step_resident.cuh"
 #include "lb_step_tile.cuh"
 #include "lb_sweep.cuh"
 #include "lb_sweep_smem.cuh"
@@ -96,6 +97,9 @@ LB_SWEEP_SMEM_EXTERN(double, double, 4)
     LB_MARCH_STEP(extern, T, SMODE, BND, SCHEME, kOdd) LB_MARCH_FIELDS(extern, T, SMODE, BND, SCHEME, kOdd)
 LB_MARCH_VARIANTS(X, float)
 LB_MARCH_VARIANTS(X, __nv_bfloat16)
+#undef X
+#define X(T, C, SMODE, NT) LB_RESIDENT(extern, T, C, SMODE, NT)
+LB_RESIDENT_VARIANTS(X)
 #undef X
 }  // namespace lbk
 
@@ -321,6 +325,7 @@ struct NvtxRange {
 };
 
 constexpr unsigned long long kDefaultWaitNs = 2000000000ull;
+constexpr long kResidentSteps = 6;
 
 struct lb_handle {
     int dev = 0;
@@ -399,6 +404,9 @@ struct lb_handle {
     MarchItem* march_items_d = nullptr;
     int* march_item_begin_d = nullptr;  // {0, n_march_items}: the residual reduction's item range
     int n_march_items = 0, march_grid = 0;
+    // resident stepping of a small single channel: CTAs of its cluster (0: not used), threads, shared memory
+    int res_cl = 0, res_threads = 0;
+    size_t res_smem = 0;
     // CUDA graphs of kGraphSteps plain tile-kernel steps, one per input buffer (an even count of
     // steps leaves the buffers where they were, so each graph starts from the buffer it names)
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
@@ -467,6 +475,16 @@ std::vector<ChanParams<C>> make_chan(const lb_handle* h) {
             q.rho_in = (C)((p.rho0 - 1.0) + 1.5 * p.g_x * (double)(h->nx + 1));
             q.rho_out = (C)((p.rho0 - 1.0) - 1.5 * p.g_x * (double)(h->nx + 1));
         }
+        q.tau_c = C(0.5) * q.tau * q.inv_gc;
+        q.cDh = C(0.5) * q.cD;
+        q.m15k = C(-1.5) * q.kdr;
+        q.om3 = C(3) * q.omega;
+        q.om15 = C(-1.5) * q.omega;
+        q.om45 = C(4.5) * q.omega;
+        q.k23 = C(3) * q.k2;
+        q.k245 = C(4.5) * q.k2;
+        q.k1h = C(0.5) * q.k1;
+        q.k12 = C(2) * q.k1;
         v[c] = q;
     }
     return v;
@@ -476,18 +494,24 @@ std::vector<ChanParams<C>> make_chan(const lb_handle* h) {
 // wide ones 32 x 8 tiles.  Row tiles are balanced: with ny >= 3 and a row target >= 4 every tile
 // gets between 2 and the target rows (one-sided differences at a wall need the two rows next to
 // it inside the tile or its halo), so a tile never holds more nodes than the CTA has threads.
-void plan_tiles(lb_handle* h) {
+// FP64 arithmetic: a tile's time is its SM's FP64 operations, so the row tiles are made more and shorter until their
+// number is the next multiple of the SMs (4 x 64: one tile -> 32; 256 x 257: 264 -> 304, two on every SM
+// instead of two on some).
+void plan_tiles(lb_handle* h, int n_sm) {
     h->items.clear();
     h->item_begin.assign(h->n_ch + 1, 0);
     int maxEX = 0, maxEY = 0;
+    int nxt = 32, nyt_target = kThreads / 32;
+    if (h->nx <= kThreads / 4) { nxt = h->nx; nyt_target = kThreads / h->nx; }
+    const int ntx = (h->nx + nxt - 1) / nxt;
+    long long total = 0;
+    for (int ny : h->ny) total += (long long)ntx * ((ny + nyt_target - 1) / nyt_target);
+    const double finer = h->csize == 8 ? (double)((total + n_sm - 1) / n_sm * n_sm) / (double)total : 1.0;
     for (int c = 0; c < h->n_ch; ++c) {
         h->item_begin[c] = (int)h->items.size();
         const int ny = h->ny[c];
-        int nxt, nyt_target;
-        if (h->nx <= kThreads / 4) { nxt = h->nx; nyt_target = kThreads / h->nx; }
-        else { nxt = 32; nyt_target = kThreads / 32; }
-        const int ntx = (h->nx + nxt - 1) / nxt;
-        const int nty = (ny + nyt_target - 1) / nyt_target;
+        const int base = (ny + nyt_target - 1) / nyt_target;
+        const int nty = std::max(base, std::min(ny / 2, (int)(base * finer)));
         for (int ty = 0; ty < nty; ++ty) {
             const int y0 = (int)((long long)ny * ty / nty), y1 = (int)((long long)ny * (ty + 1) / nty);
             for (int tx = 0; tx < ntx; ++tx) {
@@ -1003,6 +1027,54 @@ cudaError_t launch_march(lb_handle* h, const StepArgs<T, C>& a) {
         return cudaErrorNotSupported;
 }
 
+// The resident kernel of a handle's types and thread count: f(stress mode, NT) as constants.
+template <typename T, typename F>
+cudaError_t resident_variant(const lb_handle* h, int threads, F&& f) {
+    auto with_mode = [&](auto nt) { return h->smode ? f(Num<1>{}, nt) : f(Num<0>{}, nt); };
+    if constexpr (std::is_same<T, double>::value) {
+        return with_mode(Num<128>{});
+    } else {
+        if (threads <= 128) return with_mode(Num<128>{});
+        if (threads <= 320) return with_mode(Num<320>{});
+        return with_mode(Num<640>{});
+    }
+}
+template <typename T, typename C>
+constexpr bool kResidentTypes = std::is_same<T, C>::value || std::is_same<T, __nv_bfloat16>::value;
+
+// Whether runs of plain steps of this handle stay on chip (lb_step_resident.cuh): one channel of the paper's
+// scheme that a cluster can hold with one node per thread, and where that is the faster way.
+void plan_resident(lb_handle* h) {
+    h->res_cl = 0;
+    if (h->n_ch != 1 || h->march || h->scheme != 0 || h->gpbc || (h->flags & (LB_GRID_TILE_ONLY | LB_GRID_NO_GRAPH)) ||
+        ((h->flags & LB_GRID_BF16_STOCHASTIC) && h->prec == LB_PREC_BF16))
+        return;
+    const int nx = h->nx, ny = h->ny[0];
+    with_types(h->prec, [&](auto tt, auto tc) {
+        LB_TYPES(tt, tc);
+        if constexpr (kResidentTypes<T, C>) {
+            const int most = std::is_same<T, double>::value ? 128 : 640;  // threads of a CTA, see lb_step_resident.cuh
+            for (int cl : {16, 8, 4, 2, 1}) {
+                if (ny / cl < 2 || (long long)nx * ny > 1 << 20) continue;
+                const int threads = resident_threads(ny, nx, cl);
+                const size_t smem = resident_smem<T, C>(ny, nx, cl);
+                if (threads > most || smem > 227 * 1024) continue;
+                int clusters = 0;
+                const cudaError_t e = resident_variant<T>(h, threads, [&](auto sm, auto nt) {
+                    return resident_capacity<T, C, decltype(sm)::value, decltype(nt)::value>(cl, threads, smem, &clusters);
+                });
+                if (e != cudaSuccess) (void)cudaGetLastError();
+                if (e != cudaSuccess || clusters < 1) continue;
+                h->res_cl = cl;
+                h->res_threads = threads;
+                h->res_smem = smem;
+                break;
+            }
+        }
+        return 0;
+    });
+}
+
 constexpr int kGraphSteps = 32;  // steps per captured graph (even)
 
 // Capture kGraphSteps plain steps (no velocity save, no residual, no stochastic rounding) starting
@@ -1048,9 +1120,27 @@ template <typename T, typename C>
 lb_status run_steps(lb_handle* h, long n) {
     const bool sr = (h->flags & LB_GRID_BF16_STOCHASTIC) && h->prec == LB_PREC_BF16;
     long s = 1;
+    // A small single channel takes its plain steps on chip, many per launch (the last two of the call, with the
+    // velocity save and the residual, follow one by one); at least kResidentSteps, since a launch costs the time
+    // of a few steps, at most 65536, so that no launch lasts longer than a fraction of a second.
+    if (h->res_cl > 0) {
+        if constexpr (kResidentTypes<T, C>) {
+            while (n - s + 1 >= kResidentSteps + 2) {
+                const long run = std::min(n - s + 1 - 2, 65536L);
+                StepArgs<T, C> a = base_args<T, C>(h);
+                a.flags = (h->flags & LB_GRID_STORE_SIGMA) ? F_STORE_SIGMA : 0;
+                LB_CK((resident_variant<T>(h, h->res_threads, [&](auto sm, auto nt) {
+                    return launch_step_resident<T, C, decltype(sm)::value, decltype(nt)::value>(
+                        a, (T*)h->popA, run, h->res_cl, h->res_threads, h->res_smem, h->stream);
+                })));
+                h->step += run;
+                s += run;
+            }
+        }
+    }
     // Runs of plain steps replay a captured graph; the last two steps of the call (velocity save,
     // residual) are always launched one by one.
-    if (!h->march && !sr && !(h->flags & LB_GRID_NO_GRAPH)) {
+    if (!h->march && h->res_cl == 0 && !sr && !(h->flags & LB_GRID_NO_GRAPH)) {
         while (n - s + 1 >= kGraphSteps + 2) {
             int slot = h->gexec_pin[0] == h->popA ? 0 : (h->gexec_pin[1] == h->popA ? 1 : -1);
             if (slot < 0) {
@@ -1642,7 +1732,9 @@ lb_status lb_create(const lb_grid* grid, const lb_params* params, const lb_bound
         h->row_off[c] = h->gny;
         h->gny += h->ny[c];
     }
-    plan_tiles(h);
+    int n_sm = 0;
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->dev);
+    plan_tiles(h, std::max(1, n_sm));
 
     auto dmalloc = [&](void** p, size_t bytes) -> cudaError_t { return cudaMalloc(p, bytes < 16 ? 16 : bytes); };
     cudaError_t e;
@@ -1742,6 +1834,7 @@ lb_status lb_create(const lb_grid* grid, const lb_params* params, const lb_bound
     if (e != cudaSuccess) return bail(cuda_fail(e, "lb_create: init kernel"));
     st = plan_march(h);
     if (st != LB_OK) return bail(st);
+    plan_resident(h);
     *out = h;
     return LB_OK;
 }

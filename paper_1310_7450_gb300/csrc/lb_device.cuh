@@ -79,25 +79,24 @@ __device__ __forceinline__ uint32_t mix32(uint32_t x) {
     return x;
 }
 
-// Store the nine post-collision deviations d + D of one node (node = its index in the channel
-// planes).  BF16 storage with stochastic rounding draws 16 random bits per value from
-// mix32(key ^ (5 node + pair)); `key` changes every step.
+// Store the nine post-collision deviations of one node (node = its index in the channel planes).  BF16 storage
+// with stochastic rounding draws 16 random bits per value from mix32(key ^ (5 node + pair)); `key` changes
+// every step.
 template <typename T, typename C>
-__device__ __forceinline__ void store_node(T* po, long long P, const C (&d)[9], const C (&D)[9], bool sr, uint32_t key,
-                                           uint32_t node) {
+__device__ __forceinline__ void store_node(T* po, long long P, const C (&n)[9], bool sr, uint32_t key, uint32_t node) {
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
         if (sr) {
             uint32_t h = 0;
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
                 if ((i & 1) == 0) h = mix32(key ^ (node * 5u + (uint32_t)(i >> 1)));
-                po[(long long)i * P] = bf16_stochastic((float)(d[i] + D[i]), (i & 1) ? (h >> 16) : (h & 0xffffu));
+                po[(long long)i * P] = bf16_stochastic((float)n[i], (i & 1) ? (h >> 16) : (h & 0xffffu));
             }
             return;
         }
     }
 #pragma unroll
-    for (int i = 0; i < 9; ++i) Store<T>::st(po + (long long)i * P, d[i] + D[i]);
+    for (int i = 0; i < 9; ++i) Store<T>::st(po + (long long)i * P, n[i]);
 }
 
 // ---- launch descriptors ----------------------------------------------------------------------
@@ -130,6 +129,11 @@ struct ChanParams {
     C beta_rho; // scheme 3: tau(rho) = tau exp(beta_rho (rho - rho_ref) / rho_ref)
     C rho_ref;
     C tau_f;    // scheme 3: memory time of the fluidity 1/tau_M (0: Eq. nlmaxwell, instantaneous)
+    // products of the above that the FP64 arithmetic would otherwise form at every node
+    C tau_c;                // tau / (2 gamma_c)
+    C cDh, m15k;            // cD / 2, -1.5 kdr
+    C om3, om15, om45;      // 3 omega, -1.5 omega, 4.5 omega
+    C k23, k245, k1h, k12;  // 3 k2, 4.5 k2, k1 / 2, 2 k1
 };
 
 struct WorkItem {
@@ -202,22 +206,46 @@ __device__ __forceinline__ void store_fields(const StepArgs<T, C>& a, long long 
 
 // ---- per-node arithmetic -------------------------------------------------------------------
 
-// Division and square root: exact IEEE operations in FP64 (the parity mode); in FP32 the PTX
-// approximations rcp.approx.ftz and rsqrt.approx.ftz (one hardware instruction each, about 1 ulp;
-// the .ftz forms skip the subnormal handling) -- every denominator here is a density near 1 or a
-// positive quantity in the normal range, and the FP32 path's parity bound is 1e-5.  The square
-// root returns 0 below the smallest normal float: sqrt(x) < 1.1e-19 there, which no quantity it
+// Division and square root.  FP32: the PTX approximations rcp.approx.ftz and rsqrt.approx.ftz (one hardware
+// instruction each, about 1 ulp; the .ftz forms skip the subnormal handling) -- every denominator here is a
+// density near 1 or a positive quantity in the normal range, and the FP32 path's parity bound is 1e-5.  The
+// square root returns 0 below the smallest normal float: sqrt(x) < 1.1e-19 there, which no quantity it
 // enters (1 + tau sqrt(II)/gamma_c) can resolve.
+// FP64 (the parity mode): this part does two FP64 operations per SM and clock, and a chain of them waits about 60
+// clocks for each, so the library's division (8 operations and a range check) and square root weigh more than
+// anything else in a step.  The reciprocal starts from the hardware's approximation (relative error e <= 2^-23)
+// and takes one third-order step, y + y (e + e^2): 3 operations, 0.51 ulp.  A quotient is a product with it, corrected by its
+// residual (Markstein, IBM J. Res. Dev. 34, 1990); the square root is one Goldschmidt step on the
+// reciprocal square root and the same correction: 7 operations, within 1 ulp, 0 below the normal range.
 template <typename C> struct Arith;
 template <> struct Arith<double> {
-    static __device__ __forceinline__ double div(double a, double b) { return a / b; }
-    static __device__ __forceinline__ double sqrt(double x) { return ::sqrt(x); }
+    static __device__ __forceinline__ double rcp(double x) {
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+        const double e = __fma_rn(-x, y, 1.0);
+        return __fma_rn(y, __fma_rn(e, e, e), y);
+    }
+    static __device__ __forceinline__ double div(double a, double b) {
+        const double y = rcp(b), q = a * y;
+        return __fma_rn(__fma_rn(-b, q, a), y, q);
+    }
+    static __device__ __forceinline__ double sqrt(double x) {
+        double y;
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+        double g = x * y, h = 0.5 * y;
+        const double r = __fma_rn(-g, h, 0.5);
+        g = __fma_rn(g, r, g);
+        h = __fma_rn(h, r, h);
+        g = __fma_rn(__fma_rn(-g, g, x), h, g);
+        return x >= 2.2250738585072014e-308 ? g : (x >= 0.0 ? 0.0 : (double)NAN);
+    }
     static __device__ __forceinline__ double exp(double x) { return ::exp(x); }
 };
 #ifdef LBK_FP32_IEEE
 // Compile-time alternative: correctly rounded FP32 division and square root (IEEE round to
 // nearest even), for measuring what the approximations cost in parity and in throughput.
 template <> struct Arith<float> {
+    static __device__ __forceinline__ float rcp(float x) { return __frcp_rn(x); }
     static __device__ __forceinline__ float div(float a, float b) { return __fdiv_rn(a, b); }
     static __device__ __forceinline__ float sqrt(float x) { return __fsqrt_rn(x); }
     static __device__ __forceinline__ float exp(float x) { return expf(x); }
@@ -254,7 +282,7 @@ template <typename C>
 __device__ __forceinline__ void gradient_velocity(const C (&d)[9], C gx, C& dR, C& jx, C& jy, C& ux, C& uy) {
     moments<C>(d, dR, jx, jy);
     jx = jx + C(0.5) * gx;  // j = sum c n + f dt/2 (Eq. rhoj)
-    const C inv = Arith<C>::div(C(1), C(1) + dR);
+    const C inv = Arith<C>::rcp(C(1) + dR);
     ux = jx * inv;
     uy = jy * inv;
 }
@@ -328,6 +356,52 @@ struct NodeState {
     C ux, uy;          // velocity handed to n^eq and F_i: j / rho_eq
 };
 
+// The same in FP64 with as few operations as the formulas allow (60 instead of about 110: FP64 operations bound
+// every FP64 kernel).  With (K, B, Q, Y) = 2 kappa, the plain differences, and W = B + Q, the solution of
+// convected_solve needs only alpha B, alpha Q and their products; the factor 1/2 of P = (A + E)/2
+// cancels against those of the numerators.
+template <int SMODE, bool TAUM>
+__device__ __forceinline__ NodeState<double> constitutive64(const ChanParams<double>& P, double K, double B, double Q,
+                                                            double Y, double dR, double jx, double jy, double drho_prev,
+                                                            double so_xx, double so_xy, double so_yy, double tau_M) {
+    NodeState<double> r;
+    const double W = B + Q;
+    if constexpr (!TAUM) {
+        // sqrt(II_D) = sqrt(2 K^2 + 2 Y^2 + W^2) / 2
+        const double z = __fma_rn(2.0, __fma_rn(K, K, Y * Y), W * W);
+        tau_M = P.tau * Arith<double>::rcp(__fma_rn(P.tau_c, Arith<double>::sqrt(z), 1.0));
+    }
+    double al = tau_M, b1, b2, b3;  // right-hand side (xx, 2 xy, yy)
+    if constexpr (SMODE == 0) {
+        const double gt = P.G * al;
+        b1 = gt * K;
+        b2 = gt * W;
+        b3 = gt * Y;
+    } else {
+        al = tau_M * Arith<double>::rcp(tau_M + 1.0);
+        b1 = al * __fma_rn(P.G, K, so_xx);
+        b2 = al * __fma_rn(P.G, W, so_xy + so_xy);
+        b3 = al * __fma_rn(P.G, Y, so_yy);
+    }
+    const double A = __fma_rn(-al, K, 1.0), E = __fma_rn(-al, Y, 1.0), P2 = A + E;
+    const double aB = al * B, aQ = al * Q, q4 = aB * aQ, AE = A * E;
+    const double i = Arith<double>::rcp(P2 * (AE - q4));
+    r.sxy = i * __fma_rn(aB * A, b3, __fma_rn(aQ * E, b1, AE * b2));
+    r.sxx = i * __fma_rn(aB * aB, b3, __fma_rn(aB * E, b2, __fma_rn(P2, E, -q4) * b1));
+    r.syy = i * __fma_rn(aQ * aQ, b1, __fma_rn(aQ * A, b2, __fma_rn(P2, A, -q4) * b3));
+    const double Nxx = __fma_rn(P.cD, K, r.sxx), Nyy = __fma_rn(P.cD, Y, r.syy);
+    r.Bxy = __fma_rn(P.cDh, W, r.sxy);
+    r.drho = P.m15k * (Nxx + Nyy);
+    r.S = __fma_rn(-P.kdr, drho_prev, r.drho);
+    r.Bxx = Nxx - Nyy;  // twice the traceless part's xx: collide64 takes k1 / 2 with it (the schemes with a
+                        // collision of their own have k1 = 0)
+    r.dReq = __fma_rn(0.5, r.S, dR);
+    const double inv = Arith<double>::rcp(1.0 + r.dReq);
+    r.ux = jx * inv;
+    r.uy = jy * inv;
+    return r;
+}
+
 // TAUM = true: the relaxation time comes in as tau_M_in (the relaxation-time extensions of
 // scheme 3) instead of Eq. (nlmaxwell) with the channel's tau.
 template <typename C, int SMODE, bool TAUM = false>
@@ -368,6 +442,22 @@ __device__ __forceinline__ NodeState<C> constitutive(const ChanParams<C>& P, C k
     r.uy = jy * inv;
     return r;
 }
+
+// The same from the doubled differences 2 kappa, in each arithmetic type's own form.
+template <typename C, int SMODE, bool TAUM = false>
+__device__ __forceinline__ NodeState<C> constitutive2(const ChanParams<C>& P, C K, C B, C Q, C Y, C dR, C jx, C jy,
+                                                      C drho_prev, C so_xx, C so_xy, C so_yy, C tau_M = C(0)) {
+    if constexpr (sizeof(C) == 8)
+        return constitutive64<SMODE, TAUM>(P, K, B, Q, Y, dR, jx, jy, drho_prev, so_xx, so_xy, so_yy, tau_M);
+    else
+        return constitutive<C, SMODE, TAUM>(P, C(0.5) * K, C(0.5) * B, C(0.5) * Q, C(0.5) * Y, dR, jx, jy, drho_prev, so_xx,
+                                            so_xy, so_yy, tau_M);
+}
+// Doubled one-sided differences of the first row (-3 u0 + 4 u1 - u2) and the last (3 u0 - 4 u1 + u2).
+template <typename C>
+__device__ __forceinline__ C first_row_difference(C u0, C u1, C u2) { return C(-3) * u0 + C(4) * u1 - u2; }
+template <typename C>
+__device__ __forceinline__ C last_row_difference(C u0, C u1, C u2) { return C(3) * u0 - C(4) * u1 + u2; }
 
 // Scheme 1 (generalized Newtonian, the first alternative of Sec. II C): a locally Newtonian fluid
 // whose viscosity is the model's effective viscosity in steady shear, eta_eff = G tau_M + eta_inf,
@@ -500,9 +590,59 @@ __device__ __forceinline__ void collide_impl(const ChanParams<C>& P, const NodeS
     D[0] = s.S - (((D[1] + D[2]) + (D[3] + D[4])) + ((D[5] + D[6]) + (D[7] + D[8])));
 }
 
+// The new populations of the paper's scheme in FP64: collide_impl with the constants multiplied out, the squares of
+// the diagonal velocities from u^2 and u_x u_y, and the three closures on the new populations themselves (mass
+// dR + S, momentum j + f/2 with j of Eq. rhoj), so that no increment is formed.  Takes constitutive64's state; 70
+// operations instead of about 115.
+__device__ __forceinline__ void collide64(const ChanParams<double>& P, const NodeState<double>& s, const double (&d)[9],
+                                          double dR, double jx, double jy, double (&n)[9]) {
+    const double ux = s.ux, uy = s.uy, gx = P.gx, rq = 1.0 + s.dReq, keep = 1.0 - P.omega;
+    const double x2 = ux * ux, usq = __fma_rn(uy, uy, x2), y2 = uy * uy, xy = ux * uy;
+    const double sux = -s.S * ux, suy = -s.S * uy;
+    const double Yxx = __fma_rn(sux, ux, (gx + gx) * ux), Yxy = __fma_rn(uy, gx, sux * uy);
+    const double sumY = __fma_rn(suy, uy, Yxx);
+    const double ntr = sumY * (-1.0 / 3.0), t2 = sumY * (2.0 / 3.0);
+    const double o3 = P.om3 * rq, o45 = P.om45 * rq, kg3 = P.k23 * gx;
+    const double base = __fma_rn(P.k2, s.S, __fma_rn(P.om15 * rq, usq, P.omega * s.dReq));
+    const double w1 = 1.0 / 9.0, w5 = 1.0 / 36.0;
+    {
+        const double E = __fma_rn(P.k1h, s.Bxx, __fma_rn(P.k245, Yxx + ntr, __fma_rn(o45, x2, base)));
+        n[1] = __fma_rn(w1, E + __fma_rn(o3, ux, kg3), keep * d[1]);
+    }
+    {
+        const double E = __fma_rn(-P.k1h, s.Bxx, __fma_rn(P.k245, __fma_rn(suy, uy, ntr), __fma_rn(o45, y2, base)));
+        n[2] = __fma_rn(w1, __fma_rn(o3, uy, E), keep * d[2]);
+    }
+    {
+        const double E = __fma_rn(P.k12, s.Bxy, __fma_rn(P.k245, __fma_rn(2.0, Yxy, t2), __fma_rn(o45, __fma_rn(2.0, xy, usq), base)));
+        const double O = __fma_rn(o3, ux + uy, kg3);
+        n[5] = __fma_rn(w5, E + O, keep * d[5]);
+        n[7] = __fma_rn(w5, E - O, keep * d[7]);
+    }
+    {
+        const double E = __fma_rn(-P.k12, s.Bxy, __fma_rn(P.k245, __fma_rn(-2.0, Yxy, t2), __fma_rn(o45, __fma_rn(-2.0, xy, usq), base)));
+        const double O = __fma_rn(o3, ux - uy, kg3);
+        n[8] = __fma_rn(w5, E + O, keep * d[8]);
+        n[6] = __fma_rn(w5, E - O, keep * d[6]);
+    }
+    const double n57 = n[5] - n[7], n86 = n[8] - n[6];
+    n[3] = (n[1] + n57) + (n86 - __fma_rn(0.5, gx, jx));
+    n[4] = (n[2] + n57) - (n86 + jy);
+    n[0] = (dR + s.S) - (((n[1] + n[2]) + (n[3] + n[4])) + ((n[5] + n[7]) + (n[8] + n[6])));
+}
+
+// The new populations of a node, paper's scheme.
 template <typename C>
-__device__ __forceinline__ void collide_node(const ChanParams<C>& P, const NodeState<C>& s, const C (&d)[9], C (&D)[9]) {
-    collide_impl<C, false>(P, s, d, D, P.omega, P.k2, P.gx, C(0));
+__device__ __forceinline__ void collide_node(const ChanParams<C>& P, const NodeState<C>& s, const C (&d)[9], C dR, C jx, C jy,
+                                             C (&n)[9]) {
+    if constexpr (sizeof(C) == 8) {
+        collide64(P, s, d, dR, jx, jy, n);
+    } else {
+        C D[9];
+        collide_impl<C, false>(P, s, d, D, P.omega, P.k2, P.gx, C(0));
+#pragma unroll
+        for (int i = 0; i < 9; ++i) n[i] = d[i] + D[i];
+    }
 }
 
 // |u| <= guard for the reported velocity j/rho_h without a division or square root (false for NaN).

@@ -698,14 +698,15 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                 T* po = a.pout + 8 * ctl.base;
                 if (sr) {
                     const uint32_t node = (uint32_t)((long long)y * nx + x0 + col0);
-                    C d0[9], d1[9], D0[9], D1[9];
+                    C n0[9], n1[9];
 #pragma unroll
                     for (int i = 0; i < 9; ++i) {
-                        d0[i] = lo(dcur[i]); d1[i] = hi(dcur[i]);
-                        D0[i] = lo(D[i]); D1[i] = hi(D[i]);
+                        const P2 v = add(dcur[i], D[i]);
+                        n0[i] = lo(v);
+                        n1[i] = hi(v);
                     }
-                    if (own0) store_node<T, C>(field_at(po, o, vo), PL, d0, D0, true, a.sr_key, node);
-                    if (own1) store_node<T, C>(field_at(po, o, vo) + 1, PL, d1, D1, true, a.sr_key, node + 1);
+                    if (own0) store_node<T, C>(field_at(po, o, vo), PL, n0, true, a.sr_key, node);
+                    if (own1) store_node<T, C>(field_at(po, o, vo) + 1, PL, n1, true, a.sr_key, node + 1);
                 } else {
 #pragma unroll
                     for (int i = 0; i < 9; ++i) st_pop(field_at(po + i * PL, o, vo), add(dcur[i], D[i]));

@@ -112,7 +112,9 @@ __global__ void __launch_bounds__(NT) k_step_tile(const StepArgs<T, C> a) {
     }
     // phase 2: halo ring (rows y0-1 and y0+nyt; columns x0-1 and x0+nxt for split tiles)
     const int R = 2 * EX + (full ? 0 : 2 * it.nyt);
-    for (int r = t; r < R; r += NT) {
+    // (from the first warp without own nodes on: in a small tile those warps run beside the own nodes' warps)
+    const int own32 = (ntile + 31) / 32 * 32;
+    for (int r = t >= own32 ? t - own32 : t + max(NT - own32, 0); r < R; r += NT) {
         int ex, ey;
         if (r < EX) { ex = r; ey = 0; }
         else if (r < 2 * EX) { ex = r - EX; ey = EY - 1; }
@@ -140,27 +142,28 @@ __global__ void __launch_bounds__(NT) k_step_tile(const StepArgs<T, C> a) {
         if (full) { exm = ecx == 0 ? EX - 1 : ecx - 1; exp_ = ecx == EX - 1 ? 0 : ecx + 1; }
         else { exm = ecx - 1; exp_ = ecx + 1; }
         const C* rowc = su + 2 * (ecy * EX);
-        const C ka = C(0.5) * (rowc[2 * exp_] - rowc[2 * exm]);          // d_x u_x
-        const C kc = C(0.5) * (rowc[2 * exp_ + 1] - rowc[2 * exm + 1]);  // d_x u_y
-        C kb, ke;
+        const C K = rowc[2 * exp_] - rowc[2 * exm];          // 2 d_x u_x
+        const C Q = rowc[2 * exp_ + 1] - rowc[2 * exm + 1];  // 2 d_x u_y
+        C B, Y;
         if (y == 0) {
             const C* r1 = su + 2 * ((ecy + 1) * EX + ecx);
             const C* r2 = su + 2 * ((ecy + 2) * EX + ecx);
             const C* r0 = su + 2 * (ecy * EX + ecx);
-            kb = C(0.5) * (C(-3) * r0[0] + C(4) * r1[0] - r2[0]);
-            ke = C(0.5) * (C(-3) * r0[1] + C(4) * r1[1] - r2[1]);
+            B = first_row_difference<C>(r0[0], r1[0], r2[0]);
+            Y = first_row_difference<C>(r0[1], r1[1], r2[1]);
         } else if (y == ny - 1) {
             const C* r1 = su + 2 * ((ecy - 1) * EX + ecx);
             const C* r2 = su + 2 * ((ecy - 2) * EX + ecx);
             const C* r0 = su + 2 * (ecy * EX + ecx);
-            kb = C(0.5) * (C(3) * r0[0] - C(4) * r1[0] + r2[0]);
-            ke = C(0.5) * (C(3) * r0[1] - C(4) * r1[1] + r2[1]);
+            B = last_row_difference<C>(r0[0], r1[0], r2[0]);
+            Y = last_row_difference<C>(r0[1], r1[1], r2[1]);
         } else {
             const C* rp = su + 2 * ((ecy + 1) * EX + ecx);
             const C* rm = su + 2 * ((ecy - 1) * EX + ecx);
-            kb = C(0.5) * (rp[0] - rm[0]);
-            ke = C(0.5) * (rp[1] - rm[1]);
+            B = rp[0] - rm[0];
+            Y = rp[1] - rm[1];
         }
+        const C ka = C(0.5) * K, kb = C(0.5) * B, kc = C(0.5) * Q, ke = C(0.5) * Y;  // (the schemes that take kappa)
         const long long pn = (long long)y * nx + x;  // node inside the channel planes
         C* dr = a.drho + P.base;
         const C drho_prev = dr[pn];
@@ -180,10 +183,10 @@ __global__ void __launch_bounds__(NT) k_step_tile(const StepArgs<T, C> a) {
         } else if constexpr (SCHEME == 3) {
             double phi_new;
             const C tau_M = relaxation_time_ext<C>(P, ka, kb, kc, ke, dR, drho_prev, a.phi[P.base + pn], &phi_new);
-            s = constitutive<C, SMODE, true>(P, ka, kb, kc, ke, dR, jx, jy, drho_prev, so_xx, so_xy, so_yy, tau_M);
+            s = constitutive2<C, SMODE, true>(P, K, B, Q, Y, dR, jx, jy, drho_prev, so_xx, so_xy, so_yy, tau_M);
             if (!(a.flags & F_FIELDS) && P.tau_f > C(0)) a.phi[P.base + pn] = phi_new;  // own node only
         } else {
-            s = constitutive<C, SMODE>(P, ka, kb, kc, ke, dR, jx, jy, drho_prev, so_xx, so_xy, so_yy);
+            s = constitutive2<C, SMODE>(P, K, B, Q, Y, dR, jx, jy, drho_prev, so_xx, so_xy, so_yy);
         }
         if (SCHEME == 2 && (a.flags & F_SNN)) {
             // scheme 2, first pass: Sigma^nN = sigma + (eta_inf - eta^N) D of every node of this step
@@ -211,7 +214,7 @@ __global__ void __launch_bounds__(NT) k_step_tile(const StepArgs<T, C> a) {
             fy += fny;
             jx += C(0.5) * fnx;
             jy += C(0.5) * fny;
-            const C inv = Arith<C>::div(C(1), C(1) + s.dReq);
+            const C inv = Arith<C>::rcp(C(1) + s.dReq);
             s.ux = jx * inv;
             s.uy = jy * inv;
         }
@@ -229,11 +232,19 @@ __global__ void __launch_bounds__(NT) k_step_tile(const StepArgs<T, C> a) {
         if (a.flags & F_FIELDS) {
             store_fields<C>(a, P.node_off + pn, urx, ury, s.sxx, s.syy, s.sxy, rho_h);
         } else {
-            C D[9];
-            if constexpr (SCHEME != 0) collide_impl<C, true>(P, s, d, D, om, k2, fx, fy);
-            else collide_node<C>(P, s, d, D);
+            C n[9];
+            // (the relaxation-time extensions collide as the paper's scheme does; their FP32 variant through the general
+            // form, as the row-march variant was matched to it)
+            if constexpr (SCHEME == 0 || (SCHEME == 3 && sizeof(C) == 8)) {
+                collide_node<C>(P, s, d, dR, jx, jy, n);
+            } else {
+                C D[9];
+                collide_impl<C, true>(P, s, d, D, om, k2, fx, fy);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) n[i] = d[i] + D[i];
+            }
             T* po = a.pout + 9 * P.base + pn;
-            store_node<T, C>(po, P.P, d, D, (a.flags & F_SR) != 0, a.sr_key ^ (uint32_t)(it.ch * 0x9E3779B9u), (uint32_t)pn);
+            store_node<T, C>(po, P.P, n, (a.flags & F_SR) != 0, a.sr_key ^ (uint32_t)(it.ch * 0x9E3779B9u), (uint32_t)pn);
             dr[pn] = s.drho;
             if (SMODE == 1) {
                 C* s3 = a.sig3 + 3 * P.base;

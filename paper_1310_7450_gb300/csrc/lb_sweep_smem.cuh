@@ -130,30 +130,30 @@ __global__ void __launch_bounds__(NT, sizeof(C) == 8 ? 1 : 512 / NT) k_sweep_sme
                 const int y = y0 + e / nx, x = e % nx;
                 const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
                 const C* row = su + 2 * ((y - ey0) * nx);
-                const C ka = C(0.5) * (row[2 * xp] - row[2 * xm]);
-                const C kc = C(0.5) * (row[2 * xp + 1] - row[2 * xm + 1]);
-                C kb, ke;
+                const C K = row[2 * xp] - row[2 * xm];
+                const C Q = row[2 * xp + 1] - row[2 * xm + 1];
+                C B, Y;
                 if (y == 0) {
                     const C* r1p = row + 2 * nx;
                     const C* r2p = row + 4 * nx;
-                    kb = C(0.5) * (C(-3) * row[2 * x] + C(4) * r1p[2 * x] - r2p[2 * x]);
-                    ke = C(0.5) * (C(-3) * row[2 * x + 1] + C(4) * r1p[2 * x + 1] - r2p[2 * x + 1]);
+                    B = first_row_difference<C>(row[2 * x], r1p[2 * x], r2p[2 * x]);
+                    Y = first_row_difference<C>(row[2 * x + 1], r1p[2 * x + 1], r2p[2 * x + 1]);
                 } else if (y == ny - 1) {
                     const C* r1m = row - 2 * nx;
                     const C* r2m = row - 4 * nx;
-                    kb = C(0.5) * (C(3) * row[2 * x] - C(4) * r1m[2 * x] + r2m[2 * x]);
-                    ke = C(0.5) * (C(3) * row[2 * x + 1] - C(4) * r1m[2 * x + 1] + r2m[2 * x + 1]);
+                    B = last_row_difference<C>(row[2 * x], r1m[2 * x], r2m[2 * x]);
+                    Y = last_row_difference<C>(row[2 * x + 1], r1m[2 * x + 1], r2m[2 * x + 1]);
                 } else {
-                    kb = C(0.5) * (row[2 * nx + 2 * x] - row[-2 * nx + 2 * x]);
-                    ke = C(0.5) * (row[2 * nx + 2 * x + 1] - row[-2 * nx + 2 * x + 1]);
+                    B = row[2 * nx + 2 * x] - row[-2 * nx + 2 * x];
+                    Y = row[2 * nx + 2 * x + 1] - row[-2 * nx + 2 * x + 1];
                 }
-                const NodeState<C> st = constitutive<C, 0>(P, ka, kb, kc, ke, dR[k], jx[k], jy[k], drv[k], C(0), C(0), C(0));
+                const NodeState<C> st = constitutive2<C, 0>(P, K, B, Q, Y, dR[k], jx[k], jy[k], drv[k], C(0), C(0), C(0));
                 const C rho_h = C(1) + st.dReq - st.drho;
                 if (!velocity_ok<C>(jx[k], jy[k], rho_h, (C)0.3)) atomicOr(a.status + ch, 1);
-                C D[9];
-                collide_node<C>(P, st, d[k], D);
+                C nw[9];
+                collide_node<C>(P, st, d[k], dR[k], jx[k], jy[k], nw);
                 const long long pn = (long long)y * nx + x;
-                store_node<T, C>(nxt + (y - yb) * nx + x, PS, d[k], D, a.sr,
+                store_node<T, C>(nxt + (y - yb) * nx + x, PS, nw, a.sr,
                                  mix32(a.sr_key ^ (uint32_t)(s * 0x9E3779B9ull) ^ (uint32_t)(ch * 0x85EBCA6Bu)), (uint32_t)pn);
                 drv[k] = st.drho;
                 if (save) {
