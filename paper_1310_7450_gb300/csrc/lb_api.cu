@@ -23,6 +23,7 @@
 #include "lb_step_resident.cuh"
 #include "lb_step_tile.cuh"
 #include "lb_sweep.cuh"
+#include "lb_sweep_pair.cuh"
 #include "lb_sweep_smem.cuh"
 #include "lbnlm.h"
 
@@ -84,13 +85,12 @@ LB_SWEEP_EXTERN(double, double, 4)
     extern template cudaError_t launch_sweep_smem<T, C, 256, 4, NX>(const SweepArgs<T, C>&, int, int, size_t, cudaStream_t); \
     extern template cudaError_t launch_sweep_smem_capacity<T, C, 128, 4, NX>(int, size_t, int*);                            \
     extern template cudaError_t launch_sweep_smem_capacity<T, C, 256, 4, NX>(int, size_t, int*);
-LB_SWEEP_SMEM_EXTERN(float, float, 0)
-LB_SWEEP_SMEM_EXTERN(__nv_bfloat16, float, 0)
 LB_SWEEP_SMEM_EXTERN(double, double, 0)
-LB_SWEEP_SMEM_EXTERN(float, float, 4)
-LB_SWEEP_SMEM_EXTERN(__nv_bfloat16, float, 4)
 LB_SWEEP_SMEM_EXTERN(double, double, 4)
 #undef LB_SWEEP_SMEM_EXTERN
+#define X(T, NT, NX) LB_SWEEP_PAIR(extern, T, NT, NX)
+LB_SWEEP_PAIR_VARIANTS(X)
+#undef X
 #define X(T, SMODE, BND, SCHEME)                                                                              \
     LB_MARCH_STEP(extern, T, SMODE, BND, SCHEME, kFull) LB_MARCH_FIELDS(extern, T, SMODE, BND, SCHEME, kFull) \
     LB_MARCH_STEP(extern, T, SMODE, BND, SCHEME, kPart) LB_MARCH_FIELDS(extern, T, SMODE, BND, SCHEME, kPart) \
@@ -1276,13 +1276,20 @@ size_t sweep_smem(const lb_handle* h, int ny_max, int cl) {
 // and its rows, halos and velocity rows fit the 227 KB of one CTA.
 size_t sweep_smem_resident(const lb_handle* h, int ny_max, int cl) {
     const int rows = (ny_max + cl - 1) / cl;
-    const size_t pops = ((size_t)2 * 9 * (rows + 6) * h->nx * h->tsize + 15) / 16 * 16;
-    return pops + (size_t)(rows + 4) * h->nx * 2 * h->csize;
+    if (h->csize == 4) return h->tsize == 2 ? sweep_pair_smem<__nv_bfloat16>(rows, h->nx) : sweep_pair_smem<float>(rows, h->nx);
+    return sweep_smem_bytes<double, double>(rows, h->nx);
 }
 bool sweep_config_fits(const lb_handle* h, const SweepGroup& g, int var, int nt, int cl) {
     if (cl < 1 || cl > 16 || (nt != 128 && nt != 256) || !sweep_fits(g.ny_max, h->nx, nt, cl)) return false;
     if (var == 0) return sweep_smem(h, g.ny_max, cl) <= 200 * 1024;
     return g.ny_min / cl >= 3 && sweep_smem_resident(h, g.ny_max, cl) <= 227 * 1024;
+}
+
+// Threads and width of a resident sweep kernel as constants.
+template <typename F>
+cudaError_t sweep_variant(const lb_handle* h, int nt, F&& f) {
+    if (h->nx == 4) return nt == 128 ? f(Num<128>{}, Num<4>{}) : f(Num<256>{}, Num<4>{});
+    return nt == 128 ? f(Num<128>{}, Num<0>{}) : f(Num<256>{}, Num<0>{});
 }
 
 template <typename T, typename C>
@@ -1306,12 +1313,11 @@ cudaError_t sweep_launch(lb_handle* h, const SweepGroup& g, int var, int nt, int
     a.sr_key = step_key(h, h->step + 0x5bd1e995ll);
     if (var == 1) {
         const size_t smem = sweep_smem_resident(h, g.ny_max, cl);
-        if (h->nx == 4) {  // the 4-column channels of the batched sweep: width known at compile time
-            if (nt == 128) return launch_sweep_smem<T, C, 128, kSweepNPT, 4>(a, g.count, cl, smem, stream);
-            return launch_sweep_smem<T, C, 256, kSweepNPT, 4>(a, g.count, cl, smem, stream);
-        }
-        if (nt == 128) return launch_sweep_smem<T, C, 128, kSweepNPT>(a, g.count, cl, smem, stream);
-        return launch_sweep_smem<T, C, 256, kSweepNPT>(a, g.count, cl, smem, stream);
+        return sweep_variant(h, nt, [&](auto threads, auto width) {  // (4 columns: width known at compile time)
+            constexpr int NT = decltype(threads)::value, NX = decltype(width)::value;
+            if constexpr (std::is_same<C, float>::value) return launch_sweep_pair<T, NT, kSweepPairs, NX>(a, g.count, cl, smem, stream);
+            else return launch_sweep_smem<T, C, NT, kSweepNPT, NX>(a, g.count, cl, smem, stream);
+        });
     }
     const size_t smem = sweep_smem(h, g.ny_max, cl);
     if (h->nx == 4) {
@@ -1340,11 +1346,11 @@ int sweep_capacity(lb_handle* h, const SweepGroup& g, int var, int nt, int cl) {
         else {
             if (var == 1) {
                 const size_t smem = sweep_smem_resident(h, g.ny_max, cl);
-                if (h->nx == 4)
-                    return nt == 128 ? launch_sweep_smem_capacity<T, C, 128, kSweepNPT, 4>(cl, smem, &n)
-                                     : launch_sweep_smem_capacity<T, C, 256, kSweepNPT, 4>(cl, smem, &n);
-                return nt == 128 ? launch_sweep_smem_capacity<T, C, 128, kSweepNPT>(cl, smem, &n)
-                                 : launch_sweep_smem_capacity<T, C, 256, kSweepNPT>(cl, smem, &n);
+                return sweep_variant(h, nt, [&](auto threads, auto width) {
+                    constexpr int NT = decltype(threads)::value, NX = decltype(width)::value;
+                    if constexpr (std::is_same<C, float>::value) return launch_sweep_pair_capacity<T, NT, kSweepPairs, NX>(cl, smem, &n);
+                    else return launch_sweep_smem_capacity<T, C, NT, kSweepNPT, NX>(cl, smem, &n);
+                });
             }
             const size_t smem = sweep_smem(h, g.ny_max, cl);
             if (h->nx == 4)

@@ -1,4 +1,5 @@
-// lb_sweep_smem.cuh -- the batched sweep with the channel state resident in shared memory.
+// lb_sweep_smem.cuh -- the batched sweep with the channel state resident in shared memory (FP64; the FP32
+// arithmetic has a kernel of its own, lb_sweep_pair.cuh).
 //
 // Same contract as k_sweep (lb_sweep.cuh): one thread-block cluster of CL CTAs per channel runs
 // that channel's time loop to a steady residual.  Here CTA r keeps its rows [y0, y1) of the
