@@ -272,13 +272,13 @@ __global__ void k_copy_to_host(const double* src, double* dst, int n) {
 }
 
 // Per-channel reduction of the step's block partials, one warp per channel in a fixed order
-// (deterministic; the row-march kernel forms the same values itself, see monitor_reduce_warp).
+// (deterministic; the row-march kernel forms the same values itself, see monitor_reduce).
 // with_residual = 0: the partials hold flux and max |u| only (F_MON); the residual slot reads -1
 __global__ void k_reduce_residual(const double* partials, const int* item_begin, const int* status, double* mon,
                                   int nx, long long state_index, int with_residual) {
     const int c = blockIdx.x;
-    monitor_reduce_warp(partials, item_begin[c], item_begin[c + 1], status[c], mon + 4 * c, nx, state_index,
-                        with_residual, threadIdx.x);
+    monitor_reduce(partials, item_begin[c], item_begin[c + 1], status[c], mon + 4 * c, nx, state_index, with_residual,
+                   threadIdx.x, false);
 }
 
 int grid_for(long long n) {

@@ -652,20 +652,47 @@ __device__ __forceinline__ bool velocity_ok(C jx, C jy, C rho_h, C guard) {
 }
 
 
-// Channel monitor from per-item partials (sum du^2, sum u^2, sum u_x, max |u|) of items [b, e):
-// one warp, lane l adding items b+l, b+l+32, ... in order, then a fixed butterfly, so every kernel
-// that forms it gives the same bits.  mon[0..3] = residual sqrt(sum du^2 / sum u^2) (-1 without
-// it), mean flux per column, max |u|, state index; NaN diagnostics when the channel's status is
-// set.  The partials are read through L2 (they may come from other CTAs of the same kernel).
-__device__ __forceinline__ void monitor_reduce_warp(const double* partials, int b, int e, int status, double* mon,
-                                                    int nx, long long state_index, int with_residual, int lane) {
+// Sums of three doubles over a warp with few FP64 operations (64 clocks each on their quarter of an SM): at the first
+// two steps the halves take different sums, so that 2 + 1 + 3 additions do instead of 15.  Lane 0 returns the
+// sum of v0 in v0; lane 8 that of v1 in v0; lane 16 that of v2 in v0.
+__device__ __forceinline__ void warp_sum3(double& v0, double v1, double v2, int lane) {
+    const bool hi16 = lane & 16, hi8 = lane & 8;
+    // lanes 0..15 keep (v0, v1), lanes 16..31 keep (v2, -)
+    const double s0 = hi16 ? v0 : v2, s1 = hi16 ? v1 : 0.0;
+    double k0 = hi16 ? v2 : v0;
+    const double k1 = hi16 ? 0.0 : v1;
+    k0 += __shfl_xor_sync(0xffffffffu, s0, 16);
+    const double r1 = __shfl_xor_sync(0xffffffffu, s1, 16);
+    const double k1s = k1 + r1;
+    // lanes 0..7 keep v0, 8..15 v1, 16..23 v2
+    const double snd = hi8 ? k0 : k1s, kp = hi8 ? k1s : k0;
+    double v = kp + __shfl_xor_sync(0xffffffffu, snd, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    v0 = v;
+}
+// max of non-negative doubles (their bits order as integers do: no FP64 operation)
+__device__ __forceinline__ double max_pos(double a, double b) {
+    return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
+}
+
+// Channel monitor from per-item partials (sum du^2, sum u^2, sum u_x, max |u| or (max_squared) max u^2) of items
+// [b, e): NW warps of one block, thread t adding items b+t, b+t+32 NW, ... in order, then a fixed reduction, so
+// the values do not depend on the order in which blocks finish.  mon[0..3] = residual sqrt(sum du^2 / sum u^2)
+// (-1 without it), mean flux per column, max |u|, state index; NaN diagnostics when the channel's status is set.
+// The partials are read through L2 (they may come from other CTAs of the same kernel).  red: 4 NW doubles of
+// shared memory (NW > 1; the caller's block synchronises around the call).
+template <int NW = 1>
+__device__ __forceinline__ void monitor_reduce(const double* partials, int b, int e, int status, double* mon, int nx,
+                                               long long state_index, int with_residual, int t, bool max_squared,
+                                               double* red = nullptr) {
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    constexpr int U = 8;  // items per lane loaded together (one round trip to L2 per batch)
-    for (int k0 = b + lane; k0 < e; k0 += 32 * U) {
+    constexpr int U = 8;  // items per thread loaded together (one round trip to L2 per batch)
+    for (int k0 = b + t; k0 < e; k0 += 32 * NW * U) {
         double2 v[U][2];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int k = k0 + 32 * u;
+            const int k = k0 + 32 * NW * u;
             if (k < e) {
                 v[u][0] = __ldcg(reinterpret_cast<const double2*>(partials + 4 * k));
                 v[u][1] = __ldcg(reinterpret_cast<const double2*>(partials + 4 * k + 2));
@@ -673,26 +700,36 @@ __device__ __forceinline__ void monitor_reduce_warp(const double* partials, int 
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (k0 + 32 * u < e) {
-                s0 += v[u][0].x;
+            if (k0 + 32 * NW * u < e) {
+                if (with_residual) s0 += v[u][0].x;
                 s1 += v[u][0].y;
                 s2 += v[u][1].x;
-                s3 = fmax(s3, v[u][1].y);
+                s3 = max_pos(s3, v[u][1].y);
             }
         }
     }
+    const int lane = t & 31;
+    warp_sum3(s0, s1, s2, lane);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-        s3 = fmax(s3, __shfl_xor_sync(0xffffffffu, s3, o));
+    for (int o = 16; o > 0; o >>= 1) s3 = max_pos(s3, __shfl_xor_sync(0xffffffffu, s3, o));
+    s1 = __shfl_sync(0xffffffffu, s0, 8);
+    s2 = __shfl_sync(0xffffffffu, s0, 16);
+    if constexpr (NW > 1) {
+        if (lane == 0) {
+            double* r = red + 4 * (t >> 5);
+            r[0] = s0; r[1] = s1; r[2] = s2; r[3] = s3;
+        }
+        __syncthreads();
+        if (t == 0)
+            for (int w = 1; w < NW; ++w) {
+                s0 += red[4 * w]; s1 += red[4 * w + 1]; s2 += red[4 * w + 2]; s3 = max_pos(s3, red[4 * w + 3]);
+            }
     }
-    if (lane == 0) {
+    if (t == 0) {
         const bool ok = status == 0;
-        mon[0] = !ok ? NAN : (!with_residual ? -1.0 : (s1 > 0 ? sqrt(s0 / s1) : 0.0));
+        mon[0] = !ok ? NAN : (!with_residual ? -1.0 : (s1 > 0 ? ::sqrt(s0 / s1) : 0.0));
         mon[1] = ok ? s2 / nx : NAN;
-        mon[2] = ok ? s3 : NAN;
+        mon[2] = ok ? (max_squared ? ::sqrt(s3) : s3) : NAN;
         mon[3] = (double)state_index;
     }
 }

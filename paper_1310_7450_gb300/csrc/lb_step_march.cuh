@@ -778,28 +778,20 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
         }
         __syncthreads();  // every slot read of this item is done before the next item's copies
         if (!bad && mon) {
-            // block reduction of (sum du^2, sum u^2, sum u_x, max |u|) into this item's partials
-            double v[4] = {(double)lo(r_du2) + (double)hi(r_du2), (double)lo(r_u2) + (double)hi(r_u2),
-                           (double)lo(r_ux) + (double)hi(r_ux), (double)r_umax2};
+            // block reduction of (sum du^2, sum u^2, sum u_x, max u^2) into this item's partials: few FP64 operations
+            // (a butterfly over four doubles, and the last block's over every item by one warp, made a
+            // monitored step of 1024 x 1024 nodes 7 us longer: 16 of them, with the force set and the monitor read, 684
+            // -> 565 us)
+            double v0 = resid ? (double)lo(r_du2) + (double)hi(r_du2) : 0.0;
+            const double v1 = (double)lo(r_u2) + (double)hi(r_u2), v2 = (double)lo(r_ux) + (double)hi(r_ux);
+            warp_sum3(v0, v1, v2, lane);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-                v[1] += __shfl_xor_sync(0xffffffffu, v[1], o);
-                v[2] += __shfl_xor_sync(0xffffffffu, v[2], o);
-                v[3] = fmax(v[3], __shfl_xor_sync(0xffffffffu, v[3], o));
-            }
+            for (int o = 16; o > 0; o >>= 1) r_umax2 = fmaxf(r_umax2, __shfl_xor_sync(0xffffffffu, r_umax2, o));
             double* red = reinterpret_cast<double*>(uwall);  // (free now)
-            if ((t & 31) == 0)
-                for (int k = 0; k < 4; ++k) red[4 * (t >> 5) + k] = v[k];
+            if ((lane & 7) == 0 && lane < 24) red[4 * wid + (lane >> 3)] = v0;
+            if (lane == 0) red[4 * wid + 3] = (double)r_umax2;
             __syncthreads();
-            if (t == 0) {
-                double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
-                for (int w = 0; w < NT / 32; ++w) {
-                    s0 += red[4 * w]; s1 += red[4 * w + 1]; s2 += red[4 * w + 2]; s3 = fmax(s3, red[4 * w + 3]);
-                }
-                double* o = a.partials + 4 * (long long)item;
-                o[0] = s0; o[1] = s1; o[2] = s2; o[3] = sqrt(s3);
-            }
+            if (t < 4) a.partials[4 * (long long)item + t] = t < 3 ? red[t] + red[4 + t] : max_pos(red[3], red[7]);
             __syncthreads();
         }
     }
@@ -824,11 +816,12 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
             s_last = atomicAdd(ctl.done_count, 1u) == gridDim.x - 1;
         }
         __syncthreads();
-        if (s_last && t < 32) {
+        if (s_last) {
             __threadfence();
             const int st = *(volatile const int*)a.status;
             if (ctl.mon != nullptr)
-                monitor_reduce_warp(a.partials, 0, ctl.n_items, st, ctl.mon, nx, ctl.state_index, ctl.with_residual, t);
+                monitor_reduce<NT / 32>(a.partials, 0, ctl.n_items, st, ctl.mon, nx, ctl.state_index, ctl.with_residual, t, true,
+                                        reinterpret_cast<double*>(uwall));
             if (t == 0) {
                 if (ctl.status_host != nullptr) *(volatile int*)ctl.status_host = st;
                 *ctl.done_count = 0u;

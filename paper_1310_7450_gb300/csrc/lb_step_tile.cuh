@@ -56,12 +56,6 @@ __device__ __forceinline__ void pull9(const T* __restrict__ pc, long long P, int
 }
 
 template <typename C>
-__device__ __forceinline__ C warp_sum(C v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-template <typename C>
 __device__ __forceinline__ C warp_max(C v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -278,18 +272,19 @@ __global__ void __launch_bounds__(NT) k_step_tile(const StepArgs<T, C> a) {
         }  // not the Sigma^nN pass
     }
     if (a.flags & (F_RESID | F_MON)) {
-        // block reduction of (sum du^2, sum u^2, sum u_x, max |u|) in double
+        // block reduction of (sum du^2, sum u^2, sum u_x, max |u|): sums in double, with few operations
         __shared__ double red[NT / 32][4];
-        double v0 = warp_sum<double>((double)res_du2), v1 = warp_sum<double>((double)res_u2);
-        double v2 = warp_sum<double>((double)res_ux), v3 = warp_max<double>((double)res_umax);
+        double v0 = (double)res_du2;
         const int w = t >> 5, l = t & 31;
-        if (l == 0) { red[w][0] = v0; red[w][1] = v1; red[w][2] = v2; red[w][3] = v3; }
+        warp_sum3(v0, (double)res_u2, (double)res_ux, l);
+        const C v3 = warp_max<C>(res_umax);
+        if ((l & 7) == 0 && l < 24) red[w][l >> 3] = v0;
+        if (l == 0) red[w][3] = (double)v3;
         __syncthreads();
-        if (t == 0) {
-            double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
-            for (int k = 0; k < NT / 32; ++k) { s0 += red[k][0]; s1 += red[k][1]; s2 += red[k][2]; s3 = fmax(s3, red[k][3]); }
-            double* o = a.partials + 4 * (long long)blockIdx.x;
-            o[0] = s0; o[1] = s1; o[2] = s2; o[3] = s3;
+        if (t < 4) {
+            double v = red[0][t];
+            for (int k = 1; k < NT / 32; ++k) v = t < 3 ? v + red[k][t] : max_pos(v, red[k][t]);
+            a.partials[4 * (long long)blockIdx.x + t] = v;
         }
     }
 }
