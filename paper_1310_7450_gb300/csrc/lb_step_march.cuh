@@ -50,6 +50,7 @@ struct MarchCtl {
     double* mon = nullptr;
     long long state_index = 0;
     int with_residual = 0;
+    bool dependent = false;  // host: programmatic dependent launch
 };
 
 // A CTA whose wait gave up waits this long for its own copies in flight before it returns.  A
@@ -208,9 +209,6 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
     auto ring = [&](int r, int col) -> C* { return uwall + 2 * ((r & 3) * UW + col + 2); };
 
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    const ChanParams<C> P = a.chan[0];
-    const int nx = a.nx, ny = P.ny;
-    const bool halted = a.status[0] != 0;  // an unstable or timed-out channel takes no more steps
 
     __shared__ int s_bad;  // set by any thread whose bounded wait gave up; read after a barrier
     __shared__ C s_delta[2];  // BND == 1 with GPBC: rho_out - mean(x = 0), rho_in - mean(x = nx-1)
@@ -225,14 +223,18 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
     auto bar_at = [&](uint32_t off) -> uint64_t* { return reinterpret_cast<uint64_t*>(slots + off + TX); };
     if (t == 0) {
         s_bad = 0;
-        if (BND == 1 && a.gcol != nullptr) {
-            const C* means = a.gcol + 6LL * a.gny;  // [channel][column] means of rho - 1
-            s_delta[0] = P.rho_out - means[0];
-            s_delta[1] = P.rho_in - means[1];
-        }
         prefetch_tmap(&tmap);
         for (int k = 0; k < K; ++k) mbar_init(bar_at(k * SLOT), 1);
         fence_barrier_init();
+    }
+    grid_dependency();
+    const ChanParams<C> P = a.chan[0];
+    const int nx = a.nx, ny = P.ny;
+    const bool halted = a.status[0] != 0;  // an unstable or timed-out channel takes no more steps
+    if (BND == 1 && t == 0 && a.gcol != nullptr) {
+        const C* means = a.gcol + 6LL * a.gny;  // [channel][column] means of rho - 1
+        s_delta[0] = P.rho_out - means[0];
+        s_delta[1] = P.rho_in - means[1];
     }
     __syncthreads();
 
@@ -859,8 +861,7 @@ cudaError_t launch_step_march(const CUtensorMap& map, const StepArgs<T, C>& a, c
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
-    k<<<grid, kMarchW / 2, smem, s>>>(map, a, ctl);
-    return cudaGetLastError();
+    return launch_dependent(ctl.dependent, k, grid, kMarchW / 2, smem, s, map, a, ctl);
 }
 
 template <typename T, typename C, int SMODE, int BND = 0, int SCHEME = 0, int STRIP = 0>

@@ -69,7 +69,8 @@ __global__ void __launch_bounds__(NT) k_step_tile(const StepArgs<T, C> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* su = reinterpret_cast<C*>(smem_raw);  // [EY*EX][2] gradient velocity
 
-    const WorkItem it = a.items[blockIdx.x];
+    const WorkItem it = a.items[blockIdx.x];  // (written once at create)
+    grid_dependency();
     if (a.status[it.ch] != 0) return;  // retired channel (uniform for the CTA)
     const ChanParams<C> P = a.chan[it.ch];
     const int nx = a.nx, ny = P.ny;
@@ -364,7 +365,6 @@ cudaError_t launch_step_tile(const StepArgs<T, C>& a, int n_items, size_t smem, 
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    if (n_items > 0) k<<<n_items, NT, smem, s>>>(a);
-    return cudaGetLastError();
+    return n_items > 0 ? launch_dependent(true, k, n_items, NT, smem, s, a) : cudaSuccess;
 }
 }  // namespace lbk
