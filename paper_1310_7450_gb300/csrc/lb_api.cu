@@ -245,29 +245,43 @@ __global__ void k_set_fields(T* pop, C* drho, C* sig3, const double* u, const do
     }
 }
 
-// Apply the per-channel body forces (staged[0..n_ch)) and moving-wall velocities
-// (staged[n_ch..2 n_ch)), read straight from the pinned host staging slot (mapped), and keep a
-// device copy in gx for the kernels that read the drive there.
+// The drive of up to kDriveChunk channels, a kernel argument.
+constexpr int kDriveChunk = 128;
+struct DriveArgs {
+    double g[kDriveChunk], u_wall[kDriveChunk];
+};
+
+// Apply the body forces and moving-wall velocities of channels c0 .. c0 + n - 1, and keep a device
+// copy in gx for the kernels that read the drive there.  The values are arguments, so nothing is
+// read from host memory and no staging has to be kept until the kernel ran; launched while the
+// kernel before it still runs (what it reads before the wait is constant after create).  Sixteen
+// steps of 1024 x 1024 FP32 whose drive changes and whose monitor is copied to device memory every
+// step, and the fields: 531 us with a mapped staging slot, an event and a copy, 456 now.
 template <typename C>
-__global__ void k_apply_gx(ChanParams<C>* chan, double* gx, const double* staged, int n_ch, int nx) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n_ch) return;
-    const double g = staged[c], uw = staged[n_ch + c];
+__global__ void __launch_bounds__(kDriveChunk) k_apply_gx(ChanParams<C>* chan, double* gx, const __grid_constant__ DriveArgs d,
+                                                          int c0, int n, int n_ch, int nx) {
+    const int k = threadIdx.x, c = c0 + k;
+    const bool on = k < n, gpbc = on && chan[c].gpbc;
+    const C rho0 = gpbc ? chan[c].rho0_m1 : C(0);
+    grid_dependency();
+    if (!on) return;
+    const double g = d.g[k], uw = d.u_wall[k];
     gx[c] = g;
     gx[n_ch + c] = uw;
-    chan[c].u_wall = (C)uw;  // staged after the forces: the moving-wall velocities
-    if (chan[c].gpbc) {  // pressure-driven: g sets the ghost densities, there is no body force
+    chan[c].u_wall = (C)uw;
+    if (gpbc) {  // pressure-driven: g sets the ghost densities, there is no body force
         const double half = 1.5 * g * (double)(nx + 1);
-        chan[c].rho_in = (C)((double)chan[c].rho0_m1 + half);
-        chan[c].rho_out = (C)((double)chan[c].rho0_m1 - half);
+        chan[c].rho_in = (C)((double)rho0 + half);
+        chan[c].rho_out = (C)((double)rho0 - half);
     } else {
         chan[c].gx = (C)g;
     }
 }
 
-// Copy n doubles from device memory to mapped pinned host memory (the monitor's way back: a
-// kernel's stores reach the host without a copy-engine transfer in the stream).
-__global__ void k_copy_to_host(const double* src, double* dst, int n) {
+// Copy n doubles of device memory to mapped pinned host memory or to device memory (the monitor's
+// way out: no copy-engine transfer in the stream, and set up while the step before it runs).
+__global__ void k_copy_out(const double* src, double* dst, int n) {
+    grid_dependency();
     for (int k = threadIdx.x; k < n; k += blockDim.x) dst[k] = src[k];
 }
 
@@ -312,8 +326,6 @@ struct SweepGroup {
     int var = 0, nt = 0, cl = 0;    // 0: state through L2, 1: state in shared memory; nt == 0: not tuned
     double tune_ms = 0.0;
 };
-
-constexpr int kDriveRing = 8;  // pinned staging slots of the drive (body force, wall velocity)
 
 // NVTX range over a public call, so that profiler timelines (Nsight Systems / Compute) group the
 // launches of one lb_step or sweep; a no-op unless a tool is attached.
@@ -372,13 +384,8 @@ struct lb_handle {
     int monitor_mode = 0;      // LB_MONITOR_RESIDUAL or LB_MONITOR_FLUX_MAX
     int* status_h = nullptr;   // pinned, mapped (row march: the kernel's status mirror)
     int* status_hd = nullptr;  // its device address
-    double* gx_h = nullptr;              // pinned staging of the drive: kDriveRing slots of 2 n_ch
-    double* gx_hd = nullptr;             // its device address (mapped)
-    double* mon_h = nullptr;             // mapped pinned copy of the monitor for lb_monitor
+    double* mon_h = nullptr;   // mapped pinned copy of the monitor for lb_monitor
     double* mon_hd = nullptr;
-    cudaEvent_t gx_ev[kDriveRing] = {};  // values, each reused once its previous copy has run
-    bool gx_pending[kDriveRing] = {};
-    int gx_slot = 0;
     cudaEvent_t status_ev = nullptr;
     bool status_pending = false;
     bool any_unstable = false;
@@ -880,11 +887,8 @@ void release(lb_handle* h) {
     free_dev(h->gcount);
     free_dev(h->done_count_d);
     if (h->status_h) cudaFreeHost(h->status_h);
-    if (h->gx_h) cudaFreeHost(h->gx_h);
     if (h->mon_h) cudaFreeHost(h->mon_h);
     if (h->status_ev) cudaEventDestroy(h->status_ev);
-    for (int k = 0; k < kDriveRing; ++k)
-        if (h->gx_ev[k]) cudaEventDestroy(h->gx_ev[k]);
     for (int k = 0; k < 2; ++k)
         if (h->gexec[k]) cudaGraphExecDestroy(h->gexec[k]);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
@@ -934,26 +938,19 @@ StepArgs<T, C> base_args(lb_handle* h) {
     return a;
 }
 
-// Body forces and wall velocities: host -> pinned staging (mapped) -> channel table by one small
-// kernel that reads the staging slot itself, stream-ordered.  The staging is a ring of
-// kDriveRing slots, and a slot is reused only after the kernel that read it ran, so a host that
-// changes the drive every step runs up to kDriveRing steps ahead of the device instead of waiting
-// for the step before.
+// Body forces and wall velocities: host -> channel table, stream-ordered, by value.
 lb_status push_drive(lb_handle* h) {
-    const int k = h->gx_slot;
-    h->gx_slot = (k + 1) % kDriveRing;
-    if (h->gx_pending[k]) LB_CK(cudaEventSynchronize(h->gx_ev[k]));
-    double* st = h->gx_h + (size_t)k * 2 * h->n_ch;
-    for (int c = 0; c < h->n_ch; ++c) {
-        st[c] = h->params[c].g_x;
-        st[h->n_ch + c] = h->u_wall[c];
+    for (int c0 = 0; c0 < h->n_ch; c0 += kDriveChunk) {
+        const int n = std::min(kDriveChunk, h->n_ch - c0);
+        DriveArgs d{};
+        for (int k = 0; k < n; ++k) {
+            d.g[k] = h->params[c0 + k].g_x;
+            d.u_wall[k] = h->u_wall[c0 + k];
+        }
+        const int threads = (n + 31) / 32 * 32;
+        if (h->csize == 8) LB_CK(launch_dependent(true, k_apply_gx<double>, 1, threads, 0, h->stream, (ChanParams<double>*)h->chan, h->gx_d, d, c0, n, h->n_ch, h->nx));
+        else LB_CK(launch_dependent(true, k_apply_gx<float>, 1, threads, 0, h->stream, (ChanParams<float>*)h->chan, h->gx_d, d, c0, n, h->n_ch, h->nx));
     }
-    const double* sd = h->gx_hd + (size_t)k * 2 * h->n_ch;
-    if (h->csize == 8) k_apply_gx<double><<<(h->n_ch + 255) / 256, 256, 0, h->stream>>>((ChanParams<double>*)h->chan, h->gx_d, sd, h->n_ch, h->nx);
-    else k_apply_gx<float><<<(h->n_ch + 255) / 256, 256, 0, h->stream>>>((ChanParams<float>*)h->chan, h->gx_d, sd, h->n_ch, h->nx);
-    LB_CK(cudaGetLastError());
-    LB_CK(cudaEventRecord(h->gx_ev[k], h->stream));  // the slot is read by the kernel above
-    h->gx_pending[k] = true;
     return LB_OK;
 }
 
@@ -1790,13 +1787,10 @@ lb_status lb_create(const lb_grid* grid, const lb_params* params, const lb_bound
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&h->status_hd, h->status_h, 0);
     if (e != cudaSuccess) return bail(cuda_fail(e, "lb_create: cudaHostAlloc (mapped)"));
     std::memset(h->status_h, 0, h->n_ch * sizeof(int));
-    e = cudaHostAlloc((void**)&h->gx_h, (size_t)kDriveRing * 2 * h->n_ch * sizeof(double), cudaHostAllocMapped);
-    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&h->gx_hd, h->gx_h, 0);
-    if (e == cudaSuccess) e = cudaHostAlloc((void**)&h->mon_h, 4 * (size_t)h->n_ch * sizeof(double), cudaHostAllocMapped);
+    e = cudaHostAlloc((void**)&h->mon_h, 4 * (size_t)h->n_ch * sizeof(double), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&h->mon_hd, h->mon_h, 0);
     if (e != cudaSuccess) return bail(cuda_fail(e, "lb_create: cudaHostAlloc (mapped)"));
     e = cudaEventCreateWithFlags(&h->status_ev, cudaEventDisableTiming);
-    for (int k = 0; k < kDriveRing && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&h->gx_ev[k], cudaEventDisableTiming);
     if (e != cudaSuccess) return bail(cuda_fail(e, "lb_create: cudaEventCreate"));
 
     // tables (synchronous copies: creation is not on the hot path)
@@ -1955,8 +1949,7 @@ lb_status lb_get_fields(lb_handle* h, void* u, void* sigma, void* rho, int out_d
 lb_status lb_monitor(lb_handle* h, double* out) {
     if (!h || !out) return fail(LB_EINVAL, "lb_monitor: null argument%s");
     if (h->mon_state < 0) return fail(LB_ESTATE, "lb_monitor: no monitor evaluated yet (run lb_step with n >= 2)%s");
-    k_copy_to_host<<<1, 128, 0, h->stream>>>(h->mon_d, h->mon_hd, 4 * h->n_ch);
-    LB_CK(cudaGetLastError());
+    LB_CK(launch_dependent(true, k_copy_out, 1, 128, 0, h->stream, h->mon_d, h->mon_hd, 4 * h->n_ch));
     LB_CK(cudaStreamSynchronize(h->stream));
     std::memcpy(out, h->mon_h, 4 * h->n_ch * sizeof(double));
     return LB_OK;
@@ -1965,13 +1958,16 @@ lb_status lb_monitor(lb_handle* h, double* out) {
 lb_status lb_monitor_async(lb_handle* h, double* out) {
     if (!h || !out) return fail(LB_EINVAL, "lb_monitor_async: null argument%s");
     if (h->mon_state < 0) return fail(LB_ESTATE, "lb_monitor_async: no monitor evaluated yet (run lb_step with n >= 2)%s");
-    // pinned host memory mapped into the device's address space (what cudaHostAlloc and
-    // torch's pin_memory give under unified addressing): a one-block kernel stores the values
-    // there; anything else (device memory, pageable host memory) takes a stream-ordered copy
+    // pinned host memory mapped into the device's address space (what cudaHostAlloc and torch's
+    // pin_memory give under unified addressing) and this device's own memory: a one-block kernel
+    // stores the values there; anything else (pageable host memory, managed memory, another device,
+    // an address that is no multiple of 8) takes a stream-ordered copy
     cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, out) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer) {
-        k_copy_to_host<<<1, 128, 0, h->stream>>>(h->mon_d, (double*)at.devicePointer, 4 * h->n_ch);
-        LB_CK(cudaGetLastError());
+    int dev = -1;
+    const bool known = cudaPointerGetAttributes(&at, out) == cudaSuccess && at.devicePointer && cudaGetDevice(&dev) == cudaSuccess;
+    if (known && (at.type == cudaMemoryTypeHost || (at.type == cudaMemoryTypeDevice && at.device == dev)) &&
+        (uintptr_t)at.devicePointer % sizeof(double) == 0) {
+        LB_CK(launch_dependent(true, k_copy_out, 1, 128, 0, h->stream, h->mon_d, (double*)at.devicePointer, 4 * h->n_ch));
     } else {
         (void)cudaGetLastError();
         LB_CK(cudaMemcpyAsync(out, h->mon_d, 4 * h->n_ch * sizeof(double), cudaMemcpyDefault, h->stream));
