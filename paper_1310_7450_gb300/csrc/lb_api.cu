@@ -605,8 +605,10 @@ struct MarchModel {
 //     1.35: 253.6; pressure-driven ends at 2048 x 1000 f = 1.7: 51.8, 1.5: 53.7, 1.3: 55.5, 1.2: 59.7.
 //   BF16 8192 x 2048: skew 0.3 f = 1.15: 214.4; f = 1.3: 212.8 (but leaves CTAs idle with eight per SM); f = 1.05: 228.4; skew 0.15 / 0.22 with
 //     f = 1.15: 214.5 / 214.9; skew 0.4: 228.6.
+//   BF16, pressure-driven ends, 4096 x 4096 / 2048 x 1000 / 256 x 8192: skew 0.22 f = 1.6: 258.0 / 47.4 / 63.1;
+//     0.3, 1.5: 254.5 / 49.5 / 64.0; 0.15, 1.5: 258.8 / 47.5 / 63.7; 0.15, 1.3: 264.7 / 49.5 / 63.7; 0, 1.5: 264.7 / 48.8 / 63.4.
 static MarchModel march_model(int prec, bool gpbc) {
-    if (prec == LB_PREC_BF16) return {0.30, gpbc ? 1.5 : 1.15, true};
+    if (prec == LB_PREC_BF16) return gpbc ? MarchModel{0.22, 1.6, true} : MarchModel{0.30, 1.15, true};
     return {0.08, gpbc ? 1.6 : 1.2, true};
 }
 
@@ -1007,7 +1009,7 @@ void march_monitor(lb_handle* h, int flags, MarchCtl& ctl) {
 // Programmatic dependent launch takes about 2 us off a march step, but lets blocks land on whichever SM frees a
 // slot first, against the plan that deals rows by a block's rank on its SM.  us per step without / with:
 // FP32 1024 x 1024 22.5 / 20.7, 2048 x 2048 72.6 / 71.2, 4096 x 4096 252 / 257; BF16 1024 x 1024 20.7 / 20.1,
-// 8192 x 2048 214 / 236; pressure-driven ends (a column kernel before every step) 2048 x 1000 52.9 / 56.5.
+// 8192 x 2048 214 / 236; pressure-driven ends (a column kernel before every step) FP32 2048 x 1000 52.0 / 56.5.
 bool march_dependent(const lb_handle* h) {
     return !h->gpbc && h->nodes <= (h->prec == LB_PREC_BF16 ? 1 << 21 : 1 << 22);
 }

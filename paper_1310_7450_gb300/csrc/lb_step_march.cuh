@@ -191,9 +191,8 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
     constexpr uint32_t SLOT = (TX + 8 + 127) / 128 * 128;            // a slot: the copy, then its mbarrier
     // measured choices, see the note above the launchers
     constexpr bool F32 = std::is_same<T, float>::value;
-    constexpr bool HALO2 = BND != 1;   // both halo columns of two rows in one pass (pressure-driven ends: the
-                                       // brackets of row y+3 come too late for it)
-    constexpr bool UNROLL2 = BND != 1; // the row loop written out for two rows
+    constexpr bool HALO2 = BND != 1 || !F32;    // both halo columns of two rows in one pass
+    constexpr bool UNROLL2 = BND != 1 || !F32;  // the row loop written out for two rows
     constexpr bool SHUFFLE = F32;      // neighbouring columns' velocities by warp shuffles, or a ring of rows
     constexpr bool OFF32 = F32;
     constexpr int UW = CW + 4;         // ring row: columns x0-2 .. x0+CW+1
@@ -301,12 +300,12 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
         auto patch_store = [&](int r, T v) {
             if (r >= 0 && r < ny && r <= rlast) reinterpret_cast<T*>(slots + row_at(slot_off(r), r))[pi * SW + ps] = v;
         };
-        // GPBC brackets: lanes 0..5 of the left edge strip's patchers (32..37 on a right edge
-        // strip) take one (boundary column, direction) each and evaluate source row r from the
+        // GPBC brackets: six lanes of the second warp (the first has the halo columns' moments) take one
+        // (boundary column, direction) each and evaluate source row r from the
         // slots, which hold the column's raw stored populations (the strip's own edge column, or
         // the halo image of the other end, patched before)
         const bool gpbc_edge = BND == 1 && (left_edge || right_edge) && a.gcol != nullptr;  // CTA-uniform
-        const int sl = left_edge ? t : t - 32;
+        const int sl = t - 32;
         const bool shifter = gpbc_edge && sl >= 0 && sl < 6;
         auto shift_row = [&](int r) {
             if (r < 0 || r >= ny || r > rlast) return;
@@ -320,33 +319,24 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
             moments<C>(e, mR, mx, my);
             s_shift[BND == 1 ? (r & 7) : 0][c][j] = gpbc_shift_core<C>(i, mR, mx, my, s_delta[c]);
         };
-        // end-crossing corrections and the moving wall on the pulled populations of node (col, r)
-        auto bound = [&](int col, int r, C (&d)[9]) {
-            if constexpr (BND == 1) {
-                if (gpbc_edge) {
-                    // the node's true column; the slots hold the raw periodic images, so every
-                    // population that crosses an end gets its shift here (Sec. II B):
-                    // populations entering x = 0 move with c_x = +1 and leave the column
-                    // x = nx-1 (boundary column c = 1); those entering x = nx-1 move with
-                    // c_x = -1 and leave x = 0 (c = 0)
-                    const int xg = x0 + col;
-                    const int X = xg < 0 ? xg + nx : (xg >= nx ? xg - nx : xg);
-                    // (direction indices fixed per end: one lane runs this for the whole CTA)
-                    if (X == 0) {  // from x = nx-1: directions 1, 5, 8 (source rows r, r-1, r+1)
-                        gpbc_add<C>(d[1], 1, s_shift[r & 7][1][0]);
-                        if (r > 0) gpbc_add<C>(d[5], 5, s_shift[(r - 1) & 7][1][1]);
-                        if (r < ny - 1) gpbc_add<C>(d[8], 8, s_shift[(r + 1) & 7][1][2]);
-                    } else if (X == nx - 1) {  // from x = 0: directions 3, 6, 7
-                        gpbc_add<C>(d[3], 3, s_shift[r & 7][0][0]);
-                        if (r > 0) gpbc_add<C>(d[6], 6, s_shift[(r - 1) & 7][0][1]);
-                        if (r < ny - 1) gpbc_add<C>(d[7], 7, s_shift[(r + 1) & 7][0][2]);
-                    }
-                }
-            }
-            if constexpr (BND >= 1) {
-                if (r == ny - 1 && a.chan[0].moving) zou_he_top<C>(d, a.chan[0].u_wall);
-            }
+        // The end-crossing corrections (Sec. II B) of one column's populations in row r: the slots hold the raw
+        // periodic images, so every population that crosses an end gets its shift where it is pulled.
+        // Populations entering x = 0 move with c_x = +1 and leave the column x = nx-1 (END 1: directions
+        // 1, 5, 8 from source rows r, r-1, r+1); those entering x = nx-1 move with c_x = -1 and leave
+        // x = 0 (END 0: directions 3, 6, 7).  get(i), set(i, v): the column's population of direction i.
+        auto cross = [&](auto end, int r, auto get, auto set) {
+            constexpr int E = decltype(end)::value, i0 = E ? 1 : 3, i1 = E ? 5 : 6, i2 = E ? 8 : 7;
+            auto add_shift = [&](int i, C core) {
+                C v = get(i);
+                gpbc_add<C>(v, i, core);
+                set(i, v);
+            };
+            add_shift(i0, s_shift[BND == 1 ? (r & 7) : 0][E][0]);
+            if (r > 0) add_shift(i1, s_shift[BND == 1 ? ((r - 1) & 7) : 0][E][1]);
+            if (r < ny - 1) add_shift(i2, s_shift[BND == 1 ? ((r + 1) & 7) : 0][E][2]);
         };
+        using End0 = std::integral_constant<int, 0>;
+        using End1 = std::integral_constant<int, 1>;
         // pulled populations of one node (col, r) from the slots (col relative to x0, -1 or CW too):
         // direction i comes from source row r - cy_i, column col - cx_i.  om, o0, op: slot offsets of
         // the source rows r-1, r, r+1
@@ -360,7 +350,17 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                 const T* sr = cy(i) == 1 ? sm : (cy(i) == -1 ? sp : s0);
                 d[i] = (C)Store<T>::cvt(wall ? s0[opp(i) * SW] : sr[i * SW - cx(i)]);
             }
-            bound(col, r, d);
+            if constexpr (BND == 1) {
+                if (gpbc_edge) {  // (a halo column beyond an end is the column at the other end)
+                    auto get = [&](int i) -> C { return d[i]; };
+                    auto set = [&](int i, C v) { d[i] = v; };
+                    if (col < 0 && left_edge) cross(End0(), r, get, set);
+                    if (col >= sw && right_edge) cross(End1(), r, get, set);
+                }
+            }
+            if constexpr (BND >= 1) {
+                if (r == ny - 1 && a.chan[0].moving) zou_he_top<C>(d, a.chan[0].u_wall);
+            }
         };
         // the same for the thread's two columns
         auto pull_pair = [&](int r, uint32_t om, uint32_t o0, uint32_t op, P2 (&d)[9]) {
@@ -381,20 +381,32 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                 for (int i = 0; i < 9; ++i)
                     if (cy(i) != 0 && (cy(i) == 1 ? r == 0 : r == ny - 1)) d[i] = even_pair(s0 + opp(i) * SW);
             }
-            if (BND >= 1) {
-                const bool near_end = gpbc_edge && ((left_edge && col0 == 0) || (right_edge && col0 + 2 >= sw));
-                if (near_end || r == ny - 1) {
-                    C e0[9], e1[9];
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) {
-                        e0[i] = lo(d[i]);
-                        e1[i] = hi(d[i]);
+            if constexpr (BND == 1) {
+                if (gpbc_edge) {  // the channel's first column is a pair's first; its last a pair's second, at an odd
+                                  // strip width (kOdd) its first
+                    auto get0 = [&](int i) -> C { return lo(d[i]); };
+                    auto set0 = [&](int i, C v) { d[i] = p2(v, hi(d[i])); };
+                    auto get1 = [&](int i) -> C { return hi(d[i]); };
+                    auto set1 = [&](int i, C v) { d[i] = p2(lo(d[i]), v); };
+                    if (left_edge && col0 == 0) cross(End1(), r, get0, set0);
+                    if (right_edge && col0 + 2 == sw) cross(End0(), r, get1, set1);
+                    if (ODD && right_edge && col0 + 1 == sw) {  // (its second is the halo column, the other end)
+                        cross(End0(), r, get0, set0);
+                        cross(End1(), r, get1, set1);
                     }
-                    bound(col0, r, e0);
-                    bound(col0 + 1, r, e1);
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) d[i] = p2(e0[i], e1[i]);
                 }
+            }
+            if (BND >= 1 && r == ny - 1 && a.chan[0].moving) {
+                C e0[9], e1[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    e0[i] = lo(d[i]);
+                    e1[i] = hi(d[i]);
+                }
+                zou_he_top<C>(e0, a.chan[0].u_wall);
+                zou_he_top<C>(e1, a.chan[0].u_wall);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) d[i] = p2(e0[i], e1[i]);
             }
         };
         // moments and gradient velocities of row r's own columns.  om, o0, op: slots of rows r-1, r, r+1
@@ -567,7 +579,7 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                        P2& jyn) -> bool {
             // 1. moments of row y+1 (its own populations are the next row's collision input);
             //    edge strips patch row y+4, which the moments of iteration y+2 read first
-            //    edge strips' halo columns: HALO2 takes rows y+1 and y+2 in one pass every other row
+            //    edge strips' halo columns: rows y+1 and y+2 are taken in one pass every other row
             if (!mbar_wait(bar_at(o2), par2, ctl.max_wait_ns)) s_bad = 1;  // (y + 2 <= rlast)
             const uint32_t o3 = next_slot(o2);
             const uint32_t par3 = o3 == 0 ? par2 ^ 1u : par2;
@@ -577,17 +589,24 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                 pv_a = pv_b;
                 pv_b = patch_load(y + 6);
             }
+            P2 so_xx = p2(0.f), so_xy = p2(0.f), so_yy = p2(0.f);
+            auto carried_stress = [&] {  // of row y
+                const C* s3 = a.sig3 + 2 * ctl.base + ibase + o;
+                so_xx = ld(s3);
+                so_xy = ld(s3 + PL);
+                so_yy = ld(s3 + 2 * PL);
+            };
+            // ahead of the barrier (FP32 4096 x 4096: 334 us, 357 at its use); with the fluidity, whose registers leave no
+            // room for it, at its use (2048 x 1024, 16 steps: 1070 us, 1091 here)
+            if constexpr (SMODE == 1 && SCHEME != 3) carried_stress();
             moments_row(y + 1, o0, o1, o2, dnext, dRn, jxn, jyn, un_x, un_y);
-            if constexpr (HALO2) {
-                if (even && t < 4) {
-                    const bool second = t >= 2 && y + 2 < y1;
-                    if (second && !mbar_wait(bar_at(o3), par3, ctl.max_wait_ns)) s_bad = 1;
-                    const int r = y + 1 + (t >> 1);
-                    if ((t < 2 || second) && r < ny)
-                        halo_node(r, (t & 1) == 0 ? -1 : sw, second ? o1 : o0, second ? o2 : o1, second ? o3 : o2);
-                }
-            } else {
-                if (t < 2 && y + 1 < ny) halo_node(y + 1, t == 0 ? -1 : sw, o0, o1, o2);
+            // (an end strip with pressure-driven ends: one row, the brackets of row y+3 come too late for two)
+            if (!HALO2 || gpbc_edge ? t < 2 : (even && t < 4)) {
+                const bool second = t >= 2 && y + 2 < y1;
+                if (second && !mbar_wait(bar_at(o3), par3, ctl.max_wait_ns)) s_bad = 1;
+                const int r = y + 1 + (t >> 1);
+                if ((t < 2 || second) && r < ny)
+                    halo_node(r, (t & 1) == 0 ? -1 : sw, second ? o1 : o0, second ? o2 : o1, second ? o3 : o2);
             }
             const P2 drho_prev = drho_next, upx_cur = upx_next, upy_cur = upy_next;
             drho_next = drho_next2;
@@ -611,10 +630,13 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                 issue(o0, x0, y + K);
                 issued_end = idx_of(y + K) + 1;
             }
-            // brackets of row y+4: its copy was waited by the shifter lanes (patchers) and its
-            // halo patched before the barrier above; the first pull that reads it is that of
-            // row y+3, two barriers later
-            if (shifter && y + 4 <= rlast) shift_row(y + 4);
+            // brackets of row y+4: its copy was waited and its halo patched by the patchers before the barrier
+            // above (so the wait here returns at once); the first pull that reads it is that of row
+            // y+3, two barriers later
+            if (shifter && y + 4 <= rlast) {
+                (void)wait_row(y + 4);
+                shift_row(y + 4);
+            }
             // 3. collision of row y, both nodes together, then the row's stores
             {
                 // the neighbouring columns' velocities: from the neighbouring lanes (across a warp's
@@ -648,13 +670,7 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                     By = sub(un_x, us_x);
                     Ey = sub(un_y, us_y);
                 }
-                P2 so_xx = p2(0.f), so_xy = p2(0.f), so_yy = p2(0.f);
-                if (SMODE == 1) {
-                    const C* s3 = a.sig3 + 2 * ctl.base + ibase + o;
-                    so_xx = ld(s3);
-                    so_xy = ld(s3 + PL);
-                    so_yy = ld(s3 + 2 * PL);
-                }
+                if constexpr (SMODE == 1 && SCHEME == 3) carried_stress();
                 PairState s;
                 P2 om = q.om, nom = q.nom, k2 = q.k2;
                 if constexpr (SCHEME == 1) {
@@ -699,16 +715,45 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
                 collide<SCHEME != 0>(q, s, dcur, D, om, nom, k2);
                 T* po = a.pout + 8 * ctl.base;
                 if (sr) {
-                    const uint32_t node = (uint32_t)((long long)y * nx + x0 + col0);
-                    C n0[9], n1[9];
+                    // store_node's draws and rounding, both nodes' values in one store; whether all are finite
+                    // (its exception) is asked once: BF16 4096 x 4096 258 us, 368 value by value
+                    if constexpr (!F32) {
+                        const uint32_t node = (uint32_t)((long long)y * nx + x0 + col0);
+                        P2 nan = p2(0.f);
 #pragma unroll
-                    for (int i = 0; i < 9; ++i) {
-                        const P2 v = add(dcur[i], D[i]);
-                        n0[i] = lo(v);
-                        n1[i] = hi(v);
+                        for (int i = 0; i < 9; ++i) {
+                            D[i] = add(dcur[i], D[i]);
+                            nan = fma(D[i], p2(0.f), nan);  // (NaN from an infinity or a NaN)
+                        }
+                        if (!(lo(nan) + hi(nan) == 0.f)) {
+                            C n0[9], n1[9];
+#pragma unroll
+                            for (int i = 0; i < 9; ++i) {
+                                n0[i] = lo(D[i]);
+                                n1[i] = hi(D[i]);
+                            }
+                            if (own0) store_node<T, C>(field_at(po, o, vo), PL, n0, true, a.sr_key, node);
+                            if (own1) store_node<T, C>(field_at(po, o, vo) + 1, PL, n1, true, a.sr_key, node + 1);
+                        } else {
+                            uint32_t h0 = 0, h1 = 0;
+#pragma unroll
+                            for (int i = 0; i < 9; ++i) {
+                                if ((i & 1) == 0) {
+                                    h0 = mix32(a.sr_key ^ (node * 5u + (uint32_t)(i >> 1)));
+                                    h1 = mix32(a.sr_key ^ ((node + 1) * 5u + (uint32_t)(i >> 1)));
+                                }
+                                const uint32_t b0 = __float_as_uint(lo(D[i])) + ((i & 1) ? h0 >> 16 : h0 & 0xffffu);
+                                const uint32_t b1 = __float_as_uint(hi(D[i])) + ((i & 1) ? h1 >> 16 : h1 & 0xffffu);
+                                T* p = field_at(po + i * PL, o, vo);
+                                if constexpr (ODD) {
+                                    if (own0) p[0] = __ushort_as_bfloat16((unsigned short)(b0 >> 16));
+                                    if (own1) p[1] = __ushort_as_bfloat16((unsigned short)(b1 >> 16));
+                                } else if (own0) {
+                                    *reinterpret_cast<uint32_t*>(p) = __byte_perm(b0, b1, 0x7632);
+                                }
+                            }
+                        }
                     }
-                    if (own0) store_node<T, C>(field_at(po, o, vo), PL, n0, true, a.sr_key, node);
-                    if (own1) store_node<T, C>(field_at(po, o, vo) + 1, PL, n1, true, a.sr_key, node + 1);
                 } else {
 #pragma unroll
                     for (int i = 0; i < 9; ++i) st_pop(field_at(po + i * PL, o, vo), add(dcur[i], D[i]));
@@ -849,7 +894,9 @@ constexpr int kMarchW = 128;  // columns per CTA (one strip)
 //    Seven fit six CTAs in FP32 without the ring of velocity rows, hence the warp shuffles; BF16 has
 //    the room and keeps the ring (215 / 20.8 against 223 / 20.8 with shuffles).
 //  - the row loop written out for two rows, so that no register moves between them: BF16 230 -> 215;
-//    with pressure-driven ends one row at a time is faster (2048 x 1000: 53.8 against 56.4).
+//    with pressure-driven ends FP32 is faster one row at a time (2048 x 1000: 51.6 against 53.0), BF16
+//    (4096 x 4096) is not (275 against 255).  A loop of its own for the end strips, the other strips running that
+//    of the periodic channels, was slower than either (53.2 and 274: two bodies share an SM).
 constexpr int kMarchK = 7;  // shared-memory row slots
 
 template <typename T, typename C, int SMODE, int BND = 0, int SCHEME = 0, bool FIELDS = false, int STRIP = 0>
