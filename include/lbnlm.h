@@ -51,15 +51,16 @@ typedef enum {
 enum { LB_PREC_F64 = 0, LB_PREC_F32 = 1, LB_PREC_BF16 = 2, LB_PREC_F64S_F32M = 3, LB_PREC_F32S_F64M = 4 };
 enum { LB_STRESS_INLM = 0, LB_STRESS_TIMESTEPPED = 1 };
 /* lb_grid.flags: LB_GRID_STORE_SIGMA writes the 4-component stress every step; LB_GRID_TILE_ONLY
- * keeps every step on the general tile kernel (single wide FP32/BF16 channels otherwise use the
+ * keeps every step on the general tile kernel (single FP32/BF16 channels otherwise use, from a few
+ * 100 000 nodes up, the
  * row-march kernel); LB_GRID_BF16_STOCHASTIC rounds BF16 populations stochastically (unbiased:
  * increments below half a BF16 step survive on average) instead of to nearest;
- * LB_GRID_NO_GRAPH launches every tile-kernel step separately (by default lb_step replays runs of
- * plain tile-kernel steps from a captured CUDA graph: the same kernels with the same arguments,
- * bitwise the same result, without the per-launch host overhead).
+ * LB_GRID_NO_GRAPH launches every step separately (by default lb_step replays runs of plain
+ * tile-kernel steps from a captured CUDA graph, and keeps a small single channel on chip for a run
+ * of steps: bitwise the same result, without a launch per step).
  * The comparison schemes of Sec. II C (the usual alternatives to the paper's forcing; at most one,
  * stress mode 0, periodic x and bounce-back walls, not in lb_run_until_steady; the
- * generalized-Newtonian scheme runs on the row-march kernel for wide single FP32/BF16 channels,
+ * generalized-Newtonian scheme runs on the row-march kernel for large single FP32/BF16 channels,
  * the divergence scheme on the tile kernel):
  * LB_GRID_GENERALIZED_NEWTONIAN relaxes each node with tau_LB(gdot) = 1/2 + eta_eff/(rho0 c_s^2)
  * (Eq. taulb with the model's steady-shear viscosity eta_eff = G_inf tau_M + G_inf tau0, tau_M of
@@ -71,7 +72,7 @@ enum { LB_STRESS_INLM = 0, LB_STRESS_TIMESTEPPED = 1 };
  * flow-induced density (two launches per step).  Both have delta rho = 0.
  * LB_GRID_RELAXATION_MODEL keeps the paper's scheme and enables the relaxation-time extensions of
  * its outlook (lb_set_relaxation_model; off until set): FP64, FP32 or BF16, either stress mode,
- * any boundary, not in lb_run_until_steady; one more plane per node (the fluidity).  Wide single
+ * any boundary, not in lb_run_until_steady; one more plane per node (the fluidity).  Large single
  * FP32/BF16 channels with periodic x and bounce-back walls step on the row-march kernel's variant,
  * the others on the tile kernel. */
 enum { LB_GRID_STORE_SIGMA = 1, LB_GRID_TILE_ONLY = 2, LB_GRID_BF16_STOCHASTIC = 4, LB_GRID_NO_GRAPH = 8,
@@ -118,7 +119,7 @@ typedef struct {
  *                  p_+ - p_- = g_x (nx + 1), rho_+- = rho0 +- (3/2) g_x (nx + 1); there is no body
  *                  force and no flow-induced density (delta rho = 0, Eq. bodyforce keeps its first
  *                  line), and lb_create starts from the linear density between rho_+ and rho_- .
- *                  lb_set_body_force changes the pressure gradient.  Wide single FP32/BF16 channels
+ *                  lb_set_body_force changes the pressure gradient.  Large single FP32/BF16 channels
  *                  step on the row-march kernel's boundary variant, the others on the tile kernel;
  *                  lb_run_until_steady / lb_sweep_tune return LB_EINVAL. */
 enum { LB_X_PERIODIC = 1, LB_X_GPBC = 2 };
@@ -128,7 +129,7 @@ enum { LB_X_PERIODIC = 1, LB_X_GPBC = 2 };
  *                         last row y = ny-1 lies on a wall moving with (u_wall, 0) whose incoming
  *                         populations follow Zou and He (gap ny - 1/2).  u_wall starts at 0 and is
  *                         set with lb_set_wall_velocity.  The prescribed velocity is that of the
- *                         wall row's populations, j / sum_i n_i.  Wide single FP32/BF16 channels
+ *                         wall row's populations, j / sum_i n_i.  Large single FP32/BF16 channels
  *                         step on the row-march kernel's boundary variant, the others on the tile
  *                         kernel; lb_run_until_steady / lb_sweep_tune return LB_EINVAL. */
 enum { LB_WALLS_BOUNCE_BACK = 1, LB_WALLS_COUETTE = 2 };
@@ -191,9 +192,8 @@ lb_status lb_set_monitor_mode(lb_handle *h, int mode);
 lb_status lb_monitor_async(lb_handle *h, double *out);
 
 /* Change the body force of one channel (channel = -1: all), e.g. 0 for cessation.  Stream-
- * ordered: the force is staged in mapped pinned memory, which a small kernel on the handle's stream
- * reads and applies to every step enqueued after this call; the call does not wait for the steps
- * enqueued before it (a ring of 8 staging slots: it waits only when the host is 8 changes ahead). */
+ * ordered: a small kernel on the handle's stream, whose arguments hold the values, applies it to
+ * every step enqueued after this call; the call does not wait for the steps enqueued before it. */
 lb_status lb_set_body_force(lb_handle *h, int channel, double g_x);
 
 /* Set the velocity of the moving wall of one channel (channel = -1: all) of a LB_WALLS_COUETTE
@@ -256,7 +256,8 @@ lb_status lb_sweep_config(lb_handle *h, int *threads, int *cluster, double *tune
 /* The sweep runs the stable channels in width classes (floor(log2 ny)), one persistent launch per
  * class on forked streams, each class with its own configuration: kernel variant 0 = the state
  * streamed through L2 every step (k_sweep), 1 = the state resident in the cluster's shared memory,
- * halo rows read from the neighbouring CTAs (k_sweep_smem; needs ny / cluster >= 3); threads per
+ * halo rows exchanged with the neighbouring CTAs (FP32 arithmetic k_sweep_pair, FP64
+ * k_sweep_smem; needs ny / cluster >= 3); threads per
  * CTA; CTAs per cluster.  lb_sweep_groups writes up to max_groups entries (any pointer may be NULL;
  * threads 0 = not tuned yet) and returns the number of classes (-1: null handle).
  * lb_sweep_config reports the widest class and the summed tuning time; lb_sweep_variant the

@@ -391,7 +391,7 @@ struct lb_handle {
     bool any_unstable = false;
     bool any_timeout = false;
     unsigned long long wait_ns = kDefaultWaitNs;  // limit of the row-march kernel's mbarrier waits
-    // row-march kernel (wide single channels, FP32 / BF16 storage)
+    // row-march kernel (large single channels, FP32 / BF16 storage)
     bool march = false;
     int march_strip = kFull;   // its strips: whole, partial, or rows of any length
     CUtensorMap mapA, mapB;    // tensor maps of the two population buffers ...
