@@ -408,6 +408,7 @@ struct lb_handle {
     bool sweep_fixed = false;               // configuration set by lb_sweep_set_config
     cudaGraphExec_t sweep_gexec = nullptr;  // the class launches captured as one graph ...
     std::vector<double> sweep_key;          // ... for these arguments and configurations
+    const void* sweep_pin = nullptr;        // ... and this population buffer
     MarchItem* march_items_d = nullptr;
     int* march_item_begin_d = nullptr;  // {0, n_march_items}: the residual reduction's item range
     int n_march_items = 0, march_grid = 0;
@@ -1492,15 +1493,15 @@ lb_status sweep_tune(lb_handle* h, bool all) {
 }
 
 // One persistent launch per width class on forked streams, joined back: captured once as a CUDA
-// graph (on the handle's private capture stream) and replayed while the arguments and the class
-// configurations stay the same.
+// graph (on the handle's private capture stream) and replayed while the arguments, the class
+// configurations and the population buffer that holds the state (lb_step swaps the two) stay the same.
 lb_status sweep_run(lb_handle* h, double tol, int check, long long max_steps) {
     const size_t G = h->sweep_groups.size();
     const uint32_t key_sr = step_key(h, h->step + 0x5bd1e995ll);
     std::vector<double> key = {tol, (double)check, (double)max_steps, (double)key_sr};
     for (const SweepGroup& g : h->sweep_groups)
         for (int v : {g.begin, g.count, g.ny_min, g.ny_max, g.var, g.nt, g.cl}) key.push_back((double)v);
-    if (!h->sweep_gexec || key != h->sweep_key) {
+    if (!h->sweep_gexec || key != h->sweep_key || h->sweep_pin != h->popA) {
         if (h->sweep_gexec) {
             LB_CK(cudaGraphExecDestroy(h->sweep_gexec));
             h->sweep_gexec = nullptr;
@@ -1540,6 +1541,7 @@ lb_status sweep_run(lb_handle* h, double tol, int check, long long max_steps) {
             return cuda_fail(e, "lb_run_until_steady: graph capture");
         }
         h->sweep_key = key;
+        h->sweep_pin = h->popA;
     }
     LB_CK(cudaGraphLaunch(h->sweep_gexec, h->stream));
     return LB_OK;
