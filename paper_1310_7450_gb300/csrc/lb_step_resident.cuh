@@ -172,10 +172,16 @@ __global__ void __launch_bounds__(NT) k_step_resident(const StepArgs<T, C> a, T*
         cur = nxt;
         stop = s_stop[s & 1];
     }
-    // the state after the last step, back into the buffer it came from
+    // the state after the last step, back into the buffer it came from; a stopped channel's also into the other
+    // one: the host goes on swapping the two for steps that do nothing
     if (own) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) gpop[(long long)i * P.P + pn] = buf[cur + i * PS + lr + x];
+        if (stop) {
+            T* other = a.pout + 9 * P.base;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) other[(long long)i * P.P + pn] = buf[cur + i * PS + lr + x];
+        }
         a.drho[P.base + pn] = drho;
         if (SMODE == 1) {
             C* s3 = a.sig3 + 3 * P.base + pn;
