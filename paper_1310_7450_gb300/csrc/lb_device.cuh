@@ -212,6 +212,18 @@ __device__ __forceinline__ void grid_dependency() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// Let a kernel take all the dynamic shared memory a CTA can have (227 KB less its static part), as a cluster of any
+// size.  The limit is a property of the kernel, which handles in several threads share, so it is never
+// that of one launch: another thread could lower it between this one's setting and launch.
+template <typename K>
+cudaError_t allow_shared_memory(K k) {
+    cudaFuncAttributes at{};
+    cudaError_t e = cudaFuncGetAttributes(&at, k);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    const int most = 227 * 1024 - (int)at.sharedSizeBytes;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    return e;
+}
 template <typename K, typename... Args>
 cudaError_t launch_dependent(bool dependent, K k, int grid, int block, size_t smem, cudaStream_t s, const Args&... args) {
     cudaLaunchConfig_t cfg = {};

@@ -192,10 +192,7 @@ __global__ void __launch_bounds__(NT) k_step_resident(const StepArgs<T, C> a, T*
     }
 }
 
-template <typename K>
-cudaError_t resident_launch_config(K k, int cl, int threads, size_t smem, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+inline void resident_launch_config(int cl, int threads, size_t smem, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
     *cfg = cudaLaunchConfig_t{};
     cfg->gridDim = dim3(cl);
     cfg->blockDim = dim3((threads + 31) / 32 * 32);
@@ -206,16 +203,17 @@ cudaError_t resident_launch_config(K k, int cl, int threads, size_t smem, cudaLa
     attr->val.clusterDim.z = 1;
     cfg->attrs = attr;
     cfg->numAttrs = 1;
-    return e;
 }
 
-// Clusters of this shape the device holds at once (0: it cannot be launched), and the launch.
+// Clusters of this shape the device holds at once (0: it cannot be launched), and the launch (after that question, which
+// sets the kernel's limits).
 template <typename T, typename C, int SMODE, int NT>
 cudaError_t resident_capacity(int cl, int threads, size_t smem, int* clusters) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     auto k = k_step_resident<T, C, SMODE, NT>;
-    cudaError_t e = resident_launch_config(k, cl, threads, smem, &cfg, attr);
+    resident_launch_config(cl, threads, smem, &cfg, attr);
+    const cudaError_t e = allow_shared_memory(k);
     return e == cudaSuccess ? cudaOccupancyMaxActiveClusters(clusters, k, &cfg) : e;
 }
 template <typename T, typename C, int SMODE, int NT>
@@ -223,11 +221,9 @@ cudaError_t launch_step_resident(const StepArgs<T, C>& a, T* pop, long long step
                                  cudaStream_t s) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    auto k = k_step_resident<T, C, SMODE, NT>;
-    cudaError_t e = resident_launch_config(k, cl, threads, smem, &cfg, attr);
-    if (e != cudaSuccess) return e;
+    resident_launch_config(cl, threads, smem, &cfg, attr);
     cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, k, a, pop, steps);
+    return cudaLaunchKernelEx(&cfg, k_step_resident<T, C, SMODE, NT>, a, pop, steps);
 }
 
 // X(T, C, SMODE, NT): the kernel's instantiations; NT bounds the threads (and so the registers) of a CTA.

@@ -229,9 +229,7 @@ __global__ void __launch_bounds__(NT, sizeof(C) == 8 ? 1 : 512 / NT) k_sweep(con
 template <typename T, typename C, int NT, int NPT, int NX = 0>
 cudaError_t launch_sweep_capacity(int cl, size_t smem, int* n_clusters) {
     auto k = k_sweep<T, C, NT, NPT, NX>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared_memory(k);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cl);
@@ -250,10 +248,7 @@ cudaError_t launch_sweep_capacity(int cl, size_t smem, int* n_clusters) {
 template <typename T, typename C, int NT, int NPT, int NX = 0>
 cudaError_t launch_sweep(const SweepArgs<T, C>& a, int n_clusters, int cl, size_t smem, cudaStream_t s) {
     auto k = k_sweep<T, C, NT, NPT, NX>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    // set every time: an earlier capacity query may have left a smaller limit
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared_memory(k);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_clusters * cl);

@@ -275,10 +275,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_sweep_pair(const SweepArgs<T, 
 
 template <typename T, int NT, int NP, int NX>
 cudaError_t sweep_pair_config(int n_clusters, int cl, size_t smem, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
-    auto k = k_sweep_pair<T, NT, NP, NX>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    // (set every time: an earlier capacity query may have left a smaller limit)
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_shared_memory(k_sweep_pair<T, NT, NP, NX>);
     *cfg = cudaLaunchConfig_t{};
     cfg->gridDim = dim3(n_clusters * cl);
     cfg->blockDim = dim3(NT);

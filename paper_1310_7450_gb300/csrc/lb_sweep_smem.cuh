@@ -280,9 +280,7 @@ constexpr size_t sweep_smem_bytes(int rows, int nx) {
 template <typename T, typename C, int NT, int NPT, int NX = 0>
 cudaError_t launch_sweep_smem_capacity(int cl, size_t smem, int* n_clusters) {
     auto k = k_sweep_smem<T, C, NT, NPT, NX>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared_memory(k);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cl);
@@ -301,9 +299,7 @@ cudaError_t launch_sweep_smem_capacity(int cl, size_t smem, int* n_clusters) {
 template <typename T, typename C, int NT, int NPT, int NX = 0>
 cudaError_t launch_sweep_smem(const SweepArgs<T, C>& a, int n_clusters, int cl, size_t smem, cudaStream_t s) {
     auto k = k_sweep_smem<T, C, NT, NPT, NX>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared_memory(k);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_clusters * cl);
