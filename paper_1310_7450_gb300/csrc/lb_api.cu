@@ -19,6 +19,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "lb_march_plan.h"
 #include "lb_step_march.cuh"
 #include "lb_step_resident.cuh"
 #include "lb_step_tile.cuh"
@@ -578,29 +579,6 @@ bool make_pop_map(const lb_handle* h, void* base, CUtensorMap* map) {
     return r == CUDA_SUCCESS;
 }
 
-// Row-march work items: strips of kMarchW columns cut into row ranges, at most one item per
-// resident CTA (one wave: a partial second wave would double the kernel time for a few CTAs).
-// Items are not equally long, because CTAs are not equally fast: the warp schedulers favour older
-// warps, so the CTAs that arrive later on an SM take longer for the same rows, and an edge strip costs more per row than an interior one (its
-// halo columns are patched from the other end; with pressure-driven ends it also applies the
-// crossing corrections).  The model: block b, of rank k = b / n_sm (blocks fill the SMs rank by
-// rank), runs at speed 1 + skew (R-1-k)/(R-1) for R CTAs per SM; strip j costs f_j per row (f for
-// the two edge strips, 1 inside).  A bisection finds the smallest common duration T whose dealing
-// needs at most R n_sm blocks; rows are then split in proportion to the blocks' speeds.  Two
-// dealings:
-//  - strip-major: each strip takes consecutive blocks until their speeds cover ny f_j / T;
-//  - chunk-major: the edge strips first, the same way, then the interior strips share their row
-//    boundaries -- row chunk c of every interior strip on consecutive blocks, T times the speed of
-//    the slowest of them in rows -- so neighbouring strips march the same rows at the same time
-//    and read each other's halo columns from L2 (with boundaries that differ between strips, BF16
-//    re-reads 9 DRAM bytes per node of halo).  Both precisions are dealt chunk-major; strip-major
-//    serves grids of one or two strips.
-// Items keep at least 8 rows on average (at most ny / 8 per strip).
-struct MarchModel {
-    double skew, fedge;
-    bool chunk_major;
-};
-
 // Constants measured with six CTAs of two warps per SM (us per step, one GPU):
 //   FP32 4096 x 4096: skew 0.06: 251.9, 0.12: 252.9, 0: 252.7, 0.2: 257.7; f = 1.2 252.9, 1.05: 264.0,
 //     1.35: 253.6; pressure-driven ends at 2048 x 1000 f = 1.7: 51.8, 1.5: 53.7, 1.3: 55.5, 1.2: 59.7.
@@ -611,111 +589,6 @@ struct MarchModel {
 static MarchModel march_model(int prec, bool gpbc) {
     if (prec == LB_PREC_BF16) return gpbc ? MarchModel{0.22, 1.6, true} : MarchModel{0.30, 1.15, true};
     return {0.08, gpbc ? 1.6 : 1.2, true};
-}
-
-static std::vector<MarchItem> march_plan(int nx, int ny, int R, int nsm, MarchModel m) {
-    // strips of one width (a multiple of 8 columns) but the last, which has two at least (a halo column's
-    // populations come from one column further on)
-    const int least = (nx + kMarchW - 1) / kMarchW;
-    int W = std::min(kMarchW, ((nx + least - 1) / least + 7) / 8 * 8);
-    while (nx % W == 1) W -= 8;
-    const int strips = (nx + W - 1) / W;
-    auto width = [&](int x0) { return std::min(W, nx - x0); };
-    const int slots = R * nsm;
-    const int maxn = std::max(1, ny / 8);
-    auto speed = [&](int b) {
-        const int k = std::min(b / nsm, R - 1);
-        return 1.0 + (R > 1 ? m.skew * (R - 1 - k) / (R - 1) : 0.0);
-    };
-    auto cost = [&](int s) { return (s == 0 || s == strips - 1) ? m.fedge : 1.0; };
-    // the rows [0, ny) of one strip split in proportion to the weights w
-    auto split = [&](std::vector<MarchItem>& out, int x0, const std::vector<double>& w) {
-        double tot = 0.0;
-        for (double v : w) tot += v;
-        double cum = 0.0;
-        int y = 0;
-        for (size_t k = 0; k < w.size(); ++k) {
-            cum += w[k];
-            const int y1 = k + 1 == w.size() ? ny : (int)std::llround(ny * cum / tot);
-            MarchItem it{};
-            it.x0 = x0;
-            it.y0 = y;
-            it.y1 = y1;
-            it.w = width(x0);
-            out.push_back(it);
-            y = y1;
-        }
-    };
-    // blocks from b on until their speeds cover ny f / T (at most maxn)
-    auto take = [&](double T, int b, double f) {
-        double acc = 0.0;
-        int n = 0;
-        while (n < maxn && acc < ny * f / T) acc += speed(b + n++);
-        return n;
-    };
-    const bool cm = m.chunk_major && strips >= 3 && strips < slots;
-    const int I = strips - 2;
-    // blocks per strip (strip-major) or [edge 0, edge 1, chunks] (chunk-major) at duration T
-    auto deal = [&](double T, std::vector<int>* out) {
-        int b = 0;
-        if (!cm) {
-            for (int s = 0; s < strips; ++s) {
-                const int n = strips >= slots ? 1 : take(T, b, cost(s));
-                if (out) out->push_back(n);
-                b += n;
-            }
-            return b;
-        }
-        for (int e = 0; e < 2; ++e) {
-            const int n = take(T, b, m.fedge);
-            if (out) out->push_back(n);
-            b += n;
-        }
-        int C = 0;
-        double acc = 0.0;
-        while (C < maxn && acc < ny) acc += T * speed(b + (++C) * I - 1);
-        if (out) out->push_back(C);
-        return b + C * I;
-    };
-    double lo = 1e-9, hi = 4.0 * ny * std::max(1.0, m.fedge);  // deal(hi): one block per strip
-    if (strips >= slots || deal(lo, nullptr) <= slots) {
-        hi = strips >= slots ? hi : lo;
-    } else {
-        for (int it = 0; it < 100; ++it) {
-            const double mid = 0.5 * (lo + hi);
-            if (deal(mid, nullptr) <= slots) hi = mid;
-            else lo = mid;
-        }
-    }
-    std::vector<int> n;
-    deal(hi, &n);
-    std::vector<MarchItem> items;
-    int b = 0;
-    auto strip_items = [&](int s, int cnt) {
-        std::vector<double> w(cnt);
-        for (int k = 0; k < cnt; ++k) w[k] = speed(b + k);
-        split(items, s * W, w);
-        b += cnt;
-    };
-    if (!cm) {
-        for (int s = 0; s < strips; ++s) strip_items(s, n[s]);
-        return items;
-    }
-    strip_items(0, n[0]);
-    strip_items(strips - 1, n[1]);
-    const int C = n[2];
-    std::vector<double> wc(C);
-    for (int c = 0; c < C; ++c) wc[c] = speed(b + (c + 1) * I - 1);
-    std::vector<MarchItem> chunk;
-    split(chunk, 0, wc);
-    for (int c = 0; c < C; ++c)
-        for (int s = 1; s <= I; ++s) {
-            MarchItem it = chunk[c];
-            it.x0 = s * W;
-            it.w = width(it.x0);
-            items.push_back(it);
-        }
-    return items;
 }
 
 // The row-march variant of a handle: f(stress mode, boundary, scheme, strips) as constants.
@@ -736,52 +609,6 @@ auto march_variant(const lb_handle* h, F&& f) {
     return with_mode(Num<0>{}, Num<0>{});
 }
 
-// A grid too small to give every resident CTA an 8-row item is cut finer, down to 2 rows: a row takes about 1.5 us
-// whatever the chip's load (its instructions wait for one another), so the launch lasts as long as its
-// longest item.  128 x 512 FP32: 18.8 us with 8-row items, 9.6 with 2-row ones.
-static std::vector<MarchItem> fine_items(std::vector<MarchItem> in, int nx, int ny, int slots) {
-    int strips = 0, W = in[0].w;
-    for (const MarchItem& it : in) {
-        strips += it.y0 == 0;
-        W = std::max(W, it.w);
-    }
-    if ((long long)strips * (ny / 8) >= slots) return in;
-    const int n = std::min(ny / 2, std::max(1, slots / strips));
-    std::vector<MarchItem> out;
-    for (int k = 0; k < n; ++k)
-        for (int s = 0; s < strips; ++s) {
-            MarchItem it{};
-            it.x0 = s * W;
-            it.w = std::min(W, nx - it.x0);
-            it.y0 = (int)((long long)ny * k / n);
-            it.y1 = (int)((long long)ny * (k + 1) / n);
-            out.push_back(it);
-        }
-    return out;
-}
-
-// The kernel addresses an item's rows with 32-bit offsets: items of 2^29 elements or more are halved.
-static std::vector<MarchItem> short_items(const std::vector<MarchItem>& in, int nx) {
-    std::vector<MarchItem> out;
-    for (MarchItem it : in) {
-        const long long most = std::max(8LL, (1LL << 29) / nx);
-        while (it.y1 - it.y0 > most) {
-            MarchItem a = it;
-            a.y1 = it.y0 + (it.y1 - it.y0) / 2;
-            it.y0 = a.y1;
-            while (a.y1 - a.y0 > most) {
-                MarchItem b = a;
-                b.y1 = a.y0 + (int)most;
-                out.push_back(b);
-                a.y0 = b.y1;
-            }
-            out.push_back(a);
-        }
-        out.push_back(it);
-    }
-    return out;
-}
-
 // Whole strips always march; other widths where that is the faster kernel.  A march step lasts 10 us at least (a
 // chain of rows), a tile step 5, but the tile kernel takes 1.3 to 2 times as long per node.  Tile / march, us:
 // FP32 100 x 1600 10.1 / 12.7, 200 x 1600 15.8 / 16.8, 500 x 800 17.5 / 16.8, 1000 x 777 30.1 / 23.0, 1001 x 777
@@ -789,7 +616,7 @@ static std::vector<MarchItem> short_items(const std::vector<MarchItem>& in, int 
 // 1000 x 300 18.1 / 13.5, 1001 x 777 44.8 / 26.8.  Below 96 columns half of a strip's threads have none.
 static bool march_pays(const lb_handle* h) {
     if (h->nx % kMarchW == 0) return true;
-    return h->nx >= 96 && (long long)h->nx * h->ny[0] >= (h->prec == LB_PREC_BF16 ? 150000 : 400000);
+    return h->nx >= 96 && march_strip_width(h->nx) > 0 && (long long)h->nx * h->ny[0] >= (h->prec == LB_PREC_BF16 ? 150000 : 400000);
 }
 
 lb_status plan_march(lb_handle* h) {

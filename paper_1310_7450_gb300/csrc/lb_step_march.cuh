@@ -24,16 +24,12 @@
 
 #include <cuda.h>
 
+#include "lb_march_plan.h"
 #include "lb_pair.cuh"
 
 namespace lbk {
 
 enum : int { kFull = 0, kPart = 1, kOdd = 2 };  // strips of a channel, see k_step_march
-
-struct MarchItem {
-    int x0, y0, y1;  // first column, rows [y0, y1)
-    int w;           // columns (kMarchW at most)
-};
 
 struct MarchCtl {
     const MarchItem* items;
@@ -880,7 +876,6 @@ __global__ void __launch_bounds__(CW / 2, 6) k_step_march(const __grid_constant_
 }  // namespace lbk
 
 namespace lbk {
-constexpr int kMarchW = 128;  // columns per CTA (one strip)
 // How the kernel is shaped, and what it measured (us per step; FP32 at 4096 x 4096 / 1024 x 1024, BF16
 // at 8192 x 2048 / 1024 x 1024; one column per thread in scalar FP32 before: 274 / 24.8 and 222 / 24.8).
 // Two columns per thread as packed FP32 take the instructions per node from 468 to 268 (FP32) and from
