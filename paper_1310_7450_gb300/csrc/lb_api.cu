@@ -360,6 +360,7 @@ struct lb_handle {
     // learned warm start: per-channel closed-form parameters, row offsets, closed form on the rows
     // [row][3] and on the network grid [channel][3][256], scales [channel][3]
     void *ws_prm = nullptr, *ws_row_off = nullptr, *ws_rows = nullptr, *ws_grid = nullptr, *ws_scale = nullptr;
+    bool ws_ready = false;     // ... allocated and filled
     void* chan = nullptr;
     WorkItem* items_d = nullptr;
     int* item_begin_d = nullptr;
@@ -1875,22 +1876,31 @@ lb_status lb_set_fields(lb_handle* h, const double* u, const double* rho, const 
     return set_fields_dev(h, su, sr, drho ? sd : nullptr);
 }
 
+// The warm start's tables and profile buffers, on the first call that gets them all: one that fails half-way (out of
+// memory, in the middle of a stream capture) leaves the next to begin anew.
+static lb_status ws_tables(lb_handle* h) {
+    if (h->ws_ready) return LB_OK;
+    for (void** q : {&h->ws_prm, &h->ws_row_off, &h->ws_rows, &h->ws_grid, &h->ws_scale}) free_dev(*q);
+    LB_CK(cudaMalloc(&h->ws_prm, sizeof(WsChan) * h->n_ch));
+    LB_CK(cudaMalloc(&h->ws_row_off, sizeof(int) * h->n_ch));
+    LB_CK(cudaMalloc(&h->ws_rows, sizeof(double) * 3 * (size_t)h->gny));
+    LB_CK(cudaMalloc(&h->ws_grid, sizeof(double) * 3 * 256 * (size_t)h->n_ch));
+    LB_CK(cudaMalloc(&h->ws_scale, sizeof(double) * 3 * (size_t)h->n_ch));
+    std::vector<WsChan> prm(h->n_ch);
+    for (int c = 0; c < h->n_ch; ++c)
+        prm[c] = WsChan{h->params[c].G_inf, h->params[c].tau0, h->params[c].theta, h->params[c].gamma_c};
+    LB_CK(cudaMemcpyAsync(h->ws_row_off, h->row_off.data(), sizeof(int) * h->n_ch, cudaMemcpyHostToDevice, h->stream));
+    LB_CK(cudaMemcpyAsync(h->ws_prm, prm.data(), sizeof(WsChan) * h->n_ch, cudaMemcpyHostToDevice, h->stream));
+    LB_CK(cudaStreamSynchronize(h->stream));  // (prm goes)
+    h->ws_ready = true;
+    return LB_OK;
+}
+
 // Learned warm start: the closed-form steady profile of every channel (current parameters) on its
 // rows and on the network grid, with the per-field scales.
 static lb_status ws_closed_form(lb_handle* h) {
-    if (!h->ws_prm) {
-        LB_CK(cudaMalloc(&h->ws_prm, sizeof(WsChan) * h->n_ch));
-        LB_CK(cudaMalloc(&h->ws_row_off, sizeof(int) * h->n_ch));
-        LB_CK(cudaMalloc(&h->ws_rows, sizeof(double) * 3 * (size_t)h->gny));
-        LB_CK(cudaMalloc(&h->ws_grid, sizeof(double) * 3 * 256 * (size_t)h->n_ch));
-        LB_CK(cudaMalloc(&h->ws_scale, sizeof(double) * 3 * (size_t)h->n_ch));
-        std::vector<WsChan> prm(h->n_ch);
-        for (int c = 0; c < h->n_ch; ++c)
-            prm[c] = WsChan{h->params[c].G_inf, h->params[c].tau0, h->params[c].theta, h->params[c].gamma_c};
-        LB_CK(cudaMemcpyAsync(h->ws_row_off, h->row_off.data(), sizeof(int) * h->n_ch, cudaMemcpyHostToDevice, h->stream));
-        LB_CK(cudaMemcpyAsync(h->ws_prm, prm.data(), sizeof(WsChan) * h->n_ch, cudaMemcpyHostToDevice, h->stream));
-        LB_CK(cudaStreamSynchronize(h->stream));  // (prm goes; the first call only)
-    }
+    lb_status st = ws_tables(h);
+    if (st != LB_OK) return st;
     for (int c = 0; c < h->n_ch; ++c) {
         const lb_params& p = h->params[c];
         if (!(p.G_inf > 0.0) || !(p.tau0 > 0.0) || !(p.g_x > 0.0))
