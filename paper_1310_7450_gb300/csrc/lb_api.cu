@@ -370,8 +370,8 @@ struct lb_handle {
     long long *base_d = nullptr, *P_d = nullptr, *node_off_d = nullptr;
     int* ny_d = nullptr;
     double* gx_d = nullptr;
-    void* fields = nullptr;    // staging of fields, 7 values per node (allocated when first needed)
-    size_t fields_bytes = 0;
+    void* fields[2] = {nullptr, nullptr};  // staging of fields as float / double, 7 values per node (each allocated
+                                           // when first needed and kept: a captured call holds its address)
     void* hstage = nullptr;    // device staging for FP64 host transfers
     size_t hstage_bytes = 0;
     // launch plan
@@ -705,7 +705,7 @@ void release(lb_handle* h) {
     free_dev(h->popA); free_dev(h->popB); free_dev(h->drho); free_dev(h->sig3); free_dev(h->sig4); free_dev(h->snn); free_dev(h->phi);
     free_dev(h->uprev); free_dev(h->chan); free_dev(h->items_d); free_dev(h->item_begin_d);
     free_dev(h->partials); free_dev(h->mon_d); free_dev(h->status_d); free_dev(h->base_d); free_dev(h->P_d);
-    free_dev(h->node_off_d); free_dev(h->ny_d); free_dev(h->gx_d); free_dev(h->fields);
+    free_dev(h->node_off_d); free_dev(h->ny_d); free_dev(h->gx_d); free_dev(h->fields[0]); free_dev(h->fields[1]);
     free_dev(h->hstage);
     free_dev(h->ws_prm); free_dev(h->ws_row_off); free_dev(h->ws_rows); free_dev(h->ws_grid); free_dev(h->ws_scale);
     free_dev(h->march_items_d);
@@ -1043,14 +1043,10 @@ lb_status fields_pass(lb_handle* h, void* fu, void* fs, void* fr, bool out64) {
     });
 }
 
-// The handle's staging buffer of 7 values per node (u, sigma, rho one after the other).
+// The handle's staging buffer of 7 values per node (u, sigma, rho one after the other), of float or double.
 lb_status ensure_fields(lb_handle* h, size_t value_size) {
-    const size_t bytes = 7 * (size_t)h->nodes * value_size + 64;
-    if (h->fields_bytes >= bytes) return LB_OK;
-    free_dev(h->fields);
-    h->fields_bytes = 0;
-    LB_CK(cudaMalloc(&h->fields, bytes));
-    h->fields_bytes = bytes;
+    void*& f = h->fields[value_size == 8];
+    if (!f) LB_CK(cudaMalloc(&f, 7 * (size_t)h->nodes * value_size + 64));
     return LB_OK;
 }
 // its parts, each on a 16-byte boundary
@@ -1058,7 +1054,7 @@ struct FieldParts {
     char *u, *sigma, *rho;
 };
 FieldParts field_parts(lb_handle* h, size_t value_size) {
-    char* b = (char*)h->fields;
+    char* b = (char*)h->fields[value_size == 8];
     const size_t n = (size_t)h->nodes * value_size;
     return FieldParts{b, b + (2 * n + 15) / 16 * 16, b + (2 * n + 15) / 16 * 16 + 4 * n};
 }
