@@ -421,6 +421,7 @@ int nblocks(long long n) {
 
 struct lb_mlp {
     int n_in = 0, H = 0, n_out = 0, max_batch = 0;
+    int dev = 0;  // device that was current at creation
     cudaStream_t stream = nullptr;
     long long n_par = 0, o_w1 = 0, o_b1 = 0, o_w2 = 0, o_b2 = 0, o_w3 = 0, o_b3 = 0;
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;  // masters, gradients, Adam moments
@@ -575,6 +576,7 @@ lb_status lb_mlp_create(int n_in, int width, int n_out, int max_batch, uint64_t 
     if (!m) return mfail(LB_ENOMEM, "lb_mlp_create: host allocation");
     m->n_in = n_in; m->H = width; m->n_out = n_out; m->max_batch = max_batch;
     m->stream = (cudaStream_t)cuda_stream;
+    cudaGetDevice(&m->dev);
     m->o_w1 = 0; m->o_b1 = m->o_w1 + (long long)width * n_in;
     m->o_w2 = m->o_b1 + width; m->o_b2 = m->o_w2 + (long long)width * width;
     m->o_w3 = m->o_b2 + width; m->o_b3 = m->o_w3 + (long long)n_out * width;
@@ -610,10 +612,11 @@ long long lb_mlp_num_params(const lb_mlp* m) { return m ? m->n_par : 0; }
 
 lb_status lb_mlp_forward(lb_mlp* m, const float* x, int batch, float* y) {
     if (!m || !x || !y || batch < 1 || batch > m->max_batch) return mfail(LB_EINVAL, "lb_mlp_forward: bad argument");
-    // device memory is written by the last layer itself; anything else gets a copy
+    // this device's memory is written by the last layer itself; anything else (another device's memory, an address
+    // that is no multiple of 4) gets a copy
     cudaPointerAttributes at{};
-    const bool direct = cudaPointerGetAttributes(&at, y) == cudaSuccess &&
-                        (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
+    const bool direct = (uintptr_t)y % sizeof(float) == 0 && cudaPointerGetAttributes(&at, y) == cudaSuccess &&
+                        ((at.type == cudaMemoryTypeDevice && at.device == m->dev) || at.type == cudaMemoryTypeManaged);
     (void)cudaGetLastError();
     lb_status st = forward(m, x, batch, direct ? y : m->y);
     if (st != LB_OK || direct) return st;
