@@ -67,7 +67,9 @@ enum Epilogue { EP_TANH, EP_LINEAR, EP_MSE, EP_DTANH, EP_GRAD };
 // What a kernel may read before the grid before it in the stream has finished.  A kernel's blocks start when all
 // blocks of that grid have passed their own wait, so the grids before that one have finished: the weights
 // (written by the last launch of a step, or by the call before) are ready for every launch but the
-// first, and an activation or gradient is when the grid that writes it lies two launches back.
+// first, and an activation or gradient is when the grid that writes it lies two launches back.  Those grids have
+// finished, so their results are in L2; that a kernel's L1 holds no older copy is promised only behind its own
+// wait, so what is read ahead of it is loaded through L2 (ld.global.cg).
 enum Ready { READY_NONE, READY_B, READY_ALL };  // READY_ALL: both operands; only the results wait
 
 struct Adam {  // Adam (Kingma & Ba 2015) on the FP32 masters, then the BF16 working copy; p == nullptr: no update
@@ -114,12 +116,16 @@ __device__ __forceinline__ void grid_dependency() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// 16 bytes as FP32 values, and one value.  EARLY: of global memory ahead of the wait, through L2 (see Ready).
+template <bool EARLY = false>
 __device__ __forceinline__ void load16(const float* p, float (&v)[4]) {
-    const float4 q = *reinterpret_cast<const float4*>(p);
+    const float4 q = EARLY ? __ldcg(reinterpret_cast<const float4*>(p)) : *reinterpret_cast<const float4*>(p);
     v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
 }
+template <bool EARLY = false>
 __device__ __forceinline__ void load16(const __nv_bfloat16* p, float (&v)[8]) {
-    const uint4 q = *reinterpret_cast<const uint4*>(p);  // (a BF16 value is the high half of its FP32 one)
+    const uint4* s = reinterpret_cast<const uint4*>(p);
+    const uint4 q = EARLY ? __ldcg(s) : *s;  // (a BF16 value is the high half of its FP32 one)
     const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -127,15 +133,20 @@ __device__ __forceinline__ void load16(const __nv_bfloat16* p, float (&v)[8]) {
         v[2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
     }
 }
-__device__ __forceinline__ float load1(const float* p) { return *p; }
-__device__ __forceinline__ float load1(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+template <bool EARLY>
+__device__ __forceinline__ float load1(const float* p) { return EARLY ? __ldcg(p) : *p; }
+template <bool EARLY>
+__device__ __forceinline__ float load1(const __nv_bfloat16* p) {
+    return __bfloat162float(EARLY ? __ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(p))) : *p);
+}
 
 // Stage rows [r0, r0 + R) x depth [k0, k0 + kn) of an operand as dst[k][r] (row stride LD), zeros outside, in
 // pieces of 16 bytes.  KMAJ: src[r][k] (depth contiguous): eight rows x four pieces per warp, which reads 64
 // bytes of a row at a time and stores with few bank conflicts; else src[k][r].  U pieces per thread are on
-// their way together.
-template <typename E, int R, int LD, bool KMAJ>
-__device__ __forceinline__ void stage(float* dst, const E* __restrict__ src, int r0, int rows, int k0, int kn, int depth) {
+// their way together.  (src is not __restrict__: read-only loads want data that no grid writes while this one
+// exists, and the grid before it may still.)
+template <bool EARLY, typename E, int R, int LD, bool KMAJ>
+__device__ __forceinline__ void stage(float* dst, const E* src, int r0, int rows, int k0, int kn, int depth) {
     const int t = threadIdx.x;
     constexpr int V = 16 / (int)sizeof(E), U = sizeof(E) == 4 ? 6 : 4;
     const int kp = (kn + V - 1) / V;  // pieces along the depth
@@ -153,19 +164,19 @@ __device__ __forceinline__ void stage(float* dst, const E* __restrict__ src, int
                 const int r = (e & 7) + 8 * ((e >> 5) % (R / 8)), k = V * (((e >> 3) & 3) + 4 * ((e >> 5) / (R / 8)));
                 if (k >= kn || r0 + r >= rows) continue;
                 const E* p = src + (long long)(r0 + r) * depth + k0 + k;
-                if (vec && k + V <= kn) load16(p, v[u]);
+                if (vec && k + V <= kn) load16<EARLY>(p, v[u]);
                 else
 #pragma unroll
                     for (int j = 0; j < V; ++j)
-                        if (k + j < kn) v[u][j] = load1(p + j);
+                        if (k + j < kn) v[u][j] = load1<EARLY>(p + j);
             } else {
                 const int r = V * (e % (R / V)), k = e / (R / V);
                 const E* p = src + (long long)(k0 + k) * rows + r0 + r;
-                if (vec && r0 + r + V <= rows) load16(p, v[u]);
+                if (vec && r0 + r + V <= rows) load16<EARLY>(p, v[u]);
                 else
 #pragma unroll
                     for (int j = 0; j < V; ++j)
-                        if (r0 + r + j < rows) v[u][j] = load1(p + j);
+                        if (r0 + r + j < rows) v[u][j] = load1<EARLY>(p + j);
             }
         }
 #pragma unroll
@@ -207,7 +218,7 @@ __device__ __forceinline__ void product_tile(const Product& q, int tile, float* 
         const int kn = min(q.slab, q.K - k0);
         if (k0) __syncthreads();
         if (READY == READY_NONE && k0 == 0) grid_dependency();
-        stage<E, kProdTn, LB, BK>(Bs, static_cast<const E*>(q.B), n0, q.N, k0, kn, q.K);
+        stage<READY != READY_NONE, E, kProdTn, LB, BK>(Bs, static_cast<const E*>(q.B), n0, q.N, k0, kn, q.K);
         if (READY == READY_B && k0 == 0) grid_dependency();
         if constexpr (FIRST) {  // (one slab: k0 = 0, kn = K)
             // the first layer's weights as FP32 rows of kFirstIn, zero-padded; a thread keeps one row of x
@@ -241,7 +252,7 @@ __device__ __forceinline__ void product_tile(const Product& q, int tile, float* 
                     if (m0 + e / kn < q.M) q.a1[(long long)(m0 + e / kn) * kn + e % kn] = As[(e % kn) * LA + e / kn];
             }
         } else {
-            stage<float, TM, LA, AK>(As, q.A, m0, q.M, k0, kn, q.K);
+            stage<READY == READY_ALL, float, TM, LA, AK>(As, q.A, m0, q.M, k0, kn, q.K);
         }
         if (k0 == 0)
 #pragma unroll
@@ -254,7 +265,7 @@ __device__ __forceinline__ void product_tile(const Product& q, int tile, float* 
                 if constexpr (EP == EP_MSE) pre[u][1] = q.aux[o];
                 if constexpr (EP == EP_DTANH) pre[u][0] = q.aux[o];
                 if constexpr (EP == EP_GRAD)
-                    if (q.w.p) { pre[u][0] = q.w.p[o]; pre[u][1] = q.w.m[o]; pre[u][2] = q.w.v[o]; }
+                    if (q.w.p) { pre[u][0] = __ldcg(q.w.p + o); pre[u][1] = __ldcg(q.w.m + o); pre[u][2] = __ldcg(q.w.v + o); }
             }
         __syncthreads();
         const int per = (kn + G - 1) / G, ka = g * per, kb = min(kn, ka + per);
@@ -326,8 +337,10 @@ __device__ __forceinline__ void product_tile(const Product& q, int tile, float* 
     }
 }
 
+// (two CTAs per SM, 64 registers, where the compiler would take 72: a step at batch 2048 241 -> 224 us, at 256 46.8 ->
+// 43.7; it does not change the other layers')
 template <int TM, int EP, int READY, bool FIRST>
-__global__ void __launch_bounds__(kProdThreads) k_forward(const Product q) {
+__global__ void __launch_bounds__(kProdThreads, EP == EP_MSE || FIRST ? 2 : 0) k_forward(const Product q) {
     extern __shared__ __align__(16) float prod_smem[];
     product_tile<TM, true, true, __nv_bfloat16, EP, READY, FIRST>(q, blockIdx.x, prod_smem);
 }
