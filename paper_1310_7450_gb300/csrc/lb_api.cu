@@ -246,36 +246,34 @@ __global__ void k_set_fields(T* pop, C* drho, C* sig3, const double* u, const do
     }
 }
 
-// The drive of up to kDriveChunk channels, a kernel argument.
-constexpr int kDriveChunk = 128;
-struct DriveArgs {
-    double g[kDriveChunk], u_wall[kDriveChunk];
-};
-
-// Apply the body forces and moving-wall velocities of channels c0 .. c0 + n - 1, and keep a device
-// copy in gx for the kernels that read the drive there.  The values are arguments, so nothing is
-// read from host memory and no staging has to be kept until the kernel ran; launched while the
-// kernel before it still runs (what it reads before the wait is constant after create).  Sixteen
-// steps of 1024 x 1024 FP32 whose drive changes and whose monitor is copied to device memory every
-// step, and the fields: 531 us with a mapped staging slot, an event and a copy, 456 now.
-template <typename C>
-__global__ void __launch_bounds__(kDriveChunk) k_apply_gx(ChanParams<C>* chan, double* gx, const __grid_constant__ DriveArgs d,
-                                                          int c0, int n, int n_ch, int nx) {
-    const int k = threadIdx.x, c = c0 + k;
-    const bool on = k < n, gpbc = on && chan[c].gpbc;
+// Give channels c0 .. c0 + n - 1 the body force (or, WALL, the moving wall's velocity) v, and keep a
+// device copy in gx for the kernels that read the drive there.  A call sets one channel or all of them, to
+// one value: an argument, so nothing is read from host memory and no staging has to be kept until the
+// kernel ran; launched while the kernel before it still runs (what it reads before the wait is constant
+// after create).  Sixteen steps of 1024 x 1024 FP32 whose drive changes and whose monitor is copied to
+// device memory every step, and the fields: 531 us with a mapped staging slot, an event and a copy, 452
+// now.  A force for all of 20 000 channels: 354 us in launches of 128 channels' values, 26 now.
+constexpr int kDriveThreads = 128;
+template <typename C, bool WALL>
+__global__ void __launch_bounds__(kDriveThreads) k_apply_drive(ChanParams<C>* chan, double* gx, double v, int c0, int n, int n_ch,
+                                                               int nx) {
+    const int k = blockIdx.x * kDriveThreads + threadIdx.x, c = c0 + k;
+    const bool on = k < n, gpbc = !WALL && on && chan[c].gpbc;
     const C rho0 = gpbc ? chan[c].rho0_m1 : C(0);
     grid_dependency();
     if (!on) return;
-    const double g = d.g[k], uw = d.u_wall[k];
-    gx[c] = g;
-    gx[n_ch + c] = uw;
-    chan[c].u_wall = (C)uw;
-    if (gpbc) {  // pressure-driven: g sets the ghost densities, there is no body force
-        const double half = 1.5 * g * (double)(nx + 1);
+    if (WALL) {
+        gx[n_ch + c] = v;
+        chan[c].u_wall = (C)v;
+        return;
+    }
+    gx[c] = v;
+    if (gpbc) {  // pressure-driven: v sets the ghost densities, there is no body force
+        const double half = 1.5 * v * (double)(nx + 1);
         chan[c].rho_in = (C)((double)rho0 + half);
         chan[c].rho_out = (C)((double)rho0 - half);
     } else {
-        chan[c].gx = (C)g;
+        chan[c].gx = (C)v;
     }
 }
 
@@ -769,19 +767,15 @@ StepArgs<T, C> base_args(lb_handle* h) {
     return a;
 }
 
-// Body forces and wall velocities: host -> channel table, stream-ordered, by value.
-lb_status push_drive(lb_handle* h) {
-    for (int c0 = 0; c0 < h->n_ch; c0 += kDriveChunk) {
-        const int n = std::min(kDriveChunk, h->n_ch - c0);
-        DriveArgs d{};
-        for (int k = 0; k < n; ++k) {
-            d.g[k] = h->params[c0 + k].g_x;
-            d.u_wall[k] = h->u_wall[c0 + k];
-        }
-        const int threads = (n + 31) / 32 * 32;
-        if (h->csize == 8) LB_CK(launch_dependent(true, k_apply_gx<double>, 1, threads, 0, h->stream, (ChanParams<double>*)h->chan, h->gx_d, d, c0, n, h->n_ch, h->nx));
-        else LB_CK(launch_dependent(true, k_apply_gx<float>, 1, threads, 0, h->stream, (ChanParams<float>*)h->chan, h->gx_d, d, c0, n, h->n_ch, h->nx));
-    }
+// A body force or (WALL) wall velocity of one channel, or all (-1): host -> channel table, stream-ordered, by value.
+template <bool WALL>
+lb_status push_drive(lb_handle* h, int channel, double v) {
+    const int c0 = std::max(channel, 0), n = channel < 0 ? h->n_ch : 1;
+    const int threads = std::min(kDriveThreads, (n + 31) / 32 * 32), grid = (n + kDriveThreads - 1) / kDriveThreads;
+    if (h->csize == 8)
+        LB_CK(launch_dependent(true, k_apply_drive<double, WALL>, grid, threads, 0, h->stream, (ChanParams<double>*)h->chan, h->gx_d, v, c0, n, h->n_ch, h->nx));
+    else
+        LB_CK(launch_dependent(true, k_apply_drive<float, WALL>, grid, threads, 0, h->stream, (ChanParams<float>*)h->chan, h->gx_d, v, c0, n, h->n_ch, h->nx));
     return LB_OK;
 }
 
@@ -1824,18 +1818,18 @@ lb_status lb_residual(lb_handle* h, double* r) {
 lb_status lb_set_body_force(lb_handle* h, int channel, double g_x) {
     if (!h || channel < -1 || channel >= h->n_ch || std::isnan(g_x) || std::isinf(g_x))
         return fail(LB_EINVAL, "lb_set_body_force: bad argument%s");
-    for (int c = 0; c < h->n_ch; ++c)
-        if (channel < 0 || c == channel) h->params[c].g_x = g_x;
-    return push_drive(h);
+    if (channel >= 0) h->params[channel].g_x = g_x;
+    else for (lb_params& p : h->params) p.g_x = g_x;
+    return push_drive<false>(h, channel, g_x);
 }
 
 lb_status lb_set_wall_velocity(lb_handle* h, int channel, double u_wall) {
     if (!h || channel < -1 || channel >= h->n_ch || std::isnan(u_wall) || std::isinf(u_wall))
         return fail(LB_EINVAL, "lb_set_wall_velocity: bad argument%s");
     if (!h->moving) return fail(LB_EINVAL, "lb_set_wall_velocity: the handle has no moving wall%s");
-    for (int c = 0; c < h->n_ch; ++c)
-        if (channel < 0 || c == channel) h->u_wall[c] = u_wall;
-    return push_drive(h);
+    if (channel >= 0) h->u_wall[channel] = u_wall;
+    else h->u_wall.assign(h->n_ch, u_wall);
+    return push_drive<true>(h, channel, u_wall);
 }
 
 // The start state of every channel from device fields in node order (u [node][2], rho, drho or
