@@ -278,10 +278,15 @@ __global__ void __launch_bounds__(kDriveThreads) k_apply_drive(ChanParams<C>* ch
 }
 
 // Copy n doubles of device memory to mapped pinned host memory or to device memory (the monitor's
-// way out: no copy-engine transfer in the stream, and set up while the step before it runs).
+// way out: no copy-engine transfer in the stream, and set up while the step before it runs).  20 000
+// channels (640 KB) to device memory: 102 us by one block of 128 threads, 2.8 by one thread per value.
 __global__ void k_copy_out(const double* src, double* dst, int n) {
     grid_dependency();
-    for (int k = threadIdx.x; k < n; k += blockDim.x) dst[k] = src[k];
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n) dst[k] = src[k];
+}
+cudaError_t copy_out(const double* src, double* dst, int n, cudaStream_t s) {
+    return launch_dependent(true, k_copy_out, (n + 127) / 128, 128, 0, s, src, dst, n);
 }
 
 // Per-channel reduction of the step's block partials, one warp per channel in a fixed order
@@ -1771,7 +1776,7 @@ lb_status lb_get_fields(lb_handle* h, void* u, void* sigma, void* rho, int out_d
 lb_status lb_monitor(lb_handle* h, double* out) {
     if (!h || !out) return fail(LB_EINVAL, "lb_monitor: null argument%s");
     if (h->mon_state < 0) return fail(LB_ESTATE, "lb_monitor: no monitor evaluated yet (run lb_step with n >= 2)%s");
-    LB_CK(launch_dependent(true, k_copy_out, 1, 128, 0, h->stream, h->mon_d, h->mon_hd, 4 * h->n_ch));
+    LB_CK(copy_out(h->mon_d, h->mon_hd, 4 * h->n_ch, h->stream));
     LB_CK(cudaStreamSynchronize(h->stream));
     std::memcpy(out, h->mon_h, 4 * h->n_ch * sizeof(double));
     return LB_OK;
@@ -1789,7 +1794,7 @@ lb_status lb_monitor_async(lb_handle* h, double* out) {
     const bool known = cudaPointerGetAttributes(&at, out) == cudaSuccess && at.devicePointer && cudaGetDevice(&dev) == cudaSuccess;
     if (known && (at.type == cudaMemoryTypeHost || (at.type == cudaMemoryTypeDevice && at.device == dev)) &&
         (uintptr_t)at.devicePointer % sizeof(double) == 0) {
-        LB_CK(launch_dependent(true, k_copy_out, 1, 128, 0, h->stream, h->mon_d, (double*)at.devicePointer, 4 * h->n_ch));
+        LB_CK(copy_out(h->mon_d, (double*)at.devicePointer, 4 * h->n_ch, h->stream));
     } else {
         (void)cudaGetLastError();
         LB_CK(cudaMemcpyAsync(out, h->mon_d, 4 * h->n_ch * sizeof(double), cudaMemcpyDefault, h->stream));

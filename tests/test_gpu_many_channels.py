@@ -1,5 +1,6 @@
-"""Drive of handles with more channels than one block has threads: a force (wall velocity) given to all channels and
-then to single ones, at the edges of the blocks, against the same values given at create."""
+"""Handles with more channels than one block has threads.  Their drive: a force (wall velocity) given to all channels and
+then to single ones, at the edges of the blocks, against the same values given at create.  Their monitor, into
+device and pinned memory, against the blocking call."""
 import numpy as np
 import pytest
 
@@ -45,3 +46,21 @@ def test_all_then_single_channels(prec, kw):
             out.append([np.concatenate([x.reshape(-1) for x in p]) for p in sim.populations()] + [sim.monitor()])
     for x, y in zip(*out):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("n_ch", [31, 32, 33, 1500])
+def test_monitor_reaches_every_kind_of_memory(n_ch):
+    import torch
+    p = dict(inputs.matched_params(0.9, 50.0, 0.1, 1e-3, 1e-5), rho_pert_amp=1e-3)
+    with lbnlm.Channels(4, [5] * n_ch, [dict(p, seed=c + 1) for c in range(n_ch)], "f32",
+                        stream=torch.cuda.current_stream().cuda_stream) as sim:
+        sim.step(4)
+        want = np.asarray(sim.monitor()).reshape(-1)
+        assert len(set(want[1::4])) > n_ch // 2                            # (channels differ)
+        dev = torch.zeros(4 * n_ch + 2, dtype=torch.float64, device="cuda")
+        pin = torch.zeros(4 * n_ch + 2, dtype=torch.float64).pin_memory()
+        for dst in (dev, pin):
+            lbnlm.lb_monitor_async(sim.h, dst[1:-1])
+        torch.cuda.synchronize()
+        for got in (dev.cpu().numpy(), pin.numpy()):
+            assert np.array_equal(got[1:-1], want) and got[0] == got[-1] == 0.0
