@@ -583,15 +583,28 @@ bool make_pop_map(const lb_handle* h, void* base, CUtensorMap* map) {
     return r == CUDA_SUCCESS;
 }
 
+// Programmatic dependent launch takes about 2 us off a march step, but lets blocks land on whichever SM frees a
+// slot first, against the plan that deals rows by a block's rank on its SM.  us per step without / with:
+// FP32 1024 x 1024 22.5 / 20.7, 2048 x 2048 72.6 / 71.2, 4096 x 4096 252 / 257; BF16 1024 x 1024 20.7 / 20.1,
+// 8192 x 2048 214 / 236.  With pressure-driven ends (a column kernel before every step): FP32 2048 x 1000 52.0 / 56.5; BF16 2048 x 1000 47.0 / 43.8, 256 x 8192 63.2 / 60.7, 4096 x 4096 257.6 / 255.7.
+static bool march_dependent(int prec, bool gpbc, long long nodes) {
+    if (gpbc) return prec == LB_PREC_BF16;
+    return nodes <= (prec == LB_PREC_BF16 ? 1 << 21 : 1 << 22);
+}
+
 // Constants measured with six CTAs of two warps per SM (us per step, one GPU):
 //   FP32 4096 x 4096: skew 0.06: 251.9, 0.12: 252.9, 0: 252.7, 0.2: 257.7; f = 1.2 252.9, 1.05: 264.0,
 //     1.35: 253.6; pressure-driven ends at 2048 x 1000 f = 1.7: 51.8, 1.5: 53.7, 1.3: 55.5, 1.2: 59.7.
 //   BF16 8192 x 2048: skew 0.3 f = 1.15: 214.4; f = 1.3: 212.8 (but leaves CTAs idle with eight per SM); f = 1.05: 228.4; skew 0.15 / 0.22 with
 //     f = 1.15: 214.5 / 214.9; skew 0.4: 228.6.
-//   BF16, pressure-driven ends, 4096 x 4096 / 2048 x 1000 / 256 x 8192: skew 0.22 f = 1.6: 258.0 / 47.4 / 63.1;
-//     0.3, 1.5: 254.5 / 49.5 / 64.0; 0.15, 1.5: 258.8 / 47.5 / 63.7; 0.15, 1.3: 264.7 / 49.5 / 63.7; 0, 1.5: 264.7 / 48.8 / 63.4.
-static MarchModel march_model(int prec, bool gpbc) {
-    if (prec == LB_PREC_BF16) return gpbc ? MarchModel{0.22, 1.6, true} : MarchModel{0.30, 1.15, true};
+//   BF16, pressure-driven ends, 4096 x 4096 / 2048 x 1000 / 256 x 8192 / 640 x 4096: skew 0.16 f = 1.4: 251.4 / 45.7 /
+//     60.9 / 63.0; f = 1.3: 261.8 / 47.6 / 61.0 / 64.3; f = 1.5: 255.5 / 45.1 / 60.8 / 62.2; skew 0.3, 1.5: 251.1 / 45.7 / 61.9 /
+//     63.0; skew 0, 1.4: 262.3 / 45.6 / 61.0 / 62.6.
+//   BF16 grids whose steps are launched while the one before runs: blocks land wherever a slot is free first, not rank by
+//     rank, so no skew: 256 x 8192 35.5 (skew 0.3: 40.1), 384 x 4096 26.9 (29.6), 1024 x 1024 19.7 (20.4).
+static MarchModel march_model(int prec, bool gpbc, long long nodes) {
+    if (prec == LB_PREC_BF16)
+        return gpbc ? MarchModel{0.16, 1.4, true} : MarchModel{march_dependent(prec, gpbc, nodes) ? 0.0 : 0.30, 1.15, true};
     return {0.08, gpbc ? 1.6 : 1.2, true};
 }
 
@@ -645,7 +658,7 @@ lb_status plan_march(lb_handle* h) {
     if (bps < 1) return LB_OK;
     const int slots = bps * nsm;
     const std::vector<MarchItem> items = short_items(
-        fine_items(march_plan(h->nx, h->ny[0], bps, nsm, march_model(h->prec, h->gpbc)), h->nx, h->ny[0], slots), h->nx);
+        fine_items(march_plan(h->nx, h->ny[0], bps, nsm, march_model(h->prec, h->gpbc, h->nodes)), h->nx, h->ny[0], slots), h->nx);
     LB_CK(cudaMalloc(&h->march_items_d, sizeof(MarchItem) * items.size()));
     LB_CK(cudaMemcpy(h->march_items_d, items.data(), sizeof(MarchItem) * items.size(), cudaMemcpyHostToDevice));
     h->n_march_items = (int)items.size();
@@ -834,21 +847,13 @@ void march_monitor(lb_handle* h, int flags, MarchCtl& ctl) {
     ctl.with_residual = (flags & F_RESID) ? 1 : 0;
 }
 
-// Programmatic dependent launch takes about 2 us off a march step, but lets blocks land on whichever SM frees a
-// slot first, against the plan that deals rows by a block's rank on its SM.  us per step without / with:
-// FP32 1024 x 1024 22.5 / 20.7, 2048 x 2048 72.6 / 71.2, 4096 x 4096 252 / 257; BF16 1024 x 1024 20.7 / 20.1,
-// 8192 x 2048 214 / 236; pressure-driven ends (a column kernel before every step) FP32 2048 x 1000 52.0 / 56.5.
-bool march_dependent(const lb_handle* h) {
-    return !h->gpbc && h->nodes <= (h->prec == LB_PREC_BF16 ? 1 << 21 : 1 << 22);
-}
-
 // The row-march kernel: a step, or (F_FIELDS) the fields of the stored state.
 template <typename T, bool FIELDS>
 cudaError_t launch_march_as(lb_handle* h, const StepArgs<T, float>& a) {
     // (the fields pass has its own wait limit: lb_set_wait_limit speaks of steps)
     MarchCtl ctl{h->march_items_d, h->n_march_items, h->status_d, h->P[0], h->base[0], FIELDS ? kDefaultWaitNs : h->wait_ns};
     march_monitor(h, a.flags, ctl);
-    ctl.dependent = march_dependent(h);
+    ctl.dependent = march_dependent(h->prec, h->gpbc, h->nodes);
     const CUtensorMap& m = ((const void*)a.pin == h->mapA_buf) ? h->mapA : h->mapB;
     return march_variant(h, [&](auto sm, auto bnd, auto sch, auto strip) {
         return launch_step_march<T, float, decltype(sm)::value, decltype(bnd)::value, decltype(sch)::value, FIELDS,
@@ -1714,7 +1719,7 @@ int lb_row_march_plan(int nx, int ny, int ctas_per_sm, int n_sm, int precision, 
     if (nx <= 0 || nx % kMarchW != 0 || ny < 16 || ctas_per_sm < 1 || n_sm < 1 || max_items < 0 ||
         (precision != LB_PREC_F32 && precision != LB_PREC_BF16))
         return -LB_EINVAL;
-    const std::vector<MarchItem> v = march_plan(nx, ny, ctas_per_sm, n_sm, march_model(precision, gpbc != 0));
+    const std::vector<MarchItem> v = march_plan(nx, ny, ctas_per_sm, n_sm, march_model(precision, gpbc != 0, (long long)nx * ny));
     if (items) {
         if ((int)v.size() > max_items) return -LB_EINVAL;
         for (size_t i = 0; i < v.size(); ++i) {

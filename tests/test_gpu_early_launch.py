@@ -12,6 +12,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny,prec,flags,kw", [
     (1024, 512, "f32", 0, {}), (1000, 777, "bf16", 0, {}), (1001, 777, "f32", 0, dict(stress_mode=1)),
     (640, 640, "f32", lbnlm.LB_GRID_TILE_ONLY, {}), (640, 640, "bf16", lbnlm.LB_GRID_TILE_ONLY, {}),
+    (1000, 512, "bf16", 0, dict(x_mode="gpbc")), (256, 2048, "bf16", 0, dict(x_mode="gpbc", stress_mode=1)),
     (100, 300, "f32", 0, dict(walls="couette", stress_mode=1)), (256, 257, "f64", 0, {}), (100, 60, "f32", 0, dict(x_mode="gpbc")),
     (256, 200, "bf16", lbnlm.LB_GRID_STRESS_DIVERGENCE, {}), (1024, 300, "f32", lbnlm.LB_GRID_RELAXATION_MODEL, {})])
 def test_steps_launched_early_equal_steps_alone(nx, ny, prec, flags, kw):
