@@ -1,8 +1,8 @@
 """Build the CUDA library ``liblbnlm.so`` (sm_103a) in-tree with nvcc.
 
 Each translation unit under ``csrc/`` is compiled in parallel, then linked into one shared
-library next to this file.  No fast-math: IEEE division and square root, FMA contraction
-allowed.
+library next to this file.  No fast-math; FMA contraction allowed.  (The kernels' own FP32 and
+FP64 reciprocals and square roots, and their errors, stand in ``csrc/lb_device.cuh``.)
 """
 from __future__ import annotations
 
