@@ -277,6 +277,11 @@ template <> struct Arith<double> {
         g = __fma_rn(__fma_rn(-g, g, x), h, g);
         return x >= 2.2250738585072014e-308 ? g : (x >= 0.0 ? 0.0 : (double)NAN);
     }
+    // a / b for any b: zero, infinite or near the ends of the range as the language divides (a branch on the exponent)
+    static __device__ __forceinline__ double div_any(double a, double b) {
+        const unsigned hi = (unsigned)__double2hiint(b) & 0x7fffffffu;
+        return hi - 0x00200000u < 0x7fd00000u - 0x00200000u ? div(a, b) : a / b;
+    }
     static __device__ __forceinline__ double exp(double x) { return ::exp(x); }
 };
 #ifdef LBK_FP32_IEEE
@@ -285,6 +290,7 @@ template <> struct Arith<double> {
 template <> struct Arith<float> {
     static __device__ __forceinline__ float rcp(float x) { return __frcp_rn(x); }
     static __device__ __forceinline__ float div(float a, float b) { return __fdiv_rn(a, b); }
+    static __device__ __forceinline__ float div_any(float a, float b) { return div(a, b); }
     static __device__ __forceinline__ float sqrt(float x) { return __fsqrt_rn(x); }
     static __device__ __forceinline__ float exp(float x) { return expf(x); }
 };
@@ -296,6 +302,7 @@ template <> struct Arith<float> {
         return r;
     }
     static __device__ __forceinline__ float div(float a, float b) { return a * rcp(b); }
+    static __device__ __forceinline__ float div_any(float a, float b) { return div(a, b); }
     static __device__ __forceinline__ float sqrt(float x) {
         float r;
         asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -537,7 +544,7 @@ __device__ __forceinline__ C relaxation_time_ext(const ChanParams<C>& P, C ka, C
     C tau = P.tau;
     if (P.beta_rho != C(0) && tau > C(0)) {
         const C rho_hat = C(1) + dR - drho_prev;
-        tau *= Arith<C>::exp(Arith<C>::div(P.beta_rho * (rho_hat - P.rho_ref), P.rho_ref));
+        tau *= Arith<C>::exp(Arith<C>::div_any(P.beta_rho * (rho_hat - P.rho_ref), P.rho_ref));
     }
     const C Dxx = C(2) * ka, Dxy = kb + kc, Dyy = C(2) * ke;
     const C sII = Arith<C>::sqrt(C(0.5) * (Dxx * Dxx + C(2) * Dxy * Dxy + Dyy * Dyy));
@@ -546,11 +553,12 @@ __device__ __forceinline__ C relaxation_time_ext(const ChanParams<C>& P, C ka, C
         // 1/tau and the weight 1/(tau_f + 1) are formed in the arithmetic type (the FP32 reciprocal
         // in the FP32 modes: FP64 divisions on this part would bound the step), the recursion in FP64
         // as an increment, phi = phi_old + (phi_ss - phi_old) / (tau_f + 1) -- the same backward
-        // Euler step, whose fixed point is phi_ss exactly whatever the rounding of the weight
-        const double phi_ss = (double)Arith<C>::div(C(1), tau) + (double)sII * (double)P.inv_gc;
+        // Euler step, whose fixed point is phi_ss exactly whatever the rounding of the weight (an infinite tau leaves
+        // the shear rate's part of it)
+        const double phi_ss = (double)Arith<C>::div_any(C(1), tau) + (double)sII * (double)P.inv_gc;
         const double w = (double)Arith<C>::div(C(1), P.tau_f + C(1));
         *phi = phi_old > 0.0 ? phi_old + (phi_ss - phi_old) * w : phi_ss;
-        return Arith<C>::div(C(1), (C)*phi);
+        return Arith<C>::div_any(C(1), (C)*phi);
     }
     return Arith<C>::div(tau, C(1) + tau * sII * P.inv_gc);
 }
