@@ -41,8 +41,10 @@ __device__ inline double grid_d(int k) { return (k + 0.5) / kWsGrid * 2.0 - 1.0;
 
 // Square root of a positive normal number: the hardware's reciprocal square root, one Goldschmidt step and
 // a final Newton correction by the residual (P. Markstein, IBM J. Res. Dev. 34, 1990): 7 FP64 operations,
-// 0.500 units of the last place at most over 2^28 arguments of exponents within +-300.
+// 0.500 units of the last place at most over 2^28 arguments of exponents within +-300.  Anything else (0 or subnormal, as
+// at the wall of a fluid with a tiny critical strain) takes the library's.
 __device__ __forceinline__ double ws_sqrt(double x) {
+    if ((unsigned)__double2hiint(x) - 0x00100000u >= 0x7fe00000u) return sqrt(x);
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     double g = x * y, h = 0.5 * y;
