@@ -15,6 +15,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <limits>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -488,7 +489,7 @@ std::vector<ChanParams<C>> make_chan(const lb_handle* h) {
             q.rho_in = (C)((p.rho0 - 1.0) + 1.5 * p.g_x * (double)(h->nx + 1));
             q.rho_out = (C)((p.rho0 - 1.0) - 1.5 * p.g_x * (double)(h->nx + 1));
         }
-        q.tau_c = C(0.5) * q.tau * q.inv_gc;
+        q.tau_c = std::min(C(0.5) * q.tau * q.inv_gc, std::numeric_limits<C>::max());  // (finite: times no shear it is 0)
         q.cDh = C(0.5) * q.cD;
         q.m15k = C(-1.5) * q.kdr;
         q.om3 = C(3) * q.omega;
