@@ -416,7 +416,6 @@ struct lb_handle {
     std::vector<double> sweep_key;          // ... for these arguments and configurations
     const void* sweep_pin = nullptr;        // ... and this population buffer
     MarchItem* march_items_d = nullptr;
-    int* march_item_begin_d = nullptr;  // {0, n_march_items}: the residual reduction's item range
     int n_march_items = 0, march_grid = 0;
     // resident stepping of a small single channel: CTAs of its cluster (0: not used), threads, shared memory
     int res_cl = 0, res_threads = 0;
@@ -663,9 +662,6 @@ lb_status plan_march(lb_handle* h) {
     LB_CK(cudaMalloc(&h->march_items_d, sizeof(MarchItem) * items.size()));
     LB_CK(cudaMemcpy(h->march_items_d, items.data(), sizeof(MarchItem) * items.size(), cudaMemcpyHostToDevice));
     h->n_march_items = (int)items.size();
-    const int ib[2] = {0, h->n_march_items};
-    LB_CK(cudaMalloc(&h->march_item_begin_d, sizeof(ib)));
-    LB_CK(cudaMemcpy(h->march_item_begin_d, ib, sizeof(ib), cudaMemcpyHostToDevice));
     if ((int)h->items.size() < h->n_march_items) {  // the partials buffer serves both plans
         cudaFree(h->partials);
         h->partials = nullptr;
@@ -726,7 +722,6 @@ void release(lb_handle* h) {
     free_dev(h->hstage);
     free_dev(h->ws_prm); free_dev(h->ws_row_off); free_dev(h->ws_rows); free_dev(h->ws_grid); free_dev(h->ws_scale);
     free_dev(h->march_items_d);
-    free_dev(h->march_item_begin_d);
     free_dev(h->sweep_steps_d);
     free_dev(h->sweep_res_d);
     free_dev(h->sweep_order_d);

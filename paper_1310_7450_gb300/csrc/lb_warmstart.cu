@@ -23,20 +23,6 @@ struct WsChan {
     double G, tau0, theta, gamma_c;  // G_inf, tau0, theta, gamma_c of the channel (the force is read where it is set)
 };
 
-// Linear interpolation of f (n points at x0 + i h) at x, end values held (np.interp on a uniform
-// abscissa).
-__device__ inline double interp_uniform(double x, double x0, double h, const double* f, int n, int stride = 1) {
-    if (x <= x0) return f[0];
-    const double xe = x0 + (n - 1) * h;
-    if (x >= xe) return f[(n - 1) * stride];
-    int i = (int)floor((x - x0) / h);
-    if (i > n - 2) i = n - 2;
-    if (i < 0) i = 0;
-    const double xa = x0 + i * h;
-    const double t = (x - xa) / h;
-    return f[i * stride] + t * (f[(i + 1) * stride] - f[i * stride]);
-}
-
 __device__ inline double grid_d(int k) { return (k + 0.5) / kWsGrid * 2.0 - 1.0; }
 
 // Square root of a positive normal number: the hardware's reciprocal square root, one Goldschmidt step and
