@@ -660,7 +660,8 @@ lb_status plan_march(lb_handle* h) {
     const std::vector<MarchItem> items = short_items(
         fine_items(march_plan(h->nx, h->ny[0], bps, nsm, march_model(h->prec, h->gpbc, h->nodes)), h->nx, h->ny[0], slots), h->nx);
     LB_CK(cudaMalloc(&h->march_items_d, sizeof(MarchItem) * items.size()));
-    LB_CK(cudaMemcpy(h->march_items_d, items.data(), sizeof(MarchItem) * items.size(), cudaMemcpyHostToDevice));
+    LB_CK(cudaMemcpyAsync(h->march_items_d, items.data(), sizeof(MarchItem) * items.size(), cudaMemcpyHostToDevice, h->stream));
+    LB_CK(cudaStreamSynchronize(h->stream));  // (the host copy goes)
     h->n_march_items = (int)items.size();
     if ((int)h->items.size() < h->n_march_items) {  // the partials buffer serves both plans
         cudaFree(h->partials);
@@ -1216,7 +1217,8 @@ lb_status sweep_order(lb_handle* h, int* n_active, const std::vector<char>* only
         LB_CK(cudaMalloc(&h->sweep_res_d, sizeof(double) * h->n_ch));
     }
     if (!order.empty())
-        LB_CK(cudaMemcpy(h->sweep_order_d, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice));
+        LB_CK(cudaMemcpyAsync(h->sweep_order_d, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, h->stream));
+    LB_CK(cudaStreamSynchronize(h->stream));  // (the host copy goes)
     std::vector<SweepGroup> groups;
     for (int k = 0; k < (int)order.size(); ++k) {
         const int ny = h->ny[order[k]];
@@ -1415,7 +1417,7 @@ lb_status lb_run_until_steady(lb_handle* h, double tol, long check_every, long m
         }
         const long long L = std::min(seg, ms - done);
         std::vector<long long> init(h->n_ch, -3);
-        LB_CK(cudaMemcpy(h->sweep_steps_d, init.data(), sizeof(long long) * h->n_ch, cudaMemcpyHostToDevice));
+        LB_CK(cudaMemcpyAsync(h->sweep_steps_d, init.data(), sizeof(long long) * h->n_ch, cudaMemcpyHostToDevice, h->stream));
         st = sweep_run(h, tol, (int)check_every, L);
         if (st != LB_OK) return st;
         LB_CK(cudaMemcpyAsync(seg_steps.data(), h->sweep_steps_d, sizeof(long long) * h->n_ch, cudaMemcpyDeviceToHost, h->stream));
@@ -1621,7 +1623,8 @@ lb_status lb_create(const lb_grid* grid, const lb_params* params, const lb_bound
     e = cudaEventCreateWithFlags(&h->status_ev, cudaEventDisableTiming);
     if (e != cudaSuccess) return bail(cuda_fail(e, "lb_create: cudaEventCreate"));
 
-    // tables (synchronous copies: creation is not on the hot path)
+    // tables, in the order of the handle's stream (a cudaMemcpy from pageable memory may return before its data have
+    // arrived, and a non-blocking stream does not wait for them); the stream is waited for below
     std::vector<double> gx(2 * h->n_ch, 0.0);
     std::vector<InitChan> ic(h->n_ch);
     for (int c = 0; c < h->n_ch; ++c) {
@@ -1634,21 +1637,23 @@ lb_status lb_create(const lb_grid* grid, const lb_params* params, const lb_bound
     e = cudaMalloc(&ic_d, sizeof(InitChan) * h->n_ch);
     if (e != cudaSuccess) return bail(cuda_fail(e, "lb_create: cudaMalloc"));
     bool ok = true;
-    ok &= cudaMemcpy(ic_d, ic.data(), sizeof(InitChan) * h->n_ch, cudaMemcpyHostToDevice) == cudaSuccess;
+    ok &= cudaMemcpyAsync(ic_d, ic.data(), sizeof(InitChan) * h->n_ch, cudaMemcpyHostToDevice, h->stream) == cudaSuccess;
     if (h->csize == 8) {
         auto v = make_chan<double>(h);
-        ok &= cudaMemcpy(h->chan, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+        ok &= cudaMemcpyAsync(h->chan, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice, h->stream) == cudaSuccess;
+        ok &= cudaStreamSynchronize(h->stream) == cudaSuccess;  // (v goes)
     } else {
         auto v = make_chan<float>(h);
-        ok &= cudaMemcpy(h->chan, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+        ok &= cudaMemcpyAsync(h->chan, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice, h->stream) == cudaSuccess;
+        ok &= cudaStreamSynchronize(h->stream) == cudaSuccess;  // (v goes)
     }
-    ok &= cudaMemcpy(h->items_d, h->items.data(), sizeof(WorkItem) * h->items.size(), cudaMemcpyHostToDevice) == cudaSuccess;
-    ok &= cudaMemcpy(h->item_begin_d, h->item_begin.data(), sizeof(int) * (h->n_ch + 1), cudaMemcpyHostToDevice) == cudaSuccess;
-    ok &= cudaMemcpy(h->base_d, h->base.data(), sizeof(long long) * h->n_ch, cudaMemcpyHostToDevice) == cudaSuccess;
-    ok &= cudaMemcpy(h->P_d, h->P.data(), sizeof(long long) * h->n_ch, cudaMemcpyHostToDevice) == cudaSuccess;
-    ok &= cudaMemcpy(h->node_off_d, h->node_off.data(), sizeof(long long) * h->n_ch, cudaMemcpyHostToDevice) == cudaSuccess;
-    ok &= cudaMemcpy(h->ny_d, h->ny.data(), sizeof(int) * h->n_ch, cudaMemcpyHostToDevice) == cudaSuccess;
-    ok &= cudaMemcpy(h->gx_d, gx.data(), sizeof(double) * 2 * h->n_ch, cudaMemcpyHostToDevice) == cudaSuccess;
+    ok &= cudaMemcpyAsync(h->items_d, h->items.data(), sizeof(WorkItem) * h->items.size(), cudaMemcpyHostToDevice, h->stream) == cudaSuccess;
+    ok &= cudaMemcpyAsync(h->item_begin_d, h->item_begin.data(), sizeof(int) * (h->n_ch + 1), cudaMemcpyHostToDevice, h->stream) == cudaSuccess;
+    ok &= cudaMemcpyAsync(h->base_d, h->base.data(), sizeof(long long) * h->n_ch, cudaMemcpyHostToDevice, h->stream) == cudaSuccess;
+    ok &= cudaMemcpyAsync(h->P_d, h->P.data(), sizeof(long long) * h->n_ch, cudaMemcpyHostToDevice, h->stream) == cudaSuccess;
+    ok &= cudaMemcpyAsync(h->node_off_d, h->node_off.data(), sizeof(long long) * h->n_ch, cudaMemcpyHostToDevice, h->stream) == cudaSuccess;
+    ok &= cudaMemcpyAsync(h->ny_d, h->ny.data(), sizeof(int) * h->n_ch, cudaMemcpyHostToDevice, h->stream) == cudaSuccess;
+    ok &= cudaMemcpyAsync(h->gx_d, gx.data(), sizeof(double) * 2 * h->n_ch, cudaMemcpyHostToDevice, h->stream) == cudaSuccess;
     ok &= cudaMemsetAsync(h->status_d, 0, sizeof(int) * h->n_ch, h->stream) == cudaSuccess;
     if (h->gcount) ok &= cudaMemsetAsync(h->gcount, 0, 2 * h->n_ch * sizeof(unsigned), h->stream) == cudaSuccess;
     ok &= cudaMemsetAsync(h->done_count_d, 0, sizeof(unsigned), h->stream) == cudaSuccess;
@@ -1694,10 +1699,12 @@ lb_status lb_set_relaxation_model(lb_handle* h, int channel, double beta_rho, do
     LB_CK(cudaStreamSynchronize(h->stream));
     if (h->csize == 8) {
         auto v = make_chan<double>(h);
-        LB_CK(cudaMemcpy(h->chan, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice));
+        LB_CK(cudaMemcpyAsync(h->chan, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice, h->stream));
+        LB_CK(cudaStreamSynchronize(h->stream));  // (v goes)
     } else {
         auto v = make_chan<float>(h);
-        LB_CK(cudaMemcpy(h->chan, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice));
+        LB_CK(cudaMemcpyAsync(h->chan, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice, h->stream));
+        LB_CK(cudaStreamSynchronize(h->stream));  // (v goes)
     }
     return LB_OK;
 }
