@@ -51,9 +51,9 @@ typedef enum {
 enum { LB_PREC_F64 = 0, LB_PREC_F32 = 1, LB_PREC_BF16 = 2, LB_PREC_F64S_F32M = 3, LB_PREC_F32S_F64M = 4 };
 enum { LB_STRESS_INLM = 0, LB_STRESS_TIMESTEPPED = 1 };
 /* lb_grid.flags: LB_GRID_STORE_SIGMA writes the 4-component stress every step; LB_GRID_TILE_ONLY
- * keeps every step on the general tile kernel (single FP32/BF16 channels otherwise use, from a few
- * 100 000 nodes up, the
- * row-march kernel); LB_GRID_BF16_STOCHASTIC rounds BF16 populations stochastically (unbiased:
+ * keeps every step on the general tile kernel (single FP32/BF16 channels of 16 rows or more otherwise
+ * use the row-march kernel: at any size where nx is a multiple of 128, from 400 000 nodes (FP32) or
+ * 150 000 (BF16) up at other nx >= 96); LB_GRID_BF16_STOCHASTIC rounds BF16 populations stochastically (unbiased:
  * increments below half a BF16 step survive on average) instead of to nearest;
  * LB_GRID_NO_GRAPH launches every step separately (by default lb_step replays runs of plain
  * tile-kernel steps from a captured CUDA graph, and keeps a small single channel on chip for a run
@@ -192,8 +192,9 @@ lb_status lb_set_monitor_mode(lb_handle *h, int mode);
 lb_status lb_monitor_async(lb_handle *h, double *out);
 
 /* Change the body force of one channel (channel = -1: all), e.g. 0 for cessation.  Stream-
- * ordered: a small kernel on the handle's stream, whose arguments hold the values, applies it to
- * every step enqueued after this call; the call does not wait for the steps enqueued before it. */
+ * ordered: a small kernel on the handle's stream, whose arguments hold the value, applies it to
+ * every step enqueued after this call; the call does not wait for the steps enqueued before it.
+ * Inside a stream capture the value becomes part of the graph: every replay sets it again. */
 lb_status lb_set_body_force(lb_handle *h, int channel, double g_x);
 
 /* Set the velocity of the moving wall of one channel (channel = -1: all) of a LB_WALLS_COUETTE
@@ -301,7 +302,8 @@ lb_status lb_field_monitor_static(const void *u_now, const void *u_prev, int dty
  * rho = 1, delta rho = -(3/2) N1(y), as lb_set_fields does.  lb_warmstart_targets: the network
  * targets of the handle's current state (column x = 0 of each row) into targets (device,
  * [n_channels][768], FP32).  Both need G_inf > 0, tau0 > 0 and g_x > 0 in every channel
- * (LB_EINVAL); both run on the handle's stream (apply synchronises it). */
+ * (LB_EINVAL); both run on the handle's stream (apply synchronises it; so does the first call of a
+ * handle, whose tables it uploads). */
 lb_status lb_warmstart_apply(lb_handle *h, const float *pred, const float *t_mu, const float *t_sd);
 lb_status lb_warmstart_targets(lb_handle *h, float *targets);
 
@@ -350,7 +352,8 @@ int lb_uses_row_march(const lb_handle *h);  /* 1 if plain steps run on the row-m
  * slower under the warp schedulers' age priority; the two edge strips cost more per row).  Grids
  * of three or more strips give all interior strips the same row boundaries (their halo reads then
  * hit L2).  This is the plan of grids that fill those CTAs with items of 8 rows; the library cuts smaller
- * ones finer (2 rows at least).
+ * ones finer (2 rows at least).  Widths that are no multiple of 128 march too, in strips of one
+ * width and a narrower last one; this call does not give their plan.
  * precision LB_PREC_F32 or LB_PREC_BF16, gpbc nonzero for pressure-driven ends (the model's edge
  * cost depends on both).  Writes (x0, y0, y1) per item into items[3 * max_items] (caller-owned
  * host memory; items may be NULL to query the count) and returns the number of items, or

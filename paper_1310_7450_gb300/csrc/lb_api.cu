@@ -626,11 +626,12 @@ auto march_variant(const lb_handle* h, F&& f) {
     return with_mode(Num<0>{}, Num<0>{});
 }
 
-// Whole strips always march; other widths where that is the faster kernel.  A march step lasts 10 us at least (a
-// chain of rows), a tile step 5, but the tile kernel takes 1.3 to 2 times as long per node.  Tile / march, us:
-// FP32 100 x 1600 10.1 / 12.7, 200 x 1600 15.8 / 16.8, 500 x 800 17.5 / 16.8, 1000 x 777 30.1 / 23.0, 1001 x 777
-// 30.7 / 25.0, 2049 x 600 52.3 / 35.0; BF16 200 x 400 9.4 / 10.6, 70 x 2000 16.2 / 15.7, 100 x 1600 16.0 / 13.3,
-// 1000 x 300 18.1 / 13.5, 1001 x 777 44.8 / 26.8.  Below 96 columns half of a strip's threads have none.
+// Whole strips always march, which makes small ones slower than they need be in FP32; other widths where that is the faster
+// kernel.  A march step lasts 7 us at least (a chain of rows), a tile step 4, but the tile kernel takes 1.3 to 2
+// times as long per node.  Tile / march, us: FP32 128 x 16 3.9 / 7.1, 128 x 512 5.4 / 7.6, 1024 x 128 7.8 / 9.3, 512 x
+// 512 11.7 / 10.7, 100 x 1600 10.1 / 12.7, 200 x 1600 15.8 / 16.8, 500 x 800 17.5 / 16.8, 1000 x 777 30.1 / 23.0, 2049 x 600
+// 52.3 / 35.0; BF16 128 x 16 7.2 / 7.0, 512 x 512 15.5 / 10.0, 200 x 400 9.4 / 10.6, 70 x 2000 16.2 / 15.7, 100 x 1600 16.0 /
+// 13.3, 1000 x 300 18.1 / 13.5, 1001 x 777 44.8 / 26.8.  Below 96 columns half of a strip's threads have none.
 static bool march_pays(const lb_handle* h) {
     if (h->nx % kMarchW == 0) return true;
     return h->nx >= 96 && march_strip_width(h->nx) > 0 && (long long)h->nx * h->ny[0] >= (h->prec == LB_PREC_BF16 ? 150000 : 400000);

@@ -14,7 +14,7 @@
 // The arithmetic is the tile kernel's, node by node: the same bits.  A node that fails the velocity guard raises
 // a flag in every CTA, which all of them read after the cluster barrier: the channel stops there.
 // us per step, launch per step in a graph -> here: FP32 4 x 64 3.2 -> 1.1, 20 x 400 4.2 -> 2.0, 4 x 1021 4.1 -> 1.6;
-// FP64 4 x 64 10.7 -> 7.1, 4 x 256 10.9 -> 7.2.
+// FP64 4 x 64 10.7 -> 6.9, 4 x 256 10.9 -> 7.0.
 // FP64: a warp's FP64 instruction takes 64 clocks on its quarter of the SM, however few lanes are active and whether
 // or not the next one depends on it, and four warps run side by side; so up to 128 threads per CTA (one warp per
 // quarter) a step costs the instructions of one node, and beyond that the tile kernel on all SMs is faster.
